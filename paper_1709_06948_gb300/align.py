@@ -366,7 +366,7 @@ def align_refine_nm(grid: Grid, xyzB, starts, step=(8.0, 8.0, 1.0, 0.1, 0.1, 0.8
     return T, mi, it
 
 
-SWEEP_KINDS = {0: "one pose per CTA", 1: "pose pairs", 2: "2-CTA cluster"}
+SWEEP_KINDS = {0: "one pose per CTA", 1: "pose pairs", 2: "2-CTA cluster", 3: "pose lattice by groups"}
 
 
 def align_eval_stats(grid: Grid):
@@ -377,7 +377,7 @@ def align_eval_stats(grid: Grid):
 
 
 def align_set_sweep(grid: Grid, kind: int):
-    """-1 automatic (default), or a kind of SWEEP_KINDS that every launch on the grid takes."""
+    """-1 automatic (default), or a kind of SWEEP_KINDS (0 to 2) that every launch on the grid takes."""
     _check(load().align_set_sweep(grid.handle, int(kind)))
 
 

@@ -67,6 +67,8 @@ struct EvalItem {
   uint32_t* hist;             // optional P x K x K full joint histograms
   unsigned long long* best;   // packed (MI, ~index) running maximum (zeroed before the launch)
   int64_t* argmax;            // one
+  const float* xyz;           // the scan itself (n_xyz x 3), for a redo without tiles (launch_redo_raw)
+  int32_t n_xyz;
   int64_t* dump;              // optional: V x 3 (n, S1, S2) of pose 0 (parity checks; S1, S2
                               // are accumulated whenever dump is set, whatever the feature)
   uint32_t* item_passes;      // optional: running max of the partitions this item's poses used
@@ -149,6 +151,8 @@ struct EvalKernels {
   cudaError_t (*launch_pack_batch)(const PackCopy* copies, int n_copies, int64_t max_out, cudaStream_t s);
   // Overlap box, phi column, MI and the running argmax of every pose.
   cudaError_t (*launch_compose)(const EvalArgs& a, cudaStream_t s);
+  // The redo kernel alone, over one item whose points are read from EvalItem::xyz.
+  cudaError_t (*launch_redo_raw)(const EvalArgs& a, int n_ctas, int vw, cudaStream_t s);
   // Each item's argmax from its packed running maximum.
   cudaError_t (*launch_argmax_finalize)(const EvalItem* items, int n_items, cudaStream_t s);
 };
@@ -188,6 +192,58 @@ struct LatticeLevel {
   uint32_t* err;            // error bits
 };
 cudaError_t launch_lattice_level(const LatticeLevel& L, cudaStream_t s);
+
+// A pose lattice evaluated group by group (lattice_eval.cu): every combination of n_rot
+// rotations and mx, my, mz values of t'_x, t'_y, t'_z, or a round of it (n_rot rotations from r0
+// on, mxr values of t'_x from ix0 on).
+constexpr int kLatticeGroup = 8;   // t'_x values per group
+constexpr int kLatticeMaxX = 64;   // ... per round
+constexpr int kLatticeMaxY = 128;
+constexpr int kLatticeMaxZ = 64;
+struct LatticeArgs {
+  GridConst gc;
+  const uint8_t* symA;
+  const float* xyz;         // n x 3
+  int64_t n;
+  const float* poses;       // P x 12
+  const int32_t* pose_of;   // [rotation][iz][iy][ix] -> pose (all rotations of the lattice)
+  int32_t P, mx, my, mz;
+  int32_t r0, n_rot, ix0, mxr;  // this round
+  int32_t first;            // clear the outputs (the first round)
+  int32_t gx, ncx;          // t'_x per group, groups per (rotation, t'_z, t'_y)
+  int32_t nsx, nsy;         // x cells of a chunk, y cells
+  int32_t n_whole, n_split; // groups evaluated as one item; parts of each of the others
+  int32_t n_items;
+  int32_t threads;          // of the evaluation kernel
+  uint32_t smem_bytes;
+  int64_t n_pad;            // n, rounded up to whole blocks of 256
+  int64_t bin_stride;       // bins of one list, padded
+  // workspace
+  uint32_t* by;             // my x (Y + 1): y cell where each voxel row starts
+  uint16_t* row_of;         // my x nsy: voxel row of a y cell
+  float* cell_u;            // ncx x nsx: a float of the x cell
+  uint16_t* bx;             // mxr x (X + 1): x cell where each voxel starts
+  // per list (rotation, t'_z, t'_x chunk):
+  uint32_t* bins;           // bin_stride: sizes, then starts of the bins (k_z, s_y)
+  uint4* raw;               // n_pad: elements in scan order, those of each warp of points together
+  uint8_t* count;           // n_pad / 32: elements of each warp
+  uint4* elems;             // n_pad: elements in bin order
+  uint32_t* next_item;
+  uint32_t* redo_mark;      // P
+  // outputs, as the table kernels'
+  uint32_t* out_c;          // P x K x K, and up to 3 words of padding
+  int32_t* out_box;         // P x 6
+  uint32_t* redo_list;
+  uint32_t* redo_count;
+  unsigned long long* best;
+};
+// Sizes of a round of at most mx values of t'_x on a's grid and lattice (gc, my, mz set): mxr, gx,
+// ncx, nsx, nsy, n_pad, bin_stride, threads, smem_bytes.  false: the lattice does not fit the kernels.
+bool lattice_layout(LatticeArgs& a, int mx, size_t smem_optin);
+cudaError_t lattice_setup();  // once per device, before any launch
+// Tables, points in bin order and the evaluation of one round: partial histograms and boxes of its
+// poses; poses with a voxel past nlim3c on the redo list.
+cudaError_t launch_lattice_eval(const LatticeArgs& a, int n_sm, cudaStream_t s);
 
 cudaError_t launch_ref_accumulate(const GridConst& gc, const float* xyz, int64_t n, const float* pose12,
                                   uint32_t* cnt, unsigned long long* s1, unsigned long long* s2,

@@ -411,6 +411,166 @@ bool use_cluster(const align_grid* g) {
 align_status enqueue_eval_core(align_grid* g, int32_t n_tiles, const float* d_poses, int64_t P, bool rotate,
                                int n_rot, const EvalOut& out, const int32_t* d_units = nullptr,
                                int32_t n_units = 0, bool cluster = false);
+align_status enqueue_lattice(align_grid* g, LatticeArgs a, const float* d_poses, const int32_t* d_pose_of,
+                             int32_t n_rot, const EvalOut& out);
+bool reserve_lattice(align_grid* g, LatticeArgs a);
+
+}  // namespace
+
+// Lays the round's workspace out from `base` (null: sizes only) and returns its bytes.
+size_t mialign::lattice_carve(LatticeArgs& a, uint8_t* base) {
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    const size_t o = off;
+    off += (bytes + 255) / 256 * 256;
+    return base ? base + o : nullptr;
+  };
+  const size_t lists = (size_t)a.n_rot * a.mz * a.ncx, n = (size_t)std::max<int64_t>(32, a.n_pad);
+  a.by = (uint32_t*)take((size_t)a.my * (a.gc.Y + 1) * 4);
+  a.row_of = (uint16_t*)take((size_t)a.my * a.nsy * 2);
+  a.cell_u = (float*)take((size_t)a.ncx * a.nsx * 4);
+  a.bx = (uint16_t*)take((size_t)a.mxr * (a.gc.X + 1) * 2);
+  a.bins = (uint32_t*)take(lists * (size_t)a.bin_stride * 4);
+  a.raw = (uint4*)take(lists * n * 16);
+  a.count = (uint8_t*)take(lists * (n / 32));
+  a.elems = (uint4*)take(lists * n * 16);
+  a.next_item = (uint32_t*)take(4);
+  a.redo_mark = (uint32_t*)take((size_t)a.P * 4);
+  return off;
+}
+
+// Sizes of a pose lattice's evaluation by groups, or false where the table kernels take it:
+// lattices with so few groups that their parts would not fill the GPU, cells that do not fit 16 bits
+// or shared memory, sparse scans on fine grids (below), or a workspace past kLatticeBudget for one
+// rotation.
+bool mialign::plan_lattice(const GridConst& gc, int n_sm, size_t smem_optin, int64_t n, int64_t n_rot, int32_t mx,
+                           int32_t my, int32_t mz, double t_max, LatticeArgs& a) {
+  // between two voxel boundaries of one t'_x lie at most two of any other (the kernel's 4-bit
+  // counts): so while a float's spacing at u is at most a sixteenth of a voxel
+  if (!((t_max + gc.X / (double)gc.inv_res) * gc.inv_res < (double)(1 << 19))) return false;
+  a.gc = gc;
+  a.n = n;
+  a.mx = mx;
+  a.my = my;
+  a.mz = mz;
+  const int64_t P = n_rot * mx * my * mz;
+  if (mx < 2 || P < 2 || P >= INT32_MAX) return false;
+  a.P = (int32_t)P;
+  if (!lattice_layout(a, mx, smem_optin)) return false;
+  // The masks of a group's rows (at least one point in each) cost about as much per word as a point
+  // does in the table kernels: measured 8.5k points on a 265 x 219 x 29 grid, 4.2 words per pose and
+  // point, 0.63 against 0.61 ms, and 41k points on 345 x 380 x 41, 4.2, 0.75 against 0.56 ms; 0.86
+  // (120k points, 320 x 320 x 32) 1.75 against 2.59 ms, 0.78 (259k, 400 x 400 x 40) 36 against 52 ms.
+  const int64_t words = std::min<int64_t>((int64_t)gc.Z * gc.Y, n / 2) * (a.nsx / 32 + 1);
+  if (words > 2 * a.gx * n) return false;
+  const int64_t chunks = ((int64_t)mx + a.gx - 1) / a.gx;
+  if (2 * n_rot * mz * my * chunks < n_sm) return false;
+  a.n_rot = 1;
+  const size_t fixed = (size_t)P * 4;
+  const size_t one = lattice_carve(a, nullptr) - fixed;
+  if (one > kLatticeBudget) return false;
+  a.n_rot = (int32_t)std::min<int64_t>({n_rot, (int64_t)(kLatticeBudget / one), 65535});
+  return true;
+}
+
+bool mialign::plan_search(const align_grid* g, int64_t n, const int32_t m[6], const double c[6], const double r[6],
+                          LatticeArgs& a) {
+  for (int i = 0; i < 6; ++i)  // finite translations at every level (the ranges only halve)
+    if (!(std::fabs(c[i]) < 1e30 && std::fabs(r[i]) < 1e30)) return false;
+  const double t_max = std::fabs(c[0]) + 2.0 * std::fabs(r[0]) + std::fabs((double)g->origin[0]);
+  return plan_lattice(g->gc, g->n_sm, g->smem_optin, n, (int64_t)m[3] * m[4] * m[5], m[0], m[1], m[2], t_max, a);
+}
+
+namespace {
+
+// The structure of a host pose batch: its distinct rotations (bitwise), each pose's rotation, and
+// whether it is a lattice: every combination of the n_rot rotations and mx, my, mz values of
+// t'_x, t'_y, t'_z (bitwise distinct), each once; then pose_of[((r mz + iz) my + iy) mx + ix].
+struct PoseSet {
+  int32_t n_rot = -1;  // -1: more than a quarter of the poses
+  std::vector<float> rots;
+  std::vector<int32_t> src;
+  bool lattice = false;
+  int32_t mx = 0, my = 0, mz = 0;
+  double t_max = 0.0;  // largest |t'_x| of a lattice
+  std::vector<int32_t> pose_of;
+};
+
+// Index of each new value of an axis among the distinct ones, in order of first appearance.  In a
+// lattice a value repeats the last one or follows it (cyclically), so hashing is rare.
+struct AxisValues {
+  std::vector<uint32_t> v;
+  std::unordered_map<uint32_t, int32_t> at;
+  int32_t last = 0;
+  int32_t index(uint32_t x) {
+    if (!v.empty()) {
+      if (v[(size_t)last] == x) return last;
+      const int32_t next = last + 1 < (int32_t)v.size() ? last + 1 : 0;
+      if (v[(size_t)next] == x) return last = next;
+    }
+    auto it = at.emplace(x, (int32_t)v.size());
+    if (it.second) v.push_back(x);
+    return last = it.first->second;
+  }
+};
+
+PoseSet pose_set(const float* poses12, int64_t P) {
+  PoseSet S;
+  AxisValues ax[3];
+  std::unordered_map<RotKey, int32_t, RotHash> seen;
+  std::vector<std::array<int32_t, 3>> c;
+  S.src.resize((size_t)P);
+  const int64_t max_rot = std::max<int64_t>(1, P / 4);
+  bool lattice = P >= 2;
+  if (lattice) c.resize((size_t)P);
+  int32_t last = 0, n_rot = 0;
+  for (int64_t p = 0; p < P; ++p) {
+    const float* q = poses12 + 12 * p;
+    // in a lattice a rotation repeats the last one or follows it (cyclically)
+    const int32_t next = last + 1 < n_rot ? last + 1 : 0;
+    if (n_rot > 0 && std::memcmp(&S.rots[(size_t)last * 9], q, 36) == 0) {
+    } else if (n_rot > 0 && std::memcmp(&S.rots[(size_t)next * 9], q, 36) == 0) {
+      last = next;
+    } else {
+      RotKey k;
+      std::memcpy(k.w, q, sizeof(k.w));
+      auto it = seen.emplace(k, n_rot);
+      if (it.second) {
+        if (n_rot >= max_rot) return PoseSet{};
+        S.rots.insert(S.rots.end(), q, q + 9);
+        ++n_rot;
+      }
+      last = it.first->second;
+    }
+    S.src[(size_t)p] = last;
+    if (!lattice) continue;
+    for (int a = 0; a < 3; ++a) {
+      uint32_t b;
+      std::memcpy(&b, q + 9 + a, 4);
+      c[(size_t)p][a] = ax[a].index(b);
+    }
+    lattice = ax[1].v.size() <= (size_t)kLatticeMaxY && ax[2].v.size() <= (size_t)kLatticeMaxZ;
+  }
+  S.n_rot = n_rot;
+  S.mx = (int32_t)ax[0].v.size();
+  S.my = (int32_t)ax[1].v.size();
+  S.mz = (int32_t)ax[2].v.size();
+  if (!lattice || (int64_t)n_rot * S.mz * S.my * S.mx != P) return S;
+  S.pose_of.assign((size_t)P, -1);
+  for (int64_t p = 0; p < P; ++p) {
+    const auto& i = c[(size_t)p];
+    int32_t& at = S.pose_of[(((size_t)S.src[(size_t)p] * S.mz + i[2]) * S.my + i[1]) * S.mx + i[0]];
+    if (at >= 0) return S;
+    at = (int32_t)p;
+  }
+  for (uint32_t b : ax[0].v) {
+    float t;
+    std::memcpy(&t, &b, 4);
+    S.t_max = std::max(S.t_max, (double)std::fabs(t));
+  }
+  S.lattice = true;
+  return S;
+}
 
 // Enqueue pack + eval + redo + compose + argmax for poses already on the device.
 // h_poses (may be NULL): the same poses on the host, used to find shared rotations (and
@@ -420,12 +580,32 @@ align_status enqueue_eval(align_grid* g, int32_t n_tiles, const float* d_poses, 
   bool rotate = true;
   int n_rot = 0;
   if (h_poses != nullptr) {
-    std::vector<float> rots;
-    std::vector<int32_t> idx;
-    const int groups = group_rotations(h_poses, P, rots, idx, max_rotation_copies(P, n_tiles));
+    const PoseSet S = pose_set(h_poses, P);
+    LatticeArgs a{};
+    if (S.lattice && out.hist == nullptr && out.dump == nullptr && g->sweep_mode < 0 && g->lattice_on &&
+        plan_lattice(g->gc, g->n_sm, g->smem_optin, g->n_points, S.n_rot, S.mx, S.my, S.mz, S.t_max, a) &&
+        reserve_lattice(g, a)) {
+      CU(g->units.ensure((size_t)P * 4), "allocate lattice order");
+      // a pageable source: staged before the call returns
+      CU(cudaMemcpyAsync(g->units.p, S.pose_of.data(), (size_t)P * 4, cudaMemcpyHostToDevice, g->stream),
+         "copy lattice order");
+      return enqueue_lattice(g, a, d_poses, g->units.as<int32_t>(), S.n_rot, out);
+    }
+    const std::vector<float>& rots = S.rots;
+    const std::vector<int32_t>& idx = S.src;
+    const int groups = S.n_rot <= max_rotation_copies(P, n_tiles) ? S.n_rot : -1;
     if (groups > 0 && out.dump == nullptr && P >= 2 && use_pairs(g)) {
       std::vector<int32_t> units;
-      const int n_units = pair_units_impl(h_poses, idx.data(), P, units);
+      if (S.lattice) {  // t'_x values 2i and 2i + 1 of the same rotation, t'_y and t'_z
+        for (int64_t at = 0; at < P; at += S.mx)
+          for (int32_t ix = 0; ix < S.mx; ix += 2) {
+            units.push_back(S.pose_of[(size_t)(at + ix)]);
+            units.push_back(ix + 1 < S.mx ? S.pose_of[(size_t)(at + ix + 1)] : -1);
+          }
+      } else {
+        pair_units_impl(h_poses, idx.data(), P, units);
+      }
+      const int n_units = (int)(units.size() / 2);
       if (n_units < P) {  // at least one pair
         CU(g->rots.ensure(rots.size() * 4), "allocate rotations");
         CU(cudaMemcpyAsync(g->rots.p, rots.data(), rots.size() * 4, cudaMemcpyHostToDevice, g->stream),
@@ -477,6 +657,7 @@ align_status enqueue_eval_core(align_grid* g, int32_t n_tiles, const float* d_po
   g->table_slots = eval_shape(0).table_slots_for(K, vw, g->smem_optin, pairs ? 2 : 1);
   g->last_pairs = pairs;
   g->last_cluster = cluster;
+  g->last_lattice = false;
   const size_t wide_bytes = (size_t)n_ctas * 2 * g->table_slots * sizeof(unsigned long long);
   if (g->wide.cap < wide_bytes || g->wide.p == nullptr) {
     CU(g->wide.ensure(wide_bytes), "allocate wide sums");
@@ -582,6 +763,129 @@ align_status enqueue_eval_core(align_grid* g, int32_t n_tiles, const float* d_po
   return ALIGN_OK;
 }
 
+// The groups' workspace; without the memory for it the table kernels take the poses.
+bool reserve_lattice(align_grid* g, LatticeArgs a) {
+  if (g->lattice_ws.ensure(lattice_carve(a, nullptr)) == cudaSuccess) return true;
+  (void)cudaGetLastError();
+  return false;
+}
+
+// One evaluation of a pose lattice by groups (lattice_eval.cu): `a` as plan_lattice left it, the
+// poses and the lattice's order on the device.
+align_status enqueue_lattice(align_grid* g, LatticeArgs a, const float* d_poses, const int32_t* d_pose_of,
+                             int32_t n_rot, const EvalOut& out) {
+  const size_t KK = (size_t)g->gc.K * g->gc.K;
+  const int64_t P = a.P;
+  CU(lattice_setup(), "set up lattice kernels");
+  CU(g->out_c.ensure((size_t)P * KK * sizeof(uint32_t) + 16), "allocate histograms");
+  CU(g->out_box.ensure((size_t)P * 6 * sizeof(int32_t)), "allocate boxes");
+  CU(g->best.ensure(sizeof(unsigned long long)), "allocate argmax");
+  CU(g->redo_list.ensure((size_t)P * 4), "allocate redo list");
+  CU(g->redo_count.ensure(16), "allocate redo count");
+  align_status st = ensure_status_words(g);
+  if (st != ALIGN_OK) return st;
+  lattice_carve(a, g->lattice_ws.as<uint8_t>());
+  a.symA = g->symA.as<uint8_t>();
+  a.xyz = g->xyz.as<float>();
+  a.poses = d_poses;
+  a.pose_of = d_pose_of;
+  a.out_c = g->out_c.as<uint32_t>();
+  a.out_box = g->out_box.as<int32_t>();
+  a.redo_list = g->redo_list.as<uint32_t>();
+  a.redo_count = g->redo_count.as<uint32_t>();
+  a.best = g->best.as<unsigned long long>();
+
+  // poses with a voxel past the 32-bit sums: the redo kernel, reading the scan itself
+  const EvalKernels& ek = eval_shape(0);
+  const int vw = g->gc.feature != ALIGN_FEAT_COUNT ? 2 : 1;
+  const int redo_ctas = (int)std::min<int64_t>(P, g->n_sm);
+  EvalItem item{};
+  item.gc = g->gc;
+  item.symA = a.symA;
+  item.sat = g->sat.as<int32_t>();
+  item.xyz = a.xyz;
+  item.n_xyz = (int32_t)a.n;
+  item.poses = d_poses;
+  item.P = (int32_t)P;
+  item.passes0 = 1;
+  item.out_c = a.out_c;
+  item.out_box = a.out_box;
+  item.mi = out.mi;
+  item.hist = out.hist;
+  item.best = a.best;
+  item.argmax = out.argmax;
+  CU(g->items.ensure(sizeof(EvalItem)), "allocate item table");
+  CU(cudaMemcpyAsync(g->items.p, &item, sizeof(EvalItem), cudaMemcpyHostToDevice, g->stream), "copy item table");
+  EvalArgs e{};
+  e.one = item;
+  e.items = g->items.as<EvalItem>();
+  e.n_items = 1;
+  e.P = (int32_t)P;
+  e.K = g->gc.K;
+  e.table_slots = ek.table_slots_for(e.K, vw, g->smem_optin, 1);
+  e.n_buckets = e.table_slots / 4;
+  e.passes0 = 1;
+  e.err = g->err.as<uint32_t>();
+  e.max_passes = g->max_passes.as<uint32_t>();
+  e.wide_count = g->wide_count.as<uint32_t>();
+  e.redo_list = a.redo_list;
+  e.redo_count = a.redo_count;
+  const size_t wide_bytes = (size_t)redo_ctas * 2 * e.table_slots * sizeof(unsigned long long);
+  if (vw > 1 && (g->wide.cap < wide_bytes || g->wide.p == nullptr)) {
+    CU(g->wide.ensure(wide_bytes), "allocate wide sums");
+    CU(cudaMemsetAsync(g->wide.p, 0, g->wide.cap, g->stream), "clear wide sums");
+  }
+  e.wide = g->wide.as<unsigned long long>();
+
+  std::array<cudaEvent_t, 3> evs{};
+  if (g->profiling) {
+    if (g->ev_pool.empty()) {
+      for (cudaEvent_t& v : evs) CU(cudaEventCreate(&v), "create event");
+    } else {
+      evs = g->ev_pool.back();
+      g->ev_pool.pop_back();
+    }
+    CU(cudaEventRecord(evs[0], g->stream), "record event");
+  }
+  const int32_t rot_round = a.n_rot, mx_round = a.mxr;
+  a.first = 1;
+  for (int32_t r0 = 0; r0 < n_rot; r0 += rot_round)
+    for (int32_t ix0 = 0; ix0 < a.mx; ix0 += mx_round) {
+      a.r0 = r0;
+      a.n_rot = std::min(rot_round, n_rot - r0);
+      a.ix0 = ix0;
+      a.mxr = std::min(mx_round, a.mx - ix0);
+      a.ncx = (a.mxr + a.gx - 1) / a.gx;
+      const int32_t groups = a.n_rot * a.mz * a.my * a.ncx;
+      // Whole groups while every CTA gets one; the rest in parts, so that the last round of CTAs
+      // costs little, each part with at least 4,096 points of the list.
+      const int32_t slots = g->n_sm * (1024 / a.threads);
+      a.n_whole = groups / slots * slots;
+      if (a.n_whole > slots && groups - a.n_whole < slots / 2) a.n_whole -= slots;
+      const int32_t rest = groups - a.n_whole;
+      a.n_split = rest == 0 ? 1
+                            : (int32_t)std::max<int64_t>(
+                                  1, std::min<int64_t>({(3 * slots + rest - 1) / rest, a.n / 4096, 16}));
+      a.n_items = a.n_whole + rest * a.n_split;
+      CU(launch_lattice_eval(a, g->n_sm, g->stream), "launch lattice evaluation");
+      a.first = 0;
+      g->stats[4] += a.n > 0 ? 5 : 2;
+    }
+  CU(ek.launch_redo_raw(e, redo_ctas, vw, g->stream), "launch redo kernel");
+  if (g->profiling) CU(cudaEventRecord(evs[1], g->stream), "record event");
+  CU(ek.launch_compose(e, g->stream), "launch compose kernel");
+  CU(ek.launch_argmax_finalize(e.items, 1, g->stream), "launch argmax");
+  if (g->profiling) {
+    CU(cudaEventRecord(evs[2], g->stream), "record event");
+    g->ev_pending.push_back(evs);
+  }
+  g->stats[4] += 3;  // redo, compose, argmax
+  g->stats[3] = std::min(a.n_items, g->n_sm * (1024 / a.threads));
+  g->stats[5] = 3;
+  g->last_lattice = true;
+  return ALIGN_OK;
+}
+
 // Add the elapsed times of all recorded event triples to the profile totals.
 align_status drain_events(align_grid* g) {
   for (auto& evs : g->ev_pending) {
@@ -601,6 +905,7 @@ align_status drain_events(align_grid* g) {
 // Key partitions the last launch's hardest pose needed: the seed of the next launch of the
 // same kind.
 void learn_passes(align_grid* g, uint32_t used) {
+  if (g->last_lattice) return;  // no tables, no partitions (the redo kernel starts from one)
   if (used == 0 || used > (1u << 16) || (used & (used - 1)) != 0) return;
   int32_t& seed = g->last_pairs ? g->passes_seed_pair[0] : g->last_cluster ? g->passes_seed_cluster : g->passes_seed[0];
   if (used > (uint32_t)seed) seed = (int32_t)used;
@@ -625,7 +930,7 @@ align_status collect_status(align_grid* g) {
   learn_passes(g, vals[1]);
   // packed-layout poses that a voxel past nlim_pack sent to the exact path: the grid's scans
   // are dense enough for the three-word layout (a limit several times larger, fewer slots)
-  if (vals[3] > 0 && g->last_vw == 2) g->layout_min = 3;
+  if (vals[3] > 0 && g->last_vw == 2 && !g->last_lattice) g->layout_min = 3;
   g->stats[0] = vals[1];
   g->stats[1] = vals[2];
   if (vals[0] & kErrDzBound) return fail(ALIGN_E_INTERNAL, "a z offset exceeded its proven bound");
@@ -691,8 +996,29 @@ align_status search_pipelined(align_grid* g, int32_t n_tiles, const double c0[6]
   g->lat_pending = true;
   // pose pairs of every level (the lattice's index structure: t_x samples 2i and 2i+1 of the
   // same rotation, t_y and t_z), decided once for the whole search
-  const bool pairs = P >= 2 && m[0] >= 2 && use_pairs(g);
-  const bool cluster = !pairs && use_cluster(g);  // likewise decided once for the search
+  // every level is a lattice: evaluated by groups where that path takes it
+  LatticeArgs lat{};
+  const bool by_groups = g->sweep_mode < 0 && g->lattice_on &&
+                         plan_search(g, g->n_points, m, c0, r0, lat) && reserve_lattice(g, lat);
+  const int32_t* d_order = nullptr;
+  if (by_groups) {
+    if (!std::equal(m, m + 6, g->lattice_order_m) || g->lattice_order.p == nullptr) {
+      std::vector<int32_t> order((size_t)P);
+      size_t at = 0;
+      for (int32_t r = 0; r < n_rot; ++r)
+        for (int32_t iz = 0; iz < m[2]; ++iz)
+          for (int32_t iy = 0; iy < m[1]; ++iy)
+            for (int32_t ix = 0; ix < m[0]; ++ix) order[at++] = ((r * m[0] + ix) * m[1] + iy) * m[2] + iz;
+      CU(g->lattice_order.ensure(order.size() * 4), "allocate lattice order");
+      // a pageable source: staged before the call returns
+      CU(cudaMemcpyAsync(g->lattice_order.p, order.data(), order.size() * 4, cudaMemcpyHostToDevice, g->stream),
+         "copy lattice order");
+      std::copy(m, m + 6, g->lattice_order_m);
+    }
+    d_order = g->lattice_order.as<int32_t>();
+  }
+  const bool pairs = !by_groups && P >= 2 && m[0] >= 2 && use_pairs(g);
+  const bool cluster = !by_groups && !pairs && use_cluster(g);  // likewise decided once for the search
   int32_t n_units = 0;
   if (pairs) {
     if (!std::equal(m, m + 6, g->lattice_units_m) || g->lat_units.p == nullptr) {
@@ -784,9 +1110,11 @@ align_status search_pipelined(align_grid* g, int32_t n_tiles, const double c0[6]
     EvalOut o{};
     o.mi = g->mi.as<float>();
     o.argmax = g->argmax.as<int64_t>();
-    align_status st = enqueue_eval_core(g, n_tiles, g->poses.as<float>(), P, false, n_rot, o,
-                                        pairs ? g->lat_units.as<int32_t>() : nullptr, n_units,
-                                        !pairs && cluster);
+    align_status st = by_groups
+                          ? enqueue_lattice(g, lat, g->poses.as<float>(), d_order, n_rot, o)
+                          : enqueue_eval_core(g, n_tiles, g->poses.as<float>(), P, false, n_rot, o,
+                                              pairs ? g->lat_units.as<int32_t>() : nullptr, n_units,
+                                              !pairs && cluster);
     if (st != ALIGN_OK) return st;
     CU(cudaMemcpyAsync(&rec[l].am, g->argmax.p, 8, cudaMemcpyDeviceToHost, g->stream), "read argmax");
     CU(cudaMemcpyAsync(&rec[l].best, g->best.p, 8, cudaMemcpyDeviceToHost, g->stream), "read best");
@@ -866,7 +1194,7 @@ align_status align_destroy_grid(align_grid* g) {
                     &g->argmax, &g->err, &g->max_passes, &g->wide_count, &g->wide, &g->dump, &g->pts4,
                     &g->pose_src, &g->rots, &g->redo_list, &g->redo_count, &g->items, &g->ovf, &g->lat_c,
                     &g->lat_cand, &g->ref_pts, &g->ref_pose, &g->ref_cnt, &g->ref_s1, &g->ref_s2, &g->ref_box,
-                    &g->units, &g->lat_units})
+                    &g->units, &g->lat_units, &g->lattice_ws, &g->lattice_order})
     b->release();
   for (HostBuf* b : {&g->lat_cand_h, &g->lat_rec_h, &g->lat_c_h, &g->ref_box_h}) b->release();
   for (cudaEvent_t e : g->lat_ev) cudaEventDestroy(e);

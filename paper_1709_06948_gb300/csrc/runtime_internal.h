@@ -76,6 +76,13 @@ align_status check_grid_device(align_grid* g);
 int pair_units(const float* poses12, const int32_t* src, int64_t P, std::vector<int32_t>& units);
 // Whether pose pairs are the automatic choice for a grid with these learned key-partition
 // counts (pairs, single poses).
+constexpr size_t kLatticeBudget = (size_t)5 << 28;  // workspace of a round of a pose lattice (1.25 GiB)
+bool plan_lattice(const GridConst& gc, int n_sm, size_t smem_optin, int64_t n, int64_t n_rot, int32_t mx, int32_t my,
+                  int32_t mz, double t_max, LatticeArgs& a);
+// The same for the levels of a lattice search over n points (align_search_ex).
+bool plan_search(const align_grid* g, int64_t n, const int32_t m[6], const double c[6], const double r[6],
+                 LatticeArgs& a);
+size_t lattice_carve(LatticeArgs& a, uint8_t* base);
 bool pairs_fit(const align_grid* g, int32_t seed_pair, int32_t seed_single);
 // One level of the coarse-to-fine lattice: FP64 poses around centre c (ranges r, m samples
 // per axis; order rx, ry, rz, tx, ty, tz with tz fastest) and their rounded FP32 form.
@@ -119,6 +126,11 @@ struct align_grid {
   int32_t passes_seed_cluster = 1;  // the 2-CTA cluster kernel (shape 0)
   int32_t sweep_mode = -1;  // -1 automatic, else the sweep kind every launch takes (align_set_sweep)
   bool last_pairs = false;    // the last eval launch evaluated pose pairs
+  bool last_lattice = false;  // ... or a pose lattice by groups
+  int32_t lattice_on = 1;     // 0: pose lattices go through the table kernels (a server's workspace
+                              // whose request was admitted without the groups' memory)
+  mialign::DevBuf lattice_ws, lattice_order;  // groups' workspace; a device-built level's pose order
+  int32_t lattice_order_m[6] = {0, 0, 0, 0, 0, 0};
   bool last_cluster = false;  // ... or ran one pose per 2-CTA cluster
   mialign::DevBuf units;    // pose pairs of the last pair launch with host poses
   mialign::DevBuf spill;    // runs queued for the later key partitions (EvalArgs::spill)

@@ -49,6 +49,7 @@ struct Req {
   int32_t counts[6];
   int32_t levels = 0;
   size_t bytes = 0;        // device memory estimate of its workspace
+  int32_t by_groups = 0;   // its lattices are evaluated by groups (another set of buffers)
   int32_t spill_np = 0;    // key partitions its spill queues serve (0: none; counted in bytes)
   double T[6] = {0, 0, 0, 0, 0, 0};
   float best_mi = 0.0f;
@@ -64,7 +65,8 @@ struct Ref {
 struct Slot {
   align_grid* ws = nullptr;      // workspace bound to one reference at a time
   cudaStream_t stream = nullptr;
-  size_t held = 0;               // device bytes its workspace may hold (estimate)
+  size_t held[2] = {0, 0};       // device bytes its workspace may hold (estimates): the table kernels'
+                                 // buffers, and those of lattices evaluated by groups
   bool busy = false;
   Req* cur = nullptr;
 };
@@ -104,7 +106,7 @@ struct align_server {
   }
   size_t used() const {
     size_t u = ref_bytes;
-    for (const Slot& sl : slots) u += sl.held;
+    for (const Slot& sl : slots) u += sl.held[0] + sl.held[1];
     return u;
   }
 };
@@ -128,6 +130,14 @@ size_t request_bytes(int64_t nB, const int32_t m[6], int K, int T, int n_sm, int
 
 // A workspace: a grid object that owns only evaluation buffers; the reference arrays it
 // reads are bound from a resident reference grid (and never released through it).
+// The same for a request whose lattices are evaluated by groups (plan `a`); the redo kernel's 64-bit
+// sums as the table kernels have them.
+size_t groups_bytes(LatticeArgs a, const GridConst& gc, int n_sm, size_t smem_optin) {
+  const int64_t per_pose = (int64_t)gc.K * gc.K * 4 + 24 + 4 + 48 + 4 + 4 + 4;
+  const int T = eval_shape(0).table_slots_for(gc.K, 2, smem_optin, 1);
+  return lattice_carve(a, nullptr) + (size_t)(a.n * 12 + a.P * per_pose + (int64_t)n_sm * 2 * T * 8);
+}
+
 align_grid* workspace_create(int device, int n_sm, size_t smem_optin, cudaStream_t stream) {
   align_grid* g = new (std::nothrow) align_grid();
   if (!g) return nullptr;
@@ -185,8 +195,8 @@ Req* try_admit_locked(align_server* s, size_t k) {
   auto need = [&]() {
     size_t others = s->ref_bytes;
     for (size_t j = 0; j < s->slots.size(); ++j)
-      if (j != k) others += s->slots[j].held;
-    return others + std::max(me.held, r->bytes);
+      if (j != k) others += s->slots[j].held[0] + s->slots[j].held[1];
+    return others + me.held[1 - r->by_groups] + std::max(me.held[r->by_groups], r->bytes);
   };
   if (need() > s->budget) {
     if (s->n_active > 0) return nullptr;  // wait until running requests finish
@@ -194,14 +204,19 @@ Req* try_admit_locked(align_server* s, size_t k) {
     // the references, as align_submit checked)
     for (size_t j = 0; j < s->slots.size(); ++j) {
       Slot& o = s->slots[j];
-      if (j == k || o.held == 0 || o.ws == nullptr) continue;
+      if (j == k || o.ws == nullptr) continue;
       workspace_destroy(o.ws);
       o.ws = nullptr;
-      o.held = 0;
+      o.held[0] = o.held[1] = 0;
+    }
+    if (need() > s->budget && me.ws != nullptr) {  // this slot's own buffers of the other kind
+      workspace_destroy(me.ws);
+      me.ws = nullptr;
+      me.held[0] = me.held[1] = 0;
     }
   }
   s->queue.pop_front();
-  me.held = std::max(me.held, r->bytes);
+  me.held[r->by_groups] = std::max(me.held[r->by_groups], r->bytes);
   me.busy = true;
   me.cur = r;
   r->t_start = s->now();
@@ -246,6 +261,7 @@ void worker_main(align_server* s, size_t k) {
         workspace_bind(ws, ref);
         ws->spill_on = r->spill_np > 0 ? 1 : 0;  // within the request's memory estimate
         ws->spill_np_max = std::max(2, r->spill_np);
+        ws->lattice_on = r->by_groups;
       }
     }
     int32_t st = ALIGN_OK;
@@ -385,6 +401,15 @@ align_status align_submit(align_server* s, const align_request* req, uint64_t* t
   r->spill_np = g->spill_on && seed >= 2 && seed <= 8 ? std::min(8, 2 * seed) : 0;
   r->bytes = request_bytes(r->nB, r->counts, g->gc.K, g->table_slots, s->n_sm, r->spill_np);
   if (s->ref_bytes + r->bytes > s->budget) return report_error(ALIGN_E_OOM, "request can never fit the memory budget");
+  LatticeArgs lat{};
+  if (g->sweep_mode < 0 && plan_search(g, r->nB, r->counts, r->c, r->r, lat)) {
+    // its lattices by groups, where that workspace fits the budget too
+    const size_t bytes = groups_bytes(lat, g->gc, s->n_sm, g->smem_optin);
+    if (s->ref_bytes + bytes <= s->budget) {
+      r->by_groups = 1;
+      r->bytes = bytes;
+    }
+  }
   r->ticket = s->next_ticket++;
   r->t_submit = s->now();
   *ticket = r->ticket;

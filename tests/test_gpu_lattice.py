@@ -1,0 +1,130 @@
+"""Pose lattices evaluated by groups (every combination of some rotations and t'_x, t'_y, t'_z) against
+the table kernels and the oracle: the same MI bit for bit, at the edges of the groups, masks, chunks and
+rounds that the path cuts its work into."""
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+import scangen
+from tests.helpers import lib_grid, mi_tolerance, oracle_grid
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def tiny():
+    return scangen.tiny_pair()
+
+
+def _lattice(counts, half, order=(3, 4, 5, 0, 1, 2), centre=np.zeros(6)):
+    axes = [np.array([c]) if m < 2 else c + np.linspace(-h, h, m) for c, h, m in zip(centre, half, counts)]
+    g = np.meshgrid(*(axes[a] for a in order), indexing="ij")
+    etas = np.empty((g[0].size, 6))
+    for a, v in zip(order, g):
+        etas[:, a] = v.reshape(-1)
+    return etas
+
+
+def _check(spec, A, B, etas, sweep=3, sample=24, **over):
+    """MI and argmax by groups equal one pose per CTA's, and a sample the oracle's."""
+    from paper_1709_06948_gb300 import align
+    L = lib_grid(spec, **over)
+    align.align_set_reference(L, A)
+    mi, am, _ = align.align_eval_mi(L, B, eta6=etas)
+    st = align.align_eval_stats(L)
+    assert st["sweep"] == sweep, st
+    redo = align.align_eval_redo_poses(L)
+    align.align_set_sweep(L, 0)
+    mi0, am0, _ = align.align_eval_mi(L, B, eta6=etas)
+    assert np.array_equal(mi.view(np.int32), mi0.view(np.int32)) and am == am0
+    pick = np.unique(np.concatenate([[am], np.linspace(0, len(etas) - 1, sample).astype(int)]))
+    G = oracle_grid(spec, **over)
+    symA, boxA = G.reference(A)
+    mo, _, _ = G.eval_mi(symA, boxA, B, align.align_round_poses(spec.origin, etas[pick]), nthreads=oracle.host_cores())
+    assert np.max(np.abs(mi[pick].astype(np.float64) - mo)) <= mi_tolerance()
+    L.close()
+    return redo
+
+
+SMALL = (0.8, 0.7, 0.3, 0.02, 0.02, 0.05)
+
+
+@pytest.mark.parametrize("counts,half,order", [
+    ((2, 8, 2, 2, 2, 3), SMALL, (3, 4, 5, 0, 1, 2)),              # the fewest t'_x of a group
+    ((3, 3, 3, 3, 3, 3), SMALL, (0, 1, 2, 3, 4, 5)),              # rotations fastest
+    ((8, 20, 1, 2, 2, 2), (3.0, 2.0, 0.0, 0.01, 0.02, 0.03), (2, 1, 0, 3, 4, 5)),
+    ((9, 13, 2, 2, 1, 3), SMALL, (5, 2, 0, 1, 3, 4)),             # two chunks of t'_x, 5 and 4
+    ((17, 40, 2, 1, 1, 2), (9.0, 0.4, 0.1, 0.0, 0.0, 0.1), (3, 4, 5, 0, 1, 2)),
+    ((70, 5, 1, 1, 1, 5), (30.0, 0.4, 0.0, 0.0, 0.0, 0.1), (3, 4, 5, 0, 1, 2)),  # two rounds of t'_x
+    ((8, 8, 3, 1, 1, 8), (1e-4, 1e-4, 1e-3, 0.0, 0.0, 0.1), (3, 4, 5, 0, 1, 2)),  # nearly equal poses
+    ((8, 8, 1, 2, 2, 5), (60.0, 60.0, 0.0, 0.5, 0.5, 3.0), (3, 4, 5, 0, 1, 2)),  # most poses leave the grid
+])
+@pytest.mark.parametrize("feature", [0, 1, 2])
+def test_groups_equal_table_kernels(tiny, counts, half, order, feature):
+    spec = scangen.GridSpec(origin=(-20.0, -20.0, -1.0), res_m=0.5, dims=(79, 83, 15), feature=feature,
+                            count_levels=7, var_levels=8 if feature == 2 else 15)
+    _check(spec, tiny.xyzA, tiny.xyzB, _lattice(counts, half, order, tiny.T))
+
+
+@pytest.mark.parametrize("n", [0, 1, 31, 33, 255, 257, 4097])
+def test_point_counts_around_warps_and_blocks(tiny, n):
+    _check(tiny.grid, tiny.xyzA, tiny.xyzB[:n], _lattice((4, 20, 2, 1, 1, 4), SMALL))
+
+
+@pytest.mark.parametrize("dims,res", [((1, 400, 3), 0.3), ((400, 1, 40), 0.2), ((33, 35, 64), 0.25), ((700, 90, 4), 0.1)])
+def test_grid_shapes(tiny, dims, res):
+    """One voxel column, one row, tall, and wide enough for groups of four t'_x."""
+    spec = scangen.GridSpec(origin=(-dims[0] * res / 2, -dims[1] * res / 2, -1.0), res_m=res, dims=dims, feature=1,
+                            var_levels=15)
+    _check(spec, tiny.xyzA, tiny.xyzB, _lattice((8, 20, 2, 1, 1, 4), SMALL))
+
+
+def test_non_finite_points_and_wide_thresholds(tiny):
+    xyz = tiny.xyzB.copy()
+    xyz[::7, 0] = np.nan
+    xyz[1::11, 1] = np.inf
+    xyz[2::13, 2] = -np.inf
+    xyz[3::17] = 3e38
+    spec = scangen.GridSpec(origin=(-20.0, -20.0, -1.0), res_m=1.0, dims=(40, 40, 8), feature=1, var_levels=5)
+    etas = _lattice((4, 20, 2, 1, 1, 4), SMALL)
+    _check(spec, tiny.xyzA, xyz, etas, var_thresh=[10, 100, 1000, 1 << 40])  # thresholds past 32 bits
+    _check(spec, tiny.xyzA, xyz, etas, var_thresh=[0, 7, 7, 100000])
+
+
+def test_dense_voxel_goes_to_the_exact_path():
+    """70,000 points in one 0.5 m voxel: past the 32-bit sums, so its poses are redone exactly."""
+    rng = np.random.default_rng(91)
+    spec = scangen.lidar_grid(0.5)
+    dense = np.stack([rng.uniform(a, a + 0.2, 70000) for a in (1.15, 2.15, 0.15)], 1)
+    rest = np.stack([rng.uniform(-30, 30, 5000), rng.uniform(-30, 30, 5000), rng.uniform(-0.5, 5, 5000)], 1)
+    xyz = np.concatenate([dense, rest]).astype(np.float32)
+    redo = _check(spec, xyz, xyz, _lattice((2, 40, 2, 1, 1, 2), (0.05, 0.05, 0.05, 0.0, 0.0, 0.001)), sample=6)
+    assert len(redo) > 0
+
+
+def test_not_a_lattice_keeps_the_table_kernels(tiny):
+    """A pose missing, repeated or moved: not every combination, so the poses go to the tables."""
+    etas = _lattice((4, 20, 2, 1, 1, 4), SMALL)
+    moved = etas.copy()
+    moved[17, 1] += 0.25
+    for e in (etas[:-1], np.concatenate([etas[1:], etas[:1], etas[:1]]), moved):
+        _check(tiny.grid, tiny.xyzA, tiny.xyzB, e, sweep=1)
+
+
+def test_search_levels_by_groups_equal_table_kernels():
+    """The six-level search of a LiDAR pair: the same poses and MI with either kind of kernel."""
+    from paper_1709_06948_gb300 import align
+    pair = scangen.lidar_pair(seed=scangen.SEED_BASE + 95, n_beams=32)
+    half = np.array([2.0, 2.0, 0.25, math.radians(1.0), math.radians(1.0), math.radians(5.0)])
+    got = []
+    for kind in (-1, 0):
+        L = lib_grid(pair.grid)
+        align.align_set_reference(L, pair.xyzA)
+        align.align_set_sweep(L, kind)
+        T, mi, lb = align.align_search(L, pair.xyzB, np.zeros(6), half, levels=6, counts=(8, 8, 2, 2, 2, 8))
+        assert align.align_eval_stats(L)["sweep"] == (3 if kind < 0 else 0)
+        got.append((T.tolist(), mi, lb.tolist()))
+        L.close()
+    assert got[0] == got[1]
