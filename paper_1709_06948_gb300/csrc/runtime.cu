@@ -1194,7 +1194,7 @@ align_status align_destroy_grid(align_grid* g) {
                     &g->argmax, &g->err, &g->max_passes, &g->wide_count, &g->wide, &g->dump, &g->pts4,
                     &g->pose_src, &g->rots, &g->redo_list, &g->redo_count, &g->items, &g->ovf, &g->lat_c,
                     &g->lat_cand, &g->ref_pts, &g->ref_pose, &g->ref_cnt, &g->ref_s1, &g->ref_s2, &g->ref_box,
-                    &g->units, &g->lat_units, &g->lattice_ws, &g->lattice_order})
+                    &g->units, &g->lat_units, &g->spill, &g->lattice_ws, &g->lattice_order})
     b->release();
   for (HostBuf* b : {&g->lat_cand_h, &g->lat_rec_h, &g->lat_c_h, &g->ref_box_h}) b->release();
   for (cudaEvent_t e : g->lat_ev) cudaEventDestroy(e);
