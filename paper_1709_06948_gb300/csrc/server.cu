@@ -403,8 +403,9 @@ align_status align_submit(align_server* s, const align_request* req, uint64_t* t
   if (s->ref_bytes + r->bytes > s->budget) return report_error(ALIGN_E_OOM, "request can never fit the memory budget");
   LatticeArgs lat{};
   if (g->sweep_mode < 0 && plan_search(g, r->nB, r->counts, r->c, r->r, lat)) {
-    // its lattices by groups, where that workspace fits the budget too
-    const size_t bytes = groups_bytes(lat, g->gc, s->n_sm, g->smem_optin);
+    // its lattices by groups, where that workspace fits the budget too; never counted below the
+    // table kernels', so that a budget that held for a request holds whichever way it runs
+    const size_t bytes = std::max(r->bytes, groups_bytes(lat, g->gc, s->n_sm, g->smem_optin));
     if (s->ref_bytes + bytes <= s->budget) {
       r->by_groups = 1;
       r->bytes = bytes;
