@@ -208,6 +208,7 @@ struct LatticeArgs {
   const float* poses;       // P x 12
   const int32_t* pose_of;   // [rotation][iz][iy][ix] -> pose (all rotations of the lattice)
   int32_t P, mx, my, mz;
+  int32_t pose_base;        // index of pose 0 on the redo list
   int32_t r0, n_rot, ix0, mxr;  // this round
   int32_t first;            // clear the outputs (the first round)
   int32_t gx, ncx;          // t'_x per group, groups per (rotation, t'_z, t'_y)
@@ -241,9 +242,10 @@ struct LatticeArgs {
 // ncx, nsx, nsy, n_pad, bin_stride, threads, smem_bytes.  false: the lattice does not fit the kernels.
 bool lattice_layout(LatticeArgs& a, int mx, size_t smem_optin);
 cudaError_t lattice_setup();  // once per device, before any launch
-// Tables, points in bin order and the evaluation of one round: partial histograms and boxes of its
-// poses; poses with a voxel past nlim3c on the redo list.
-cudaError_t launch_lattice_eval(const LatticeArgs& a, int n_sm, cudaStream_t s);
+// The whole lattice (n_rot rotations), in rounds of a.n_rot rotations and a.mxr values of t'_x: partial
+// histograms and boxes of its poses; poses with a voxel past nlim3c on the redo list.  Adds the
+// kernels launched to *launches.
+cudaError_t launch_lattice(LatticeArgs a, int32_t n_rot, int n_sm, cudaStream_t s, int32_t* launches);
 
 cudaError_t launch_ref_accumulate(const GridConst& gc, const float* xyz, int64_t n, const float* pose12,
                                   uint32_t* cnt, unsigned long long* s1, unsigned long long* s2,

@@ -45,8 +45,10 @@ struct PairPlan {
   int n_copies = 1;          // tile copies: rotations (pre-rotated) or 1 (raw)
   bool prerot = false;
   std::vector<float> hposes;  // host fp32 poses (when given on the host)
-  std::vector<int32_t> idx;   // pose -> rotation copy
-  std::vector<float> rots;    // distinct rotations
+  PoseSet set;                // their structure (rotations, lattice)
+  bool by_groups = false;     // a lattice evaluated by groups (no tiles, no table)
+  LatticeArgs lat{};
+  int64_t order_off = 0;      // its poses' order (in order)
   std::vector<int32_t> units; // pose pairs (pair kernel), two local pose indices per unit
   int32_t n_units = 0;        // 0: one pose per CTA step (eval_kernel)
   int64_t unit_off = 0;       // units before this pair's (in units)
@@ -62,7 +64,7 @@ struct PairPlan {
 // Workspace sizes of one launch; a change of any of them re-allocates and drops the graph.
 struct Sizes {
   size_t xyz = 0, poses = 0, pts = 0, pose_src = 0, copies = 0, items = 0, starts = 0, outc = 0, box = 0,
-         best = 0, mi = 0, argmax = 0, redo = 0, wide = 0, ipasses = 0, ovf = 0, units = 0, spill = 0;
+         best = 0, mi = 0, argmax = 0, redo = 0, wide = 0, ipasses = 0, ovf = 0, units = 0, spill = 0, order = 0, lattice = 0;
 };
 
 std::string env_cache_path() {
@@ -124,7 +126,7 @@ struct align_batch {
   std::string device_name;
   int shape_fixed = -1;
   DevBuf xyz, poses, pts, pose_src, copies, items, starts, outc, box, best, mi, argmax, redo_list, redo_count, wide,
-      status, ipasses, ovf, units, spill;
+      status, ipasses, ovf, units, spill, order, lattice;
   // page-locked staging of the poses and their tile copies (asynchronous copies; a call's
   // copies are done when it returns, since every call synchronises its stream)
   mialign::HostBuf h_poses, h_src;
@@ -137,6 +139,7 @@ struct align_batch {
   Sizes cap;
   // graph of the last launch sequence
   cudaGraphExec_t exec = nullptr;
+  int32_t graph_launches = 0;           // kernels of its pairs
   std::vector<int64_t> sig;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   int64_t stats[9] = {0, 0, 0, 0, 0, 0, 0, 0, 1};
@@ -168,6 +171,8 @@ struct Launch {
   // one single-pair eval + redo launch per pair: its arguments (the pair in the parameter
   // bank, its poses p_begin..P-1 of the batch) and its table layout
   std::vector<EvalArgs> evals;
+  std::vector<LatticeArgs> lats;   // its lattice by groups instead (n_items 0: not)
+  std::vector<int32_t> lat_rots;   // ... and its rotations
   std::vector<int> vws;
   int n_ctas = 0;
   bool rotate = false;
@@ -177,7 +182,8 @@ struct Launch {
 };
 
 // The launch sequence that a graph captures: clear, pack, eval + redo, compose, argmax.
-align_status enqueue_launch(align_batch* b, const Launch& L) {
+// Adds the pairs' kernels to *launches.
+align_status enqueue_launch(align_batch* b, const Launch& L, int32_t* launches) {
   cudaStream_t s = b->stream;
   BCU(cudaMemsetAsync(b->best.p, 0, (size_t)L.n_items * 8, s), "clear argmax keys");
   BCU(cudaMemsetAsync(b->ipasses.p, 0, (size_t)L.n_items * 4, s), "clear partition counts");
@@ -186,7 +192,14 @@ align_status enqueue_launch(align_batch* b, const Launch& L) {
   for (size_t k = 0; k < L.evals.size(); ++k) {
     // each pair's redo kernel finishes only that pair's poses
     if (k > 0) BCU(cudaMemsetAsync(b->redo_count.p, 0, 4, s), "clear redo count");
-    BCU(L.ek->launch_eval(L.evals[k], L.n_ctas, L.vws[k], L.rotate, s), "launch eval kernel");
+    if (L.lat_rots[k] > 0) {
+      BCU(launch_lattice(L.lats[k], L.lat_rots[k], b->n_sm, s, launches), "launch lattice evaluation");
+      BCU(eval_shape(0).launch_redo_raw(L.evals[k], b->n_sm, L.vws[k], s), "launch redo kernel");
+      *launches += 1;
+    } else {
+      BCU(L.ek->launch_eval(L.evals[k], L.n_ctas, L.vws[k], L.rotate, s), "launch eval kernel");
+      *launches += 2;
+    }
   }
   BCU(L.ek->launch_compose(L.a, s), "launch compose kernel");
   BCU(L.ek->launch_argmax_finalize(L.a.items, L.n_items, s), "launch argmax");
@@ -195,12 +208,14 @@ align_status enqueue_launch(align_batch* b, const Launch& L) {
 
 align_status run_launch(align_batch* b, const Launch& L, bool use_graph, const std::vector<int64_t>& sig) {
   BCU(cudaEventRecord(b->ev0, b->stream), "record event");
+  int32_t launches = 0;
   if (use_graph) {
     if (!b->exec || b->sig != sig) {
       drop_graph(b);
       cudaGraph_t graph = nullptr;
       BCU(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
-      align_status st = enqueue_launch(b, L);
+      b->graph_launches = 0;
+      align_status st = enqueue_launch(b, L, &b->graph_launches);
       cudaError_t e = cudaStreamEndCapture(b->stream, &graph);
       if (st != ALIGN_OK) {
         if (graph) cudaGraphDestroy(graph);
@@ -216,13 +231,14 @@ align_status run_launch(align_batch* b, const Launch& L, bool use_graph, const s
       b->stats[2] += 1;
     }
     BCU(cudaGraphLaunch(b->exec, b->stream), "launch graph");
+    launches = b->graph_launches;
   } else {
-    align_status st = enqueue_launch(b, L);
+    align_status st = enqueue_launch(b, L, &launches);
     if (st != ALIGN_OK) return st;
   }
   BCU(cudaEventRecord(b->ev1, b->stream), "record event");
   b->stats[0] += 1;
-  b->stats[5] += 3 + 2 * (int64_t)L.evals.size();  // pack, eval + redo per pair, compose, argmax
+  b->stats[5] += 3 + launches;  // pack, the pairs' kernels, compose, argmax
   return ALIGN_OK;
 }
 
@@ -311,7 +327,7 @@ align_status align_batch_destroy(align_batch* b) {
   drop_graph(b);
   for (DevBuf* d : {&b->xyz, &b->poses, &b->pts, &b->pose_src, &b->copies, &b->items, &b->starts, &b->outc, &b->box,
                     &b->best, &b->mi, &b->argmax, &b->redo_list, &b->redo_count, &b->wide, &b->status, &b->ipasses, &b->ovf,
-                    &b->units, &b->spill})
+                    &b->units, &b->spill, &b->order, &b->lattice})
     d->release();
   b->h_poses.release();
   b->h_src.release();
@@ -373,17 +389,16 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
   for (PairPlan& pp : plans) {
     pp.n_tiles = (int32_t)std::max<int64_t>(ek.min_tiles(), (pp.nB + tile - 1) / tile);
     pp.n_pad = (int64_t)pp.n_tiles * tile;
-    if (rotate) continue;
-    const int max_groups = (int)std::max<int64_t>(1, pp.P / 4);
-    const int groups = group_pose_rotations(pp.hposes.data(), pp.P, pp.rots, pp.idx, max_groups);
+    if (rotate || pp.by_groups) continue;
+    const int groups = pp.set.n_rot;
     prerot_bytes += (size_t)std::max(groups, 1) * (size_t)pp.n_pad * 16;
     if (groups <= 0 || prerot_bytes > kPrerotBudget) rotate = true;
   }
-  int64_t units_n = 0;
+  int64_t units_n = 0, order_n = 0;
   int64_t spill_words = 0;  // largest (queues x runs per queue) of a pair with spill queues
   for (PairPlan& pp : plans) {
-    pp.prerot = !rotate;
-    pp.n_copies = rotate ? 1 : (int)(pp.rots.size() / 9);
+    pp.prerot = !rotate && !pp.by_groups;
+    pp.n_copies = pp.by_groups ? 0 : rotate ? 1 : pp.set.n_rot;
     // pose pairs: a pair's poses with the same rotation, t_y and t_z (pre-rotated tiles only);
     // a pair whose poses form no pair keeps the single-pose kernel
     pp.n_units = 0;
@@ -396,7 +411,7 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
                           : pairs_fit(pp.g, __atomic_load_n(&pp.g->passes_seed_pair[shape], __ATOMIC_RELAXED),
                                       __atomic_load_n(&pp.g->passes_seed[shape], __ATOMIC_RELAXED));
     if (pose_pairs && fits && pp.prerot && pp.P >= 2) {
-      const int nu = pair_units(pp.hposes.data(), pp.idx.data(), pp.P, pp.units);
+      const int nu = pair_units(pp.hposes.data(), pp.set, pp.P, pp.units);
       if (nu < pp.P) pp.n_units = nu;
       else pp.units.clear();
     }
@@ -406,7 +421,7 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
                                  __ATOMIC_RELAXED);
     pp.spill_np = 0;
     pp.spill_cap = 0;
-    if (pp.g->spill_on && pp.passes0 >= 2 && pp.passes0 <= 8) {
+    if (pp.g->spill_on && !pp.by_groups && pp.passes0 >= 2 && pp.passes0 <= 8) {
       pp.spill_np = std::min(8, 2 * pp.passes0);
       const int64_t runs = pp.g->spill_runs > 0 ? pp.g->spill_runs : pp.n_units > 0 ? pp.n_pad : pp.n_pad / 2;
       pp.spill_cap = (runs + 31) / 32 * 32;
@@ -418,10 +433,12 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
     pp.pose_off = poses_n;
     pp.pts_off = pts_n;
     pp.outc_off = outc_n;
+    pp.order_off = order_n;
+    if (pp.by_groups) order_n += pp.P;
     xyz_f += pp.nB * 3;
     poses_n += pp.P;
     pts_n += (int64_t)pp.n_copies * pp.n_pad;
-    outc_n += pp.P * (int64_t)pp.g->gc.K * pp.g->gc.K;
+    outc_n += (pp.P * (int64_t)pp.g->gc.K * pp.g->gc.K + 3) / 4 * 4;  // cleared four words at a time
     n_copies += pp.n_copies;
     max_out = std::max(max_out, pp.n_pad);
   }
@@ -431,6 +448,12 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
   std::vector<int> vws, Ts;
   int T = 0;  // the largest table of the launches (sizes the 64-bit side sums)
   for (const PairPlan& pp : plans) {
+    if (pp.by_groups) {  // the redo kernel's tables
+      vws.push_back(pp.g->gc.feature != ALIGN_FEAT_COUNT ? 2 : 1);
+      Ts.push_back(eval_shape(0).table_slots_for(pp.g->gc.K, vws.back(), b->smem_optin, 1));
+      T = std::max(T, Ts.back());
+      continue;
+    }
     int vw = eval_layout(pp.g->gc, var);  // at least the layout the grid has learned to need
     if (var) vw = std::max(vw, (int)__atomic_load_n(&pp.g->layout_min, __ATOMIC_RELAXED));
     vws.push_back(vw);
@@ -460,6 +483,7 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
   GROW(ovf, ovf, (size_t)n_ctas * ek.ovf_cap() * 16, "allocate overflow lists", false);
   GROW(units, units, (size_t)std::max<int64_t>(1, units_n) * 8, "allocate pose pairs", false);
   GROW(spill, spill, (size_t)n_ctas * (size_t)std::max<int64_t>(1, spill_words) * 16, "allocate spill queues", false);
+  GROW(order, order, (size_t)std::max<int64_t>(1, order_n) * 4, "allocate lattice order", false);
 #undef GROW
   if (!b->status.p || !b->redo_count.p) {
     drop_graph(b);
@@ -500,7 +524,7 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
           "copy poses");
     }
     if (pp.prerot)
-      for (int64_t p = 0; p < pp.P; ++p) hsrc[(size_t)(pp.pose_off + p)] = pp.idx[(size_t)p];
+      for (int64_t p = 0; p < pp.P; ++p) hsrc[(size_t)(pp.pose_off + p)] = pp.set.src[(size_t)p];
     for (int c = 0; c < pp.n_copies; ++c) {
       PackCopy pc{};
       pc.xyz = b->xyz.as<float>() + pp.xyz_off;
@@ -508,7 +532,7 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
       pc.n_out = pp.n_pad;
       pc.out = b->pts.as<float4>() + pp.pts_off + (int64_t)c * pp.n_pad;
       pc.rotate = pp.prerot ? 1 : 0;
-      for (int k = 0; k < 9; ++k) pc.R[k] = pp.prerot ? pp.rots[(size_t)c * 9 + k] : 0.0f;
+      for (int k = 0; k < 9; ++k) pc.R[k] = pp.prerot ? pp.set.rots[(size_t)c * 9 + k] : 0.0f;
       hcopies.push_back(pc);
     }
     EvalItem& it = hitems[(size_t)i];
@@ -517,6 +541,8 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
     it.sat = g->sat.as<int32_t>();
     it.src = b->pts.as<float4>() + pp.pts_off;
     it.src_stride = (uint64_t)pp.n_pad;
+    it.xyz = b->xyz.as<float>() + pp.xyz_off;
+    it.n_xyz = (int32_t)pp.nB;
     it.pose_src = pp.prerot ? b->pose_src.as<int32_t>() + pp.pose_off : nullptr;
     it.poses = b->poses.as<float>() + pp.pose_off * 12;
     it.n_tiles = pp.n_tiles;
@@ -535,6 +561,10 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
                           cudaMemcpyHostToDevice, s),
           "copy pose pairs");
     it.item_passes = b->ipasses.as<uint32_t>() + i;
+    if (pp.by_groups)  // likewise
+      BCU(cudaMemcpyAsync(b->order.as<int32_t>() + pp.order_off, pp.set.pose_of.data(), (size_t)pp.P * 4,
+                          cudaMemcpyHostToDevice, s),
+          "copy lattice order");
     hstarts[(size_t)i] = (int32_t)pp.pose_off;
   }
   hstarts[(size_t)n] = (int32_t)poses_n;
@@ -597,10 +627,29 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
       ai.spill_np = plans[(size_t)i].spill_np;
     }
     L.evals.push_back(ai);
+    LatticeArgs la = plans[(size_t)i].lat;
+    if (plans[(size_t)i].by_groups) {
+      const EvalItem& it = hitems[(size_t)i];
+      lattice_carve(la, b->lattice.as<uint8_t>());
+      la.symA = it.symA;
+      la.xyz = it.xyz;
+      la.poses = it.poses;
+      la.pose_of = b->order.as<int32_t>() + plans[(size_t)i].order_off;
+      la.pose_base = it.pose_base;
+      la.out_c = it.out_c;
+      la.out_box = it.out_box;
+      la.best = it.best;
+      la.redo_list = a.redo_list;
+      la.redo_count = a.redo_count;
+    }
+    L.lats.push_back(la);
+    L.lat_rots.push_back(plans[(size_t)i].by_groups ? plans[(size_t)i].set.n_rot : 0);
   }
   b->last_grids.clear();
   b->last_pairs.clear();
   b->last_vws = vws;
+  for (size_t i = 0; i < plans.size(); ++i)
+    if (plans[i].by_groups) b->last_vws[i] = 0;  // no table layout to learn from
   for (const PairPlan& pp : plans) {
     b->last_grids.push_back(pp.g);
     b->last_pairs.push_back(pp.n_units > 0 ? 1 : 0);
@@ -614,9 +663,13 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
                               poses_n, n_copies, max_out,   maxK,      (int64_t)(uintptr_t)b->pts.p,
                               (int64_t)(uintptr_t)b->items.p, (int64_t)h};
   for (size_t i = 0; i < vws.size(); ++i)
-    sig.insert(sig.end(), {vws[i], Ts[i], plans[i].n_units, plans[i].spill_np, plans[i].spill_cap});
+    sig.insert(sig.end(), {vws[i], Ts[i], plans[i].n_units, plans[i].spill_np, plans[i].spill_cap,
+                           plans[i].by_groups ? plans[i].set.n_rot : 0, plans[i].set.mx, plans[i].set.my,
+                           plans[i].set.mz, plans[i].nB});
   sig.push_back((int64_t)(uintptr_t)b->units.p);
   sig.push_back((int64_t)(uintptr_t)b->spill.p);
+  sig.push_back((int64_t)(uintptr_t)b->order.p);
+  sig.push_back((int64_t)(uintptr_t)b->lattice.p);
   st = run_launch(b, L, (flags & ALIGN_BATCH_GRAPH) != 0, sig);
   if (st != ALIGN_OK) return st;
   b->stats[3] = shape;
@@ -679,11 +732,30 @@ extern "C" align_status align_eval_batch(align_batch* b, const align_pair* pairs
     BCU(cudaStreamSynchronize(b->stream), "synchronize");
     return ALIGN_OK;
   }
+  // Lattices by groups, unless the caller fixed the table kernels' shape or poses per CTA: those with
+  // a group per SM (smaller ones share the table kernels' launches, two per pair).
+  for (PairPlan& pp : plans) {
+    if (pp.hposes.empty()) continue;
+    pp.set = pose_set(pp.hposes.data(), pp.P);
+    pp.by_groups = b->shape_fixed < 0 && b->pairs_fixed < 0 && pp.set.lattice && pp.g->sweep_mode < 0 &&
+                   plan_lattice(pp.g->gc, b->n_sm, b->smem_optin, pp.nB, pp.set.n_rot, pp.set.mx, pp.set.my, pp.set.mz,
+                                pp.set.t_max, b->n_sm, pp.lat);
+  }
+  size_t lattice_bytes = 0;
+  for (PairPlan& pp : plans)
+    if (pp.by_groups) lattice_bytes = std::max(lattice_bytes, lattice_carve(pp.lat, nullptr));
+  if (lattice_bytes > 0) {
+    BCU(lattice_setup(), "set up lattice kernels");  // before any capture
+    // without the memory for it the table kernels take the poses
+    if (grow(b, b->lattice, b->cap.lattice, lattice_bytes, "allocate lattice workspace") != ALIGN_OK)
+      for (PairPlan& pp : plans) pp.by_groups = false;
+  }
+  const bool tables = std::any_of(plans.begin(), plans.end(), [](const PairPlan& pp) { return !pp.by_groups; });
   // kernel shape and poses per CTA: fixed, tuned (cached per batch class) or the default
   // (shape 0, pose pairs)
   int shape = b->shape_fixed >= 0 ? b->shape_fixed : 0;
   bool pose_pairs = b->pairs_fixed != 1;
-  if ((b->shape_fixed < 0 || b->pairs_fixed < 0) && (flags & ALIGN_BATCH_TUNE)) {
+  if (tables && (b->shape_fixed < 0 || b->pairs_fixed < 0) && (flags & ALIGN_BATCH_TUNE)) {
     int64_t pts_tot = 0, poses_tot = 0;
     int maxK = 0;
     bool dev_poses = false;

@@ -839,7 +839,7 @@ __global__ void __launch_bounds__(kNT, 1024 / kNT) lattice_eval_kernel(const __g
       if (i >= 3 && v != INT_MIN) atomicMax(ob, v);
     }
     if (tid < G && C.wide[tid] && atomicExch(a.redo_mark + C.pose[tid], 1u) == 0u)
-      a.redo_list[atomicAdd(a.redo_count, 1u)] = (uint32_t)C.pose[tid];
+      a.redo_list[atomicAdd(a.redo_count, 1u)] = (uint32_t)(a.pose_base + C.pose[tid]);
     __syncthreads();  // the histograms are read before the next item clears them
   }
 }
@@ -923,21 +923,45 @@ cudaError_t lattice_setup() {
   return cudaSuccess;
 }
 
-cudaError_t launch_lattice_eval(const LatticeArgs& a, int n_sm, cudaStream_t s) {
+cudaError_t launch_lattice(LatticeArgs a, int32_t n_rot, int n_sm, cudaStream_t s, int32_t* launches) {
   cudaError_t e;
-  setup_kernel<<<2 * n_sm, 256, 0, s>>>(a);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (a.n > 0) {
-    const dim3 grid((unsigned)((a.n + 255) / 256), (unsigned)a.n_rot);
-    points_kernel<<<grid, 256, 0, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    offsets_kernel<<<a.n_rot * a.mz * a.ncx, 1024, 0, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    scatter_kernel<<<grid, 256, 0, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  const int ctas = std::min(a.n_items, n_sm * (1024 / a.threads));
-  return a.threads == 512 ? launch_eval_nt<512>(a, ctas, s) : launch_eval_nt<1024>(a, ctas, s);
+  const int32_t rot_round = a.n_rot, mx_round = a.mxr;
+  a.first = 1;
+  for (int32_t r0 = 0; r0 < n_rot; r0 += rot_round)
+    for (int32_t ix0 = 0; ix0 < a.mx; ix0 += mx_round, a.first = 0) {
+      a.r0 = r0;
+      a.n_rot = std::min(rot_round, n_rot - r0);
+      a.ix0 = ix0;
+      a.mxr = std::min(mx_round, a.mx - ix0);
+      a.ncx = (a.mxr + a.gx - 1) / a.gx;
+      // Whole groups while every CTA gets one; the rest in parts, so that the last round of CTAs
+      // costs little, each part with at least 4,096 points of the list (512 groups on 304 CTAs: 0.88
+      // ms with two parts of every group, 0.79 ms so).
+      const int32_t groups = a.n_rot * a.mz * a.my * a.ncx, slots = n_sm * (1024 / a.threads);
+      a.n_whole = groups / slots * slots;
+      if (a.n_whole > slots && groups - a.n_whole < slots / 2) a.n_whole -= slots;
+      const int32_t rest = groups - a.n_whole;
+      a.n_split = rest == 0 ? 1
+                            : (int32_t)std::max<int64_t>(
+                                  1, std::min<int64_t>({(3 * slots + rest - 1) / rest, a.n / 4096, 16}));
+      a.n_items = a.n_whole + rest * a.n_split;
+      setup_kernel<<<2 * n_sm, 256, 0, s>>>(a);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      if (a.n > 0) {
+        const dim3 grid((unsigned)((a.n + 255) / 256), (unsigned)a.n_rot);
+        points_kernel<<<grid, 256, 0, s>>>(a);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        offsets_kernel<<<a.n_rot * a.mz * a.ncx, 1024, 0, s>>>(a);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        scatter_kernel<<<grid, 256, 0, s>>>(a);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      }
+      const int ctas = std::min(a.n_items, slots);
+      e = a.threads == 512 ? launch_eval_nt<512>(a, ctas, s) : launch_eval_nt<1024>(a, ctas, s);
+      if (e != cudaSuccess) return e;
+      *launches += a.n > 0 ? 5 : 2;
+    }
+  return cudaSuccess;
 }
 
 }  // namespace mialign

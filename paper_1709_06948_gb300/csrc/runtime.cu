@@ -285,30 +285,6 @@ struct RotHash {
   }
 };
 
-int group_rotations(const float* poses12, int64_t P, std::vector<float>& rots, std::vector<int32_t>& idx,
-                    int max_groups) {
-  std::unordered_map<RotKey, int32_t, RotHash> seen;
-  rots.clear();
-  idx.resize((size_t)P);
-  for (int64_t p = 0; p < P; ++p) {
-    // lattices list poses rotation-major: most poses share the previous pose's rotation
-    if (p > 0 && std::memcmp(poses12 + 12 * p, poses12 + 12 * (p - 1), 9 * sizeof(float)) == 0) {
-      idx[(size_t)p] = idx[(size_t)(p - 1)];
-      continue;
-    }
-    RotKey k;
-    std::memcpy(k.w, poses12 + 12 * p, sizeof(k.w));
-    auto it = seen.find(k);
-    if (it == seen.end()) {
-      if ((int)seen.size() >= max_groups) return -1;
-      it = seen.emplace(k, (int32_t)seen.size()).first;
-      rots.insert(rots.end(), poses12 + 12 * p, poses12 + 12 * p + 9);
-    }
-    idx[(size_t)p] = it->second;
-  }
-  return (int)seen.size();
-}
-
 // Error word and counters: allocated once per grid and zeroed (cudaMalloc memory is not).
 align_status ensure_status_words(align_grid* g) {
   if (g->err.p && g->max_passes.p && g->wide_count.p) return ALIGN_OK;
@@ -440,11 +416,11 @@ size_t mialign::lattice_carve(LatticeArgs& a, uint8_t* base) {
 }
 
 // Sizes of a pose lattice's evaluation by groups, or false where the table kernels take it:
-// lattices with so few groups that their parts would not fill the GPU, cells that do not fit 16 bits
+// lattices with fewer than min_groups groups (their parts would not fill the GPU), cells that do not fit 16 bits
 // or shared memory, sparse scans on fine grids (below), or a workspace past kLatticeBudget for one
 // rotation.
 bool mialign::plan_lattice(const GridConst& gc, int n_sm, size_t smem_optin, int64_t n, int64_t n_rot, int32_t mx,
-                           int32_t my, int32_t mz, double t_max, LatticeArgs& a) {
+                           int32_t my, int32_t mz, double t_max, int min_groups, LatticeArgs& a) {
   // between two voxel boundaries of one t'_x lie at most two of any other (the kernel's 4-bit
   // counts): so while a float's spacing at u is at most a sixteenth of a voxel
   if (!((t_max + gc.X / (double)gc.inv_res) * gc.inv_res < (double)(1 << 19))) return false;
@@ -464,7 +440,7 @@ bool mialign::plan_lattice(const GridConst& gc, int n_sm, size_t smem_optin, int
   const int64_t words = std::min<int64_t>((int64_t)gc.Z * gc.Y, n / 2) * (a.nsx / 32 + 1);
   if (words > 2 * a.gx * n) return false;
   const int64_t chunks = ((int64_t)mx + a.gx - 1) / a.gx;
-  if (2 * n_rot * mz * my * chunks < n_sm) return false;
+  if (n_rot * mz * my * chunks < min_groups) return false;
   a.n_rot = 1;
   const size_t fixed = (size_t)P * 4;
   const size_t one = lattice_carve(a, nullptr) - fixed;
@@ -478,23 +454,11 @@ bool mialign::plan_search(const align_grid* g, int64_t n, const int32_t m[6], co
   for (int i = 0; i < 6; ++i)  // finite translations at every level (the ranges only halve)
     if (!(std::fabs(c[i]) < 1e30 && std::fabs(r[i]) < 1e30)) return false;
   const double t_max = std::fabs(c[0]) + 2.0 * std::fabs(r[0]) + std::fabs((double)g->origin[0]);
-  return plan_lattice(g->gc, g->n_sm, g->smem_optin, n, (int64_t)m[3] * m[4] * m[5], m[0], m[1], m[2], t_max, a);
+  return plan_lattice(g->gc, g->n_sm, g->smem_optin, n, (int64_t)m[3] * m[4] * m[5], m[0], m[1], m[2], t_max,
+                      g->n_sm / 2, a);
 }
 
 namespace {
-
-// The structure of a host pose batch: its distinct rotations (bitwise), each pose's rotation, and
-// whether it is a lattice: every combination of the n_rot rotations and mx, my, mz values of
-// t'_x, t'_y, t'_z (bitwise distinct), each once; then pose_of[((r mz + iz) my + iy) mx + ix].
-struct PoseSet {
-  int32_t n_rot = -1;  // -1: more than a quarter of the poses
-  std::vector<float> rots;
-  std::vector<int32_t> src;
-  bool lattice = false;
-  int32_t mx = 0, my = 0, mz = 0;
-  double t_max = 0.0;  // largest |t'_x| of a lattice
-  std::vector<int32_t> pose_of;
-};
 
 // Index of each new value of an axis among the distinct ones, in order of first appearance.  In a
 // lattice a value repeats the last one or follows it (cyclically), so hashing is rare.
@@ -514,7 +478,8 @@ struct AxisValues {
   }
 };
 
-PoseSet pose_set(const float* poses12, int64_t P) {
+}  // namespace
+PoseSet mialign::pose_set(const float* poses12, int64_t P) {
   PoseSet S;
   AxisValues ax[3];
   std::unordered_map<RotKey, int32_t, RotHash> seen;
@@ -572,6 +537,18 @@ PoseSet pose_set(const float* poses12, int64_t P) {
   return S;
 }
 
+int mialign::pair_units(const float* poses12, const PoseSet& S, int64_t P, std::vector<int32_t>& units) {
+  if (!S.lattice) return pair_units_impl(poses12, S.src.data(), P, units);
+  units.clear();
+  for (int64_t at = 0; at < P; at += S.mx)  // t'_x values 2i and 2i + 1 of the same rotation, t'_y and t'_z
+    for (int32_t ix = 0; ix < S.mx; ix += 2) {
+      units.push_back(S.pose_of[(size_t)(at + ix)]);
+      units.push_back(ix + 1 < S.mx ? S.pose_of[(size_t)(at + ix + 1)] : -1);
+    }
+  return (int)(units.size() / 2);
+}
+namespace {
+
 // Enqueue pack + eval + redo + compose + argmax for poses already on the device.
 // h_poses (may be NULL): the same poses on the host, used to find shared rotations (and
 // pose pairs).
@@ -583,7 +560,8 @@ align_status enqueue_eval(align_grid* g, int32_t n_tiles, const float* d_poses, 
     const PoseSet S = pose_set(h_poses, P);
     LatticeArgs a{};
     if (S.lattice && out.hist == nullptr && out.dump == nullptr && g->sweep_mode < 0 && g->lattice_on &&
-        plan_lattice(g->gc, g->n_sm, g->smem_optin, g->n_points, S.n_rot, S.mx, S.my, S.mz, S.t_max, a) &&
+        plan_lattice(g->gc, g->n_sm, g->smem_optin, g->n_points, S.n_rot, S.mx, S.my, S.mz, S.t_max,
+                     g->n_sm / 2, a) &&
         reserve_lattice(g, a)) {
       CU(g->units.ensure((size_t)P * 4), "allocate lattice order");
       // a pageable source: staged before the call returns
@@ -596,16 +574,7 @@ align_status enqueue_eval(align_grid* g, int32_t n_tiles, const float* d_poses, 
     const int groups = S.n_rot <= max_rotation_copies(P, n_tiles) ? S.n_rot : -1;
     if (groups > 0 && out.dump == nullptr && P >= 2 && use_pairs(g)) {
       std::vector<int32_t> units;
-      if (S.lattice) {  // t'_x values 2i and 2i + 1 of the same rotation, t'_y and t'_z
-        for (int64_t at = 0; at < P; at += S.mx)
-          for (int32_t ix = 0; ix < S.mx; ix += 2) {
-            units.push_back(S.pose_of[(size_t)(at + ix)]);
-            units.push_back(ix + 1 < S.mx ? S.pose_of[(size_t)(at + ix + 1)] : -1);
-          }
-      } else {
-        pair_units_impl(h_poses, idx.data(), P, units);
-      }
-      const int n_units = (int)(units.size() / 2);
+      const int n_units = pair_units(h_poses, S, P, units);
       if (n_units < P) {  // at least one pair
         CU(g->rots.ensure(rots.size() * 4), "allocate rotations");
         CU(cudaMemcpyAsync(g->rots.p, rots.data(), rots.size() * 4, cudaMemcpyHostToDevice, g->stream),
@@ -847,30 +816,8 @@ align_status enqueue_lattice(align_grid* g, LatticeArgs a, const float* d_poses,
     }
     CU(cudaEventRecord(evs[0], g->stream), "record event");
   }
-  const int32_t rot_round = a.n_rot, mx_round = a.mxr;
-  a.first = 1;
-  for (int32_t r0 = 0; r0 < n_rot; r0 += rot_round)
-    for (int32_t ix0 = 0; ix0 < a.mx; ix0 += mx_round) {
-      a.r0 = r0;
-      a.n_rot = std::min(rot_round, n_rot - r0);
-      a.ix0 = ix0;
-      a.mxr = std::min(mx_round, a.mx - ix0);
-      a.ncx = (a.mxr + a.gx - 1) / a.gx;
-      const int32_t groups = a.n_rot * a.mz * a.my * a.ncx;
-      // Whole groups while every CTA gets one; the rest in parts, so that the last round of CTAs
-      // costs little, each part with at least 4,096 points of the list.
-      const int32_t slots = g->n_sm * (1024 / a.threads);
-      a.n_whole = groups / slots * slots;
-      if (a.n_whole > slots && groups - a.n_whole < slots / 2) a.n_whole -= slots;
-      const int32_t rest = groups - a.n_whole;
-      a.n_split = rest == 0 ? 1
-                            : (int32_t)std::max<int64_t>(
-                                  1, std::min<int64_t>({(3 * slots + rest - 1) / rest, a.n / 4096, 16}));
-      a.n_items = a.n_whole + rest * a.n_split;
-      CU(launch_lattice_eval(a, g->n_sm, g->stream), "launch lattice evaluation");
-      a.first = 0;
-      g->stats[4] += a.n > 0 ? 5 : 2;
-    }
+  int32_t launches = 0;
+  CU(launch_lattice(a, n_rot, g->n_sm, g->stream, &launches), "launch lattice evaluation");
   CU(ek.launch_redo_raw(e, redo_ctas, vw, g->stream), "launch redo kernel");
   if (g->profiling) CU(cudaEventRecord(evs[1], g->stream), "record event");
   CU(ek.launch_compose(e, g->stream), "launch compose kernel");
@@ -879,8 +826,8 @@ align_status enqueue_lattice(align_grid* g, LatticeArgs a, const float* d_poses,
     CU(cudaEventRecord(evs[2], g->stream), "record event");
     g->ev_pending.push_back(evs);
   }
-  g->stats[4] += 3;  // redo, compose, argmax
-  g->stats[3] = std::min(a.n_items, g->n_sm * (1024 / a.threads));
+  g->stats[4] += launches + 3;  // and redo, compose, argmax
+  g->stats[3] = g->n_sm * (1024 / a.threads);
   g->stats[5] = 3;
   g->last_lattice = true;
   return ALIGN_OK;
@@ -1741,14 +1688,7 @@ align_status report_errorf(align_status st, const char* fmt, ...) {
   va_end(ap);
   return fail(st, "%s", buf);
 }
-int group_pose_rotations(const float* poses12, int64_t P, std::vector<float>& rots, std::vector<int32_t>& idx,
-                         int max_groups) {
-  return group_rotations(poses12, P, rots, idx, max_groups);
-}
 align_status check_grid_device(align_grid* g) { return check_grid(g); }
-int pair_units(const float* poses12, const int32_t* src, int64_t P, std::vector<int32_t>& units) {
-  return pair_units_impl(poses12, src, P, units);
-}
 void lattice_poses(const float origin[3], const double c[6], const double r[6], const int32_t m[6],
                    std::vector<double>& eta, std::vector<float>& poses) {
   build_lattice(c, r, m, eta);

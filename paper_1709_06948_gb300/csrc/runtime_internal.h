@@ -65,20 +65,28 @@ struct HostBuf {
 
 // Error reporting into the thread-local message of align_last_error.
 align_status report_errorf(align_status st, const char* fmt, ...);
-// Distinct rotations (bitwise-equal 3x3 blocks) of a host pose batch and each pose's
-// group; -1 when there are more than max_groups.
-int group_pose_rotations(const float* poses12, int64_t P, std::vector<float>& rots, std::vector<int32_t>& idx,
-                         int max_groups);
+// The structure of a host pose batch: its distinct rotations (bitwise), each pose's rotation, and
+// whether it is a lattice: every combination of the n_rot rotations and mx, my, mz values of
+// t'_x, t'_y, t'_z (bitwise distinct), each once; then pose_of[((r mz + iz) my + iy) mx + ix].
+struct PoseSet {
+  int32_t n_rot = -1;  // -1: more than a quarter of the poses
+  std::vector<float> rots;
+  std::vector<int32_t> src;
+  bool lattice = false;
+  int32_t mx = 0, my = 0, mz = 0;
+  double t_max = 0.0;  // largest |t'_x| of a lattice
+  std::vector<int32_t> pose_of;
+};
+PoseSet pose_set(const float* poses12, int64_t P);
 align_status check_grid_device(align_grid* g);
-// Pose pairs of a host pose batch for the pair kernel: poses with the same tile copy
-// (src, or all one copy when NULL) and bitwise equal t'_y, t'_z, two per unit in order of
-// their first pose (local indices; the second -1 for a single pose).  Returns the units.
-int pair_units(const float* poses12, const int32_t* src, int64_t P, std::vector<int32_t>& units);
+// Pose pairs for the pair kernel: poses with the same rotation (tile copy) and bitwise equal
+// t'_y, t'_z, two per unit (local indices; the second -1 for a single pose).  Returns the units.
+int pair_units(const float* poses12, const PoseSet& set, int64_t P, std::vector<int32_t>& units);
 // Whether pose pairs are the automatic choice for a grid with these learned key-partition
 // counts (pairs, single poses).
 constexpr size_t kLatticeBudget = (size_t)5 << 28;  // workspace of a round of a pose lattice (1.25 GiB)
 bool plan_lattice(const GridConst& gc, int n_sm, size_t smem_optin, int64_t n, int64_t n_rot, int32_t mx, int32_t my,
-                  int32_t mz, double t_max, LatticeArgs& a);
+                  int32_t mz, double t_max, int min_groups, LatticeArgs& a);
 // The same for the levels of a lattice search over n points (align_search_ex).
 bool plan_search(const align_grid* g, int64_t n, const int32_t m[6], const double c[6], const double r[6],
                  LatticeArgs& a);

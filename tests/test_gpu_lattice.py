@@ -128,3 +128,30 @@ def test_search_levels_by_groups_equal_table_kernels():
         got.append((T.tolist(), mi, lb.tolist()))
         L.close()
     assert got[0] == got[1]
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_batch_mixes_groups_and_tables(tiny, graph):
+    """Lattices of several grids and features beside pose sets that are none, in one batch (twice, the
+    second with other poses): every pair's result is align_eval_mi's alone."""
+    from paper_1709_06948_gb300 import align
+    rng = np.random.default_rng(92)
+    specs = [scangen.GridSpec(origin=(-20.0, -20.0, -1.0), res_m=r, dims=(int(40 / r), int(39 / r), int(8 / r)), feature=f,
+                              count_levels=7, var_levels=8 if f == 2 else 15) for r, f in ((0.5, 2), (1.0, 1), (0.5, 0), (1.0, 2))]
+    grids = []
+    for spec in specs:
+        L = lib_grid(spec)
+        align.align_set_reference(L, tiny.xyzA)
+        grids.append(L)
+    b = align.align_batch_create()
+    for shift in (0.0, 0.07):
+        sets = [_lattice((3, 20, 2, 2, 1, 4), SMALL, centre=tiny.T + shift), _lattice((9, 13, 2, 2, 1, 3), SMALL, (0, 1, 2, 3, 4, 5)),
+                tiny.T + rng.uniform(-0.5, 0.5, (40, 6)), _lattice((3, 20, 2, 2, 1, 4), SMALL, centre=tiny.T - shift)]
+        pairs = [(L, tiny.xyzB[k::2], etas) for k, (L, etas) in enumerate(zip(grids, sets))]
+        got = align.align_eval_batch(b, pairs, graph=graph)
+        for (mi, am), (L, B, etas) in zip(got, pairs):
+            align.align_set_sweep(L, 0)
+            mi0, am0, _ = align.align_eval_mi(L, B, eta6=etas)
+            align.align_set_sweep(L, -1)
+            assert np.array_equal(mi.view(np.int32), mi0.view(np.int32)) and am == am0
+    align.align_batch_destroy(b)
