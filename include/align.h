@@ -176,15 +176,17 @@ align_status align_refine_nm(align_grid* grid, const float* xyzB, int64_t nB, in
    swept its poses: 0 one pose per CTA, 1 pose pairs (two poses per CTA that share their
    rotation, t_y and t_z), 2 one pose per 2-CTA cluster sharing a table split between the
    two CTAs' shared memories (grids whose single poses need 8 or more key partitions),
-   3 a pose lattice by groups that share the voxel map (no table: [0] stays as the others
-   left it, [2] too).
+   3 a pose lattice by groups that share the voxel map, 4 up to 32 poses with rotations of
+   their own (or one pose) with their points spread over the GPU (3, 4: no table, [0] and [2]
+   stay as the others left them).
    Each way learns its own key-partition count; results are the same whichever runs. */
 align_status align_eval_stats(align_grid* grid, int64_t out[6]);
 
 /* How this grid's launches sweep their poses (the kinds of align_eval_stats [5]): -1
    automatic (the default: a batch of poses that is a lattice, i.e. every combination of some
    rotations and some t'_x, t'_y, t'_z, is evaluated by groups where these fill the GPU and no
-   histograms are asked for; otherwise pairs while their tables need no more key partitions than
+   histograms are asked for; up to 32 poses whose rotations do not repeat, or one pose,
+   are spread over the GPU; otherwise pairs while their tables need no more key partitions than
    single poses', or, with spill queues and both partitioned, no more than twice as many up
    to 8; the cluster while single poses need 8 or more key partitions), 0 one pose per CTA, 1 pose
    pairs wherever the poses form pairs (single poses elsewhere), 2 one pose per 2-CTA

@@ -366,7 +366,8 @@ def align_refine_nm(grid: Grid, xyzB, starts, step=(8.0, 8.0, 1.0, 0.1, 0.1, 0.8
     return T, mi, it
 
 
-SWEEP_KINDS = {0: "one pose per CTA", 1: "pose pairs", 2: "2-CTA cluster", 3: "pose lattice by groups"}
+SWEEP_KINDS = {0: "one pose per CTA", 1: "pose pairs", 2: "2-CTA cluster", 3: "pose lattice by groups",
+               4: "points spread over the GPU"}
 
 
 def align_eval_stats(grid: Grid):

@@ -247,6 +247,29 @@ cudaError_t lattice_setup();  // once per device, before any launch
 // kernels launched to *launches.
 cudaError_t launch_lattice(LatticeArgs a, int32_t n_rot, int n_sm, cudaStream_t s, int32_t* launches);
 
+// Poses that share nothing, their points spread over the GPU (scatter_eval.cu).
+constexpr int64_t kScatterMaxPoints = (int64_t)1 << 22;  // the packed sums' bound
+struct ScatterArgs {
+  GridConst gc;
+  const uint8_t* symA;
+  const float* xyz;          // n x 3
+  int64_t n;
+  const float* poses;        // P x 12
+  int32_t P;
+  int64_t V;
+  unsigned long long* sums;  // P x V x 2 (1 without z sums), zero between calls
+  uint32_t* list;            // P x list_cap: occupied voxels
+  int64_t list_cap;
+  uint32_t* list_n;          // P
+  uint32_t* wide_count;      // voxels past the 32-bit sums
+  uint32_t* out_c;           // P x K x K, and up to 3 words of padding
+  int32_t* out_box;          // P x 6
+  uint32_t* redo_count;      // set to 0 (no pose needs the exact path)
+  unsigned long long* best;
+};
+size_t scatter_pose_bytes(const GridConst& gc, int64_t n);  // sums and list of one pose
+cudaError_t launch_scatter(const ScatterArgs& a, int n_sm, cudaStream_t s, int32_t* launches);
+
 cudaError_t launch_ref_accumulate(const GridConst& gc, const float* xyz, int64_t n, const float* pose12,
                                   uint32_t* cnt, unsigned long long* s1, unsigned long long* s2,
                                   cudaStream_t s);

@@ -93,4 +93,46 @@ __device__ __forceinline__ int feature_symbol(int feature, int Lc, int Lv, const
   return 1 + count_level(ct, Lc, n) * Lv + var_level(vt, Lv, n, s1, s2);
 }
 
+// Feature symbol of a voxel whose sums fit the 32-bit table (n <= nlim, so n*S2 < 2^64 and
+// S1^2 < 2^62): the same integer tests as feature_symbol, in 64-bit arithmetic.  The variance
+// test n*S2 - S1^2 >= t*n^2 compares the 128-bit product t*n^2 by its high and low words.
+__device__ __forceinline__ int feature_symbol_small(const GridConst& gc, uint32_t n, int32_t s1, uint32_t s2) {
+  if (n == 0u) return 0;
+  int lc = 0, lv = 0;
+  if (gc.feature != 1) {  // count level: #{j : n >= ct[j]}, a prefix of the ascending thresholds
+    int lo = 0, hi = gc.Lc - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (n >= gc.count_thresh[mid]) lo = mid + 1;
+      else hi = mid;
+    }
+    lc = lo;
+  }
+  if (gc.feature != 0) {  // variance level: #{j : n*S2 - S1^2 >= vt[j] * n^2}
+    const uint64_t spread = (uint64_t)n * s2 - (uint64_t)((int64_t)s1 * s1);  // >= 0 (Cauchy-Schwarz)
+    int lo = 0, hi = gc.Lv - 1;
+    if (gc.sym32) {  // n < 2^16 and every threshold < 2^32: t * n^2 is one 32 x 32-bit product
+      const uint32_t n2 = n * n;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if ((uint64_t)(uint32_t)gc.var_thresh[mid] * n2 <= spread) lo = mid + 1;
+        else hi = mid;
+      }
+    } else {
+      const uint64_t n2 = (uint64_t)n * n;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        const uint64_t t = (uint64_t)gc.var_thresh[mid];  // thresholds are >= 0
+        const bool reached = __umul64hi(t, n2) == 0ull && t * n2 <= spread;
+        if (reached) lo = mid + 1;
+        else hi = mid;
+      }
+    }
+    lv = lo;
+  }
+  if (gc.feature == 0) return 1 + lc;
+  if (gc.feature == 1) return 1 + lv;
+  return 1 + lc * gc.Lv + lv;
+}
+
 }  // namespace mialign

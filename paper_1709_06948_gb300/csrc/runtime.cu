@@ -390,6 +390,7 @@ align_status enqueue_eval_core(align_grid* g, int32_t n_tiles, const float* d_po
 align_status enqueue_lattice(align_grid* g, LatticeArgs a, const float* d_poses, const int32_t* d_pose_of,
                              int32_t n_rot, const EvalOut& out);
 bool reserve_lattice(align_grid* g, LatticeArgs a);
+align_status enqueue_scatter(align_grid* g, const float* d_poses, int64_t P, const EvalOut& out, bool* taken);
 
 }  // namespace
 
@@ -600,6 +601,12 @@ align_status enqueue_eval(align_grid* g, int32_t n_tiles, const float* d_poses, 
       n_rot = groups;
     }
   }
+  // poses that share no rotations (or a single pose): spread over the GPU
+  if ((rotate || P == 1) && P <= kScatterMaxPoses && out.dump == nullptr && g->sweep_mode < 0) {
+    bool taken = false;
+    align_status st = enqueue_scatter(g, d_poses, P, out, &taken);
+    if (st != ALIGN_OK || taken) return st;
+  }
   return enqueue_eval_core(g, n_tiles, d_poses, P, rotate, n_rot, out, nullptr, 0,
                            out.dump == nullptr && use_cluster(g));
 }
@@ -732,6 +739,22 @@ align_status enqueue_eval_core(align_grid* g, int32_t n_tiles, const float* d_po
   return ALIGN_OK;
 }
 
+// Record event i of a launch's (before eval, after eval, after argmax) while profiling.
+align_status profile_event(align_grid* g, std::array<cudaEvent_t, 3>& evs, int i) {
+  if (!g->profiling) return ALIGN_OK;
+  if (i == 0) {
+    if (g->ev_pool.empty()) {
+      for (cudaEvent_t& v : evs) CU(cudaEventCreate(&v), "create event");
+    } else {
+      evs = g->ev_pool.back();
+      g->ev_pool.pop_back();
+    }
+  }
+  CU(cudaEventRecord(evs[(size_t)i], g->stream), "record event");
+  if (i == 2) g->ev_pending.push_back(evs);
+  return ALIGN_OK;
+}
+
 // The groups' workspace; without the memory for it the table kernels take the poses.
 bool reserve_lattice(align_grid* g, LatticeArgs a) {
   if (g->lattice_ws.ensure(lattice_carve(a, nullptr)) == cudaSuccess) return true;
@@ -807,29 +830,102 @@ align_status enqueue_lattice(align_grid* g, LatticeArgs a, const float* d_poses,
   e.wide = g->wide.as<unsigned long long>();
 
   std::array<cudaEvent_t, 3> evs{};
-  if (g->profiling) {
-    if (g->ev_pool.empty()) {
-      for (cudaEvent_t& v : evs) CU(cudaEventCreate(&v), "create event");
-    } else {
-      evs = g->ev_pool.back();
-      g->ev_pool.pop_back();
-    }
-    CU(cudaEventRecord(evs[0], g->stream), "record event");
-  }
+  if ((st = profile_event(g, evs, 0)) != ALIGN_OK) return st;
   int32_t launches = 0;
   CU(launch_lattice(a, n_rot, g->n_sm, g->stream, &launches), "launch lattice evaluation");
   CU(ek.launch_redo_raw(e, redo_ctas, vw, g->stream), "launch redo kernel");
-  if (g->profiling) CU(cudaEventRecord(evs[1], g->stream), "record event");
+  if ((st = profile_event(g, evs, 1)) != ALIGN_OK) return st;
   CU(ek.launch_compose(e, g->stream), "launch compose kernel");
   CU(ek.launch_argmax_finalize(e.items, 1, g->stream), "launch argmax");
-  if (g->profiling) {
-    CU(cudaEventRecord(evs[2], g->stream), "record event");
-    g->ev_pending.push_back(evs);
-  }
+  if ((st = profile_event(g, evs, 2)) != ALIGN_OK) return st;
   g->stats[4] += launches + 3;  // and redo, compose, argmax
   g->stats[3] = g->n_sm * (1024 / a.threads);
   g->stats[5] = 3;
   g->last_lattice = true;
+  return ALIGN_OK;
+}
+
+// Poses that share nothing: their points spread over the GPU (scatter_eval.cu).  *taken: whether
+// this path took them (not: more points than its sums hold, or no memory for the sums).
+align_status enqueue_scatter(align_grid* g, const float* d_poses, int64_t P, const EvalOut& out, bool* taken) {
+  *taken = false;
+  const size_t one = scatter_pose_bytes(g->gc, g->n_points);
+  if (g->n_points > kScatterMaxPoints || one * (size_t)P > kScatterBudget) return ALIGN_OK;
+  ScatterArgs a{};
+  a.gc = g->gc;
+  a.n = g->n_points;
+  a.P = (int32_t)P;
+  a.V = g->V;
+  a.list_cap = std::min<int64_t>(g->V, std::max<int64_t>(a.n, 1));
+  const size_t words = g->gc.feature != ALIGN_FEAT_COUNT ? 16 : 8;
+  const size_t sum_bytes = (size_t)P * (size_t)g->V * words;
+  if (g->scatter_sums.cap < sum_bytes || g->scatter_sums.p == nullptr) {
+    if (g->scatter_sums.ensure(sum_bytes) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return ALIGN_OK;
+    }
+    CU(cudaMemsetAsync(g->scatter_sums.p, 0, g->scatter_sums.cap, g->stream), "clear sums");
+  }
+  if (g->scatter_list.ensure((size_t)P * (size_t)a.list_cap * 4) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return ALIGN_OK;
+  }
+  *taken = true;
+  const size_t KK = (size_t)g->gc.K * g->gc.K;
+  CU(g->out_c.ensure((size_t)P * KK * sizeof(uint32_t) + 16), "allocate histograms");
+  CU(g->out_box.ensure((size_t)P * 6 * sizeof(int32_t)), "allocate boxes");
+  CU(g->best.ensure(sizeof(unsigned long long)), "allocate argmax");
+  CU(g->redo_list.ensure((size_t)P * 4), "allocate redo list");
+  CU(g->redo_count.ensure(16), "allocate redo count");
+  CU(g->scatter_n.ensure((size_t)P * 4), "allocate list sizes");
+  align_status st = ensure_status_words(g);
+  if (st != ALIGN_OK) return st;
+  a.symA = g->symA.as<uint8_t>();
+  a.xyz = g->xyz.as<float>();
+  a.poses = d_poses;
+  a.sums = g->scatter_sums.as<unsigned long long>();
+  a.list = g->scatter_list.as<uint32_t>();
+  a.list_n = g->scatter_n.as<uint32_t>();
+  a.wide_count = g->wide_count.as<uint32_t>();
+  a.out_c = g->out_c.as<uint32_t>();
+  a.out_box = g->out_box.as<int32_t>();
+  a.redo_count = g->redo_count.as<uint32_t>();
+  a.best = g->best.as<unsigned long long>();
+
+  EvalItem item{};
+  item.gc = g->gc;
+  item.symA = a.symA;
+  item.sat = g->sat.as<int32_t>();
+  item.poses = d_poses;
+  item.P = (int32_t)P;
+  item.out_c = a.out_c;
+  item.out_box = a.out_box;
+  item.mi = out.mi;
+  item.hist = out.hist;
+  item.best = a.best;
+  item.argmax = out.argmax;
+  CU(g->items.ensure(sizeof(EvalItem)), "allocate item table");
+  CU(cudaMemcpyAsync(g->items.p, &item, sizeof(EvalItem), cudaMemcpyHostToDevice, g->stream), "copy item table");
+  EvalArgs e{};
+  e.one = item;
+  e.items = g->items.as<EvalItem>();
+  e.n_items = 1;
+  e.P = (int32_t)P;
+  e.K = g->gc.K;
+  const EvalKernels& ek = eval_shape(0);
+  std::array<cudaEvent_t, 3> evs{};
+  st = profile_event(g, evs, 0);
+  if (st != ALIGN_OK) return st;
+  int32_t launches = 0;
+  CU(launch_scatter(a, g->n_sm, g->stream, &launches), "launch scattered evaluation");
+  if ((st = profile_event(g, evs, 1)) != ALIGN_OK) return st;
+  CU(ek.launch_compose(e, g->stream), "launch compose kernel");
+  CU(ek.launch_argmax_finalize(e.items, 1, g->stream), "launch argmax");
+  if ((st = profile_event(g, evs, 2)) != ALIGN_OK) return st;
+  g->stats[3] = 0;
+  g->stats[4] += launches + 2;  // and compose, argmax
+  g->stats[5] = 4;
+  g->last_lattice = true;  // no tables: nothing to learn
   return ALIGN_OK;
 }
 
@@ -1141,7 +1237,8 @@ align_status align_destroy_grid(align_grid* g) {
                     &g->argmax, &g->err, &g->max_passes, &g->wide_count, &g->wide, &g->dump, &g->pts4,
                     &g->pose_src, &g->rots, &g->redo_list, &g->redo_count, &g->items, &g->ovf, &g->lat_c,
                     &g->lat_cand, &g->ref_pts, &g->ref_pose, &g->ref_cnt, &g->ref_s1, &g->ref_s2, &g->ref_box,
-                    &g->units, &g->lat_units, &g->spill, &g->lattice_ws, &g->lattice_order})
+                    &g->units, &g->lat_units, &g->spill, &g->lattice_ws, &g->lattice_order, &g->scatter_sums,
+                    &g->scatter_list, &g->scatter_n})
     b->release();
   for (HostBuf* b : {&g->lat_cand_h, &g->lat_rec_h, &g->lat_c_h, &g->ref_box_h}) b->release();
   for (cudaEvent_t e : g->lat_ev) cudaEventDestroy(e);

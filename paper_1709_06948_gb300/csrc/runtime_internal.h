@@ -84,6 +84,11 @@ align_status check_grid_device(align_grid* g);
 int pair_units(const float* poses12, const PoseSet& set, int64_t P, std::vector<int32_t>& units);
 // Whether pose pairs are the automatic choice for a grid with these learned key-partition
 // counts (pairs, single poses).
+constexpr size_t kScatterBudget = (size_t)1 << 30;  // sums and lists of poses spread over the GPU
+// Beyond about this many poses a CTA per pose is faster (an L2 atomic per run, not a shared one):
+// they cross at 36 poses (0.25 m LiDAR grid), 42 (0.5 m), 56 (1 m), 22 on the 6.4M-voxel grid, where
+// the budget holds 10.
+constexpr int64_t kScatterMaxPoses = 32;
 constexpr size_t kLatticeBudget = (size_t)5 << 28;  // workspace of a round of a pose lattice (1.25 GiB)
 bool plan_lattice(const GridConst& gc, int n_sm, size_t smem_optin, int64_t n, int64_t n_rot, int32_t mx, int32_t my,
                   int32_t mz, double t_max, int min_groups, LatticeArgs& a);
@@ -139,6 +144,7 @@ struct align_grid {
                               // whose request was admitted without the groups' memory)
   mialign::DevBuf lattice_ws, lattice_order;  // groups' workspace; a device-built level's pose order
   int32_t lattice_order_m[6] = {0, 0, 0, 0, 0, 0};
+  mialign::DevBuf scatter_sums, scatter_list, scatter_n;  // poses that share nothing (zeroed sums)
   bool last_cluster = false;  // ... or ran one pose per 2-CTA cluster
   mialign::DevBuf units;    // pose pairs of the last pair launch with host poses
   mialign::DevBuf spill;    // runs queued for the later key partitions (EvalArgs::spill)
