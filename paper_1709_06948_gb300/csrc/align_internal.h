@@ -75,8 +75,9 @@ struct EvalItem {
 };
 
 struct EvalArgs {
-  EvalItem one;               // a copy of items[0] when n_items == 1 (read from the parameter bank)
-  const EvalItem* items;
+  EvalItem one;               // the item of a single-item launch (item_start == nullptr), read from the
+                              // parameter bank
+  const EvalItem* items;      // the items of the others
   const int32_t* item_start;  // n_items + 1 ascending global pose offsets (nullptr: one item)
   int32_t n_items;
   int32_t P;                  // poses over all items
@@ -155,6 +156,7 @@ struct EvalKernels {
   cudaError_t (*launch_redo_raw)(const EvalArgs& a, int n_ctas, int vw, cudaStream_t s);
   // Each item's argmax from its packed running maximum.
   cudaError_t (*launch_argmax_finalize)(const EvalItem* items, int n_items, cudaStream_t s);
+  cudaError_t (*launch_argmax_one)(const EvalItem& item, cudaStream_t s);  // a single item's
 };
 constexpr int kEvalShapes = 3;
 // Table value words per slot for a launch over grids with constants gc: 1 without z sums

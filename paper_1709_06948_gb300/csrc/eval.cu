@@ -838,9 +838,10 @@ __device__ __forceinline__ void store_point(float4* out, int64_t i, float x, flo
 __device__ __forceinline__ void select_item(const EvalSmem& S, const EvalArgs& a, int it) {
   if (*(volatile int32_t*)S.item == it) return;
   __syncthreads();
-  const uint32_t* src = reinterpret_cast<const uint32_t*>(&a.items[it].gc);
+  // a single item is read from the kernel parameters
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(a.item_start != nullptr ? &a.items[it].gc : &a.one.gc);
   uint32_t* dst = reinterpret_cast<uint32_t*>(S.gc);
-  for (int i = threadIdx.x; i < kGcWords; i += blockDim.x) dst[i] = __ldg(src + i);
+  for (int i = threadIdx.x; i < kGcWords; i += blockDim.x) dst[i] = src[i];
   __syncthreads();
   if (threadIdx.x == 0) *S.item = it;
   __syncthreads();
@@ -1706,7 +1707,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) redo_kernel(const __grid
     const int gp = (int)a.redo_list[i];
     const int it = item_of(a, gp);
     select_item(S, a, it);
-    const EvalItem& I = a.items[it];
+    const EvalItem& I = a.item_start != nullptr ? a.items[it] : a.one;
     const int lp = gp - I.pose_base;
     const VoxelConst vc = voxel_const<3>(*S.gc);
     const uint32_t run_lim = S.gc->nlim;  // runs with 32-bit sums of dz and dz^2, cut at nlim
@@ -1891,13 +1892,14 @@ __device__ __forceinline__ float neg_plogp(uint64_t c, float N) {
   return -q * logf(q);
 }
 
+template <bool kOne>
 __global__ void __launch_bounds__(kComposeThreads) compose_kernel(const __grid_constant__ EvalArgs a) {
   __shared__ uint32_t h[kMaxSymbols * kMaxSymbols];
   __shared__ long long cntA[kMaxSymbols];
   __shared__ float red[kComposeThreads / 32];
   const int gp = blockIdx.x;
   const int tid = threadIdx.x;
-  const EvalItem& I = a.items[item_of(a, gp)];
+  const EvalItem& I = item_at<kOne>(a, kOne ? 0 : item_of(a, gp));
   const GridConst& gc = I.gc;
   const int lp = gp - I.pose_base;
   const int K = gc.K, KK = K * K;
@@ -1959,12 +1961,14 @@ __global__ void __launch_bounds__(kComposeThreads) compose_kernel(const __grid_c
     for (int i = tid; i < KK; i += kComposeThreads) I.hist[(size_t)lp * KK + i] = h[i];
 }
 
+__device__ __forceinline__ int64_t best_index(unsigned long long b) {
+  return b == 0ull ? -1 : (int64_t)(0xFFFFFFFFu - (uint32_t)(b & 0xFFFFFFFFull));
+}
 __global__ void argmax_finalize_kernel(const EvalItem* items, int n_items) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n_items) return;
-  const unsigned long long b = *items[i].best;
-  *items[i].argmax = (b == 0ull) ? -1 : (int64_t)(0xFFFFFFFFu - (uint32_t)(b & 0xFFFFFFFFull));
+  if (i < n_items) *items[i].argmax = best_index(*items[i].best);
 }
+__global__ void argmax_one_kernel(const unsigned long long* best, int64_t* argmax) { *argmax = best_index(*best); }
 
 template <int kVW, bool kRot>
 cudaError_t setup_t(int smem) {
@@ -2105,7 +2109,8 @@ cudaError_t launch_pack_points(const float* xyz, int64_t n, int64_t n_out, const
 
 cudaError_t launch_compose(const EvalArgs& a, cudaStream_t s) {
   if (a.P <= 0) return cudaSuccess;
-  compose_kernel<<<a.P, kComposeThreads, 0, s>>>(a);
+  if (a.item_start != nullptr) compose_kernel<false><<<a.P, kComposeThreads, 0, s>>>(a);
+  else compose_kernel<true><<<a.P, kComposeThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -2115,12 +2120,18 @@ cudaError_t launch_argmax_finalize(const EvalItem* items, int n_items, cudaStrea
   return cudaGetLastError();
 }
 
+cudaError_t launch_argmax_one(const EvalItem& item, cudaStream_t s) {
+  argmax_one_kernel<<<1, 1, 0, s>>>(item.best, item.argmax);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 const EvalKernels& MI_EVAL_SHAPE_FN() {
   static const EvalKernels k{MI_STR(MI_EVAL_SHAPE_FN), kThreads, kPPT, kCtasPerSm, eval_tile_points, eval_ovf_cap, eval_min_tiles,
                              eval_smem_bytes, eval_table_slots_for, eval_setup, launch_eval, launch_pack_points,
-                             launch_pack_batch, launch_compose, launch_redo_raw, launch_argmax_finalize};
+                             launch_pack_batch, launch_compose, launch_redo_raw, launch_argmax_finalize,
+                             launch_argmax_one};
   return k;
 }
 

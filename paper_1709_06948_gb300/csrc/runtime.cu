@@ -9,6 +9,7 @@
 #include <climits>
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -285,15 +286,12 @@ struct RotHash {
   }
 };
 
-// Error word and counters: allocated once per grid and zeroed (cudaMalloc memory is not).
-align_status ensure_status_words(align_grid* g) {
-  if (g->err.p && g->max_passes.p && g->wide_count.p) return ALIGN_OK;
-  CU(g->err.ensure(16), "allocate error word");
-  CU(g->max_passes.ensure(16), "allocate counters");
-  CU(g->wide_count.ensure(16), "allocate counters");
-  CU(cudaMemsetAsync(g->err.p, 0, 16, g->stream), "clear error word");
-  CU(cudaMemsetAsync(g->max_passes.p, 0, 16, g->stream), "clear counters");
-  CU(cudaMemsetAsync(g->wide_count.p, 0, 16, g->stream), "clear counters");
+// The grid's head block: allocated once, its counters zeroed (cudaMalloc memory is not).
+align_status ensure_head(align_grid* g) {
+  if (g->head.p) return ALIGN_OK;
+  CU(g->head_h.ensure(kHeadBytes), "allocate pinned results");
+  CU(g->head.ensure(kHeadBytes), "allocate results");
+  CU(cudaMemsetAsync(g->head.p, 0, sizeof(GridHead), g->stream), "clear counters");
   return ALIGN_OK;
 }
 
@@ -620,8 +618,7 @@ align_status enqueue_eval_core(align_grid* g, int32_t n_tiles, const float* d_po
   const size_t KK = (size_t)K * K;
   CU(g->out_c.ensure((size_t)P * KK * sizeof(uint32_t)), "allocate histograms");
   CU(g->out_box.ensure((size_t)P * 6 * sizeof(int32_t)), "allocate boxes");
-  CU(g->best.ensure(sizeof(unsigned long long)), "allocate argmax");
-  align_status st0 = ensure_status_words(g);
+  align_status st0 = ensure_head(g);
   if (st0 != ALIGN_OK) return st0;
   const bool pairs = d_units != nullptr && n_units > 0 && !rotate;
   cluster = cluster && !pairs;
@@ -639,7 +636,7 @@ align_status enqueue_eval_core(align_grid* g, int32_t n_tiles, const float* d_po
     CU(g->wide.ensure(wide_bytes), "allocate wide sums");
     CU(cudaMemsetAsync(g->wide.p, 0, g->wide.cap, g->stream), "clear wide sums");
   }
-  CU(cudaMemsetAsync(g->best.p, 0, sizeof(unsigned long long), g->stream), "reset argmax");
+  CU(cudaMemsetAsync(&g->dev_head()->best, 0, sizeof(unsigned long long), g->stream), "reset argmax");
   CU(g->redo_list.ensure((size_t)P * 4), "allocate redo list");
   CU(g->redo_count.ensure(16), "allocate redo count");
   CU(cudaMemsetAsync(g->redo_count.p, 0, 4, g->stream), "reset redo count");
@@ -673,15 +670,12 @@ align_status enqueue_eval_core(align_grid* g, int32_t n_tiles, const float* d_po
   item.out_box = g->out_box.as<int32_t>();
   item.mi = out.mi;
   item.hist = out.hist;
-  item.best = g->best.as<unsigned long long>();
+  item.best = &g->dev_head()->best;
   item.argmax = out.argmax;
   item.dump = out.dump;
-  CU(g->items.ensure(sizeof(EvalItem)), "allocate item table");
-  CU(cudaMemcpyAsync(g->items.p, &item, sizeof(EvalItem), cudaMemcpyHostToDevice, g->stream), "copy item table");
 
   EvalArgs a{};
   a.one = item;
-  a.items = g->items.as<EvalItem>();
   a.item_start = nullptr;
   a.n_items = 1;
   a.P = (int32_t)P;
@@ -692,10 +686,10 @@ align_status enqueue_eval_core(align_grid* g, int32_t n_tiles, const float* d_po
   a.units = pairs ? d_units : nullptr;
   a.n_units = pairs ? n_units : 0;
   a.cluster = cluster ? 1 : 0;
-  a.err = g->err.as<uint32_t>();
-  a.max_passes = g->max_passes.as<uint32_t>();
-  a.wide_count = g->wide_count.as<uint32_t>();
-  a.wide_poses = g->wide_count.as<uint32_t>() + 1;  // the counter buffer's second word
+  a.err = &g->dev_head()->err;
+  a.max_passes = &g->dev_head()->max_passes;
+  a.wide_count = &g->dev_head()->wide_count;
+  a.wide_poses = &g->dev_head()->wide_poses;
   a.wide = g->wide.as<unsigned long long>();
   a.redo_list = g->redo_list.as<uint32_t>();
   a.redo_count = g->redo_count.as<uint32_t>();
@@ -727,7 +721,7 @@ align_status enqueue_eval_core(align_grid* g, int32_t n_tiles, const float* d_po
   CU(ek.launch_eval(a, n_ctas, vw, rotate, g->stream), "launch eval kernel");
   if (g->profiling) CU(cudaEventRecord(evs[1], g->stream), "record event");
   CU(ek.launch_compose(a, g->stream), "launch compose kernel");
-  CU(ek.launch_argmax_finalize(a.items, 1, g->stream), "launch argmax");
+  CU(ek.launch_argmax_one(item, g->stream), "launch argmax");
   if (g->profiling) {
     CU(cudaEventRecord(evs[2], g->stream), "record event");
     g->ev_pending.push_back(evs);
@@ -771,10 +765,9 @@ align_status enqueue_lattice(align_grid* g, LatticeArgs a, const float* d_poses,
   CU(lattice_setup(), "set up lattice kernels");
   CU(g->out_c.ensure((size_t)P * KK * sizeof(uint32_t) + 16), "allocate histograms");
   CU(g->out_box.ensure((size_t)P * 6 * sizeof(int32_t)), "allocate boxes");
-  CU(g->best.ensure(sizeof(unsigned long long)), "allocate argmax");
   CU(g->redo_list.ensure((size_t)P * 4), "allocate redo list");
   CU(g->redo_count.ensure(16), "allocate redo count");
-  align_status st = ensure_status_words(g);
+  align_status st = ensure_head(g);
   if (st != ALIGN_OK) return st;
   lattice_carve(a, g->lattice_ws.as<uint8_t>());
   a.symA = g->symA.as<uint8_t>();
@@ -785,7 +778,7 @@ align_status enqueue_lattice(align_grid* g, LatticeArgs a, const float* d_poses,
   a.out_box = g->out_box.as<int32_t>();
   a.redo_list = g->redo_list.as<uint32_t>();
   a.redo_count = g->redo_count.as<uint32_t>();
-  a.best = g->best.as<unsigned long long>();
+  a.best = &g->dev_head()->best;
 
   // poses with a voxel past the 32-bit sums: the redo kernel, reading the scan itself
   const EvalKernels& ek = eval_shape(0);
@@ -806,20 +799,17 @@ align_status enqueue_lattice(align_grid* g, LatticeArgs a, const float* d_poses,
   item.hist = out.hist;
   item.best = a.best;
   item.argmax = out.argmax;
-  CU(g->items.ensure(sizeof(EvalItem)), "allocate item table");
-  CU(cudaMemcpyAsync(g->items.p, &item, sizeof(EvalItem), cudaMemcpyHostToDevice, g->stream), "copy item table");
   EvalArgs e{};
   e.one = item;
-  e.items = g->items.as<EvalItem>();
   e.n_items = 1;
   e.P = (int32_t)P;
   e.K = g->gc.K;
   e.table_slots = ek.table_slots_for(e.K, vw, g->smem_optin, 1);
   e.n_buckets = e.table_slots / 4;
   e.passes0 = 1;
-  e.err = g->err.as<uint32_t>();
-  e.max_passes = g->max_passes.as<uint32_t>();
-  e.wide_count = g->wide_count.as<uint32_t>();
+  e.err = &g->dev_head()->err;
+  e.max_passes = &g->dev_head()->max_passes;
+  e.wide_count = &g->dev_head()->wide_count;
   e.redo_list = a.redo_list;
   e.redo_count = a.redo_count;
   const size_t wide_bytes = (size_t)redo_ctas * 2 * e.table_slots * sizeof(unsigned long long);
@@ -836,7 +826,7 @@ align_status enqueue_lattice(align_grid* g, LatticeArgs a, const float* d_poses,
   CU(ek.launch_redo_raw(e, redo_ctas, vw, g->stream), "launch redo kernel");
   if ((st = profile_event(g, evs, 1)) != ALIGN_OK) return st;
   CU(ek.launch_compose(e, g->stream), "launch compose kernel");
-  CU(ek.launch_argmax_finalize(e.items, 1, g->stream), "launch argmax");
+  CU(ek.launch_argmax_one(item, g->stream), "launch argmax");
   if ((st = profile_event(g, evs, 2)) != ALIGN_OK) return st;
   g->stats[4] += launches + 3;  // and redo, compose, argmax
   g->stats[3] = g->n_sm * (1024 / a.threads);
@@ -874,11 +864,10 @@ align_status enqueue_scatter(align_grid* g, const float* d_poses, int64_t P, con
   const size_t KK = (size_t)g->gc.K * g->gc.K;
   CU(g->out_c.ensure((size_t)P * KK * sizeof(uint32_t) + 16), "allocate histograms");
   CU(g->out_box.ensure((size_t)P * 6 * sizeof(int32_t)), "allocate boxes");
-  CU(g->best.ensure(sizeof(unsigned long long)), "allocate argmax");
   CU(g->redo_list.ensure((size_t)P * 4), "allocate redo list");
   CU(g->redo_count.ensure(16), "allocate redo count");
   CU(g->scatter_n.ensure((size_t)P * 4), "allocate list sizes");
-  align_status st = ensure_status_words(g);
+  align_status st = ensure_head(g);
   if (st != ALIGN_OK) return st;
   a.symA = g->symA.as<uint8_t>();
   a.xyz = g->xyz.as<float>();
@@ -886,11 +875,11 @@ align_status enqueue_scatter(align_grid* g, const float* d_poses, int64_t P, con
   a.sums = g->scatter_sums.as<unsigned long long>();
   a.list = g->scatter_list.as<uint32_t>();
   a.list_n = g->scatter_n.as<uint32_t>();
-  a.wide_count = g->wide_count.as<uint32_t>();
+  a.wide_count = &g->dev_head()->wide_count;
   a.out_c = g->out_c.as<uint32_t>();
   a.out_box = g->out_box.as<int32_t>();
   a.redo_count = g->redo_count.as<uint32_t>();
-  a.best = g->best.as<unsigned long long>();
+  a.best = &g->dev_head()->best;
 
   EvalItem item{};
   item.gc = g->gc;
@@ -904,11 +893,8 @@ align_status enqueue_scatter(align_grid* g, const float* d_poses, int64_t P, con
   item.hist = out.hist;
   item.best = a.best;
   item.argmax = out.argmax;
-  CU(g->items.ensure(sizeof(EvalItem)), "allocate item table");
-  CU(cudaMemcpyAsync(g->items.p, &item, sizeof(EvalItem), cudaMemcpyHostToDevice, g->stream), "copy item table");
   EvalArgs e{};
   e.one = item;
-  e.items = g->items.as<EvalItem>();
   e.n_items = 1;
   e.P = (int32_t)P;
   e.K = g->gc.K;
@@ -920,7 +906,7 @@ align_status enqueue_scatter(align_grid* g, const float* d_poses, int64_t P, con
   CU(launch_scatter(a, g->n_sm, g->stream, &launches), "launch scattered evaluation");
   if ((st = profile_event(g, evs, 1)) != ALIGN_OK) return st;
   CU(ek.launch_compose(e, g->stream), "launch compose kernel");
-  CU(ek.launch_argmax_finalize(e.items, 1, g->stream), "launch argmax");
+  CU(ek.launch_argmax_one(item, g->stream), "launch argmax");
   if ((st = profile_event(g, evs, 2)) != ALIGN_OK) return st;
   g->stats[3] = 0;
   g->stats[4] += launches + 2;  // and compose, argmax
@@ -954,31 +940,34 @@ void learn_passes(align_grid* g, uint32_t used) {
   if (used > (uint32_t)seed) seed = (int32_t)used;
 }
 
-// Read back the kernels' error word and counters (synchronises the stream).
-align_status collect_status(align_grid* g) {
-  uint32_t vals[4] = {0, 0, 0, 0};
-  CU(cudaMemcpyAsync(&vals[0], g->err.p, 4, cudaMemcpyDeviceToHost, g->stream), "read error word");
-  CU(cudaMemcpyAsync(&vals[1], g->max_passes.p, 4, cudaMemcpyDeviceToHost, g->stream), "read counters");
-  CU(cudaMemcpyAsync(&vals[2], g->wide_count.p, 8, cudaMemcpyDeviceToHost, g->stream), "read counters");
+// Read back the head block and the MI of n_mi poses behind it (synchronises the stream).
+align_status read_head(align_grid* g, int64_t n_mi) {
+  CU(cudaMemcpyAsync(g->head_h.p, g->head.p, sizeof(GridHead) + (size_t)n_mi * 4, cudaMemcpyDeviceToHost, g->stream),
+     "read results");
   CU(cudaStreamSynchronize(g->stream), "synchronize");
+  return ALIGN_OK;
+}
+
+// The counters of a head that was read: learn from them, reset them, report errors.
+align_status collect_status(align_grid* g) {
+  const GridHead& h = *g->head_h.as<GridHead>();
   {
     align_status stp = drain_events(g);
     if (stp != ALIGN_OK) return stp;
   }
-  CU(cudaMemsetAsync(g->err.p, 0, 4, g->stream), "reset error word");
-  CU(cudaMemsetAsync(g->wide_count.p, 0, 8, g->stream), "reset counters");
-  CU(cudaMemsetAsync(g->max_passes.p, 0, 4, g->stream), "reset counters");  // a per-launch maximum
+  // (max_passes is a per-launch maximum)
+  CU(cudaMemsetAsync(g->head.p, 0, offsetof(GridHead, argmax), g->stream), "reset counters");
   // seed the next launch of the same kind (pairs or single poses) with the largest
   // partition count a pose needed (a power of two)
-  learn_passes(g, vals[1]);
+  learn_passes(g, h.max_passes);
   // packed-layout poses that a voxel past nlim_pack sent to the exact path: the grid's scans
   // are dense enough for the three-word layout (a limit several times larger, fewer slots)
-  if (vals[3] > 0 && g->last_vw == 2 && !g->last_lattice) g->layout_min = 3;
-  g->stats[0] = vals[1];
-  g->stats[1] = vals[2];
-  if (vals[0] & kErrDzBound) return fail(ALIGN_E_INTERNAL, "a z offset exceeded its proven bound");
-  if (vals[0] & kErrPassLimit) return fail(ALIGN_E_INTERNAL, "key partitioning limit reached");
-  if (vals[0] & kErrLattice) return fail(ALIGN_E_INTERNAL, "a lattice level found its argmax out of range");
+  if (h.wide_poses > 0 && g->last_vw == 2 && !g->last_lattice) g->layout_min = 3;
+  g->stats[0] = h.max_passes;
+  g->stats[1] = h.wide_count;
+  if (h.err & kErrDzBound) return fail(ALIGN_E_INTERNAL, "a z offset exceeded its proven bound");
+  if (h.err & kErrPassLimit) return fail(ALIGN_E_INTERNAL, "key partitioning limit reached");
+  if (h.err & kErrLattice) return fail(ALIGN_E_INTERNAL, "a lattice level found its argmax out of range");
   return ALIGN_OK;
 }
 
@@ -1012,21 +1001,14 @@ align_status search_pipelined(align_grid* g, int32_t n_tiles, const double c0[6]
                               const int32_t m[6], int64_t P, int32_t n_rot, int32_t levels, double T_out[6],
                               float* mi_out, int64_t* level_best) {
   const size_t slot = (size_t)n_rot * n_rot * 9;  // floats of one level's rotation table
-  struct Rec {
-    int64_t am;
-    unsigned long long best;
-    uint32_t max_passes;
-    uint32_t pad;
-  };
   CU(g->lat_c.ensure((size_t)(levels + 1) * 6 * sizeof(double)), "allocate lattice centres");
   CU(g->lat_cand.ensure(2 * slot * sizeof(float)), "allocate rotation tables");
   CU(g->poses.ensure((size_t)P * 48), "allocate poses");
   CU(g->rots.ensure((size_t)n_rot * 36), "allocate rotations");
   CU(g->pose_src.ensure((size_t)P * 4), "allocate pose sources");
   CU(g->mi.ensure((size_t)P * 4), "allocate MI");
-  CU(g->argmax.ensure(8), "allocate argmax");
   CU(g->lat_cand_h.ensure(2 * slot * sizeof(float)), "allocate pinned rotation tables");
-  CU(g->lat_rec_h.ensure((size_t)levels * sizeof(Rec)), "allocate pinned read-back");
+  CU(g->lat_rec_h.ensure((size_t)levels * sizeof(GridHead)), "allocate pinned read-back");
   CU(g->lat_c_h.ensure(6 * sizeof(double)), "allocate pinned centre");
   while ((int32_t)g->lat_ev.size() < levels) {
     cudaEvent_t e;
@@ -1082,7 +1064,7 @@ align_status search_pipelined(align_grid* g, int32_t n_tiles, const double c0[6]
     }
     n_units = (int32_t)(g->lattice_units.size() / 2);
   }
-  Rec* rec = g->lat_rec_h.as<Rec>();
+  GridHead* rec = g->lat_rec_h.as<GridHead>();  // each level's head (max_passes: over the levels so far)
   std::vector<std::array<double, 6>> c((size_t)levels + 1), r((size_t)levels);
   for (int a = 0; a < 6; ++a) c[0][a] = c0[a], r[0][a] = r0[a];
   for (int32_t l = 1; l < levels; ++l)
@@ -1095,9 +1077,9 @@ align_status search_pipelined(align_grid* g, int32_t n_tiles, const double c0[6]
   for (int32_t l = 0; l < levels; ++l) {
     if (l >= 2) {  // level l-1's centre, from level l-2's argmax
       CU(cudaEventSynchronize(g->lat_ev[(size_t)l - 2]), "wait for a lattice level");
-      const Rec& q = rec[l - 2];
-      if (q.am < 0 || q.am >= P) return fail(ALIGN_E_INTERNAL, "argmax out of range");
-      lattice_sample(c[(size_t)l - 2].data(), r[(size_t)l - 2].data(), m, q.am, c[(size_t)l - 1].data());
+      const GridHead& q = rec[l - 2];
+      if (q.argmax < 0 || q.argmax >= P) return fail(ALIGN_E_INTERNAL, "argmax out of range");
+      lattice_sample(c[(size_t)l - 2].data(), r[(size_t)l - 2].data(), m, q.argmax, c[(size_t)l - 1].data());
       passes_used = std::max(passes_used, q.max_passes);
       learn_passes(g, q.max_passes);
     }
@@ -1141,41 +1123,38 @@ align_status search_pipelined(align_grid* g, int32_t n_tiles, const double c0[6]
     L.n_rot = n_rot;
     L.P = (int32_t)P;
     L.c_prev = d_c + 6 * (size_t)l;
-    L.am_prev = l > 0 ? g->argmax.as<int64_t>() : nullptr;
+    L.am_prev = l > 0 ? &g->dev_head()->argmax : nullptr;
     L.cand = d_tab;
     L.c_out = d_c + 6 * ((size_t)l + 1);
     L.poses = g->poses.as<float>();
     L.pose_src = g->pose_src.as<int32_t>();
     L.rots = g->rots.as<float>();
-    L.err = g->err.as<uint32_t>();
+    L.err = &g->dev_head()->err;
     CU(launch_lattice_level(L, g->stream), "launch lattice level");
     g->stats[4] += 1;
     EvalOut o{};
     o.mi = g->mi.as<float>();
-    o.argmax = g->argmax.as<int64_t>();
+    o.argmax = &g->dev_head()->argmax;
     align_status st = by_groups
                           ? enqueue_lattice(g, lat, g->poses.as<float>(), d_order, n_rot, o)
                           : enqueue_eval_core(g, n_tiles, g->poses.as<float>(), P, false, n_rot, o,
                                               pairs ? g->lat_units.as<int32_t>() : nullptr, n_units,
                                               !pairs && cluster);
     if (st != ALIGN_OK) return st;
-    CU(cudaMemcpyAsync(&rec[l].am, g->argmax.p, 8, cudaMemcpyDeviceToHost, g->stream), "read argmax");
-    CU(cudaMemcpyAsync(&rec[l].best, g->best.p, 8, cudaMemcpyDeviceToHost, g->stream), "read best");
-    CU(cudaMemcpyAsync(&rec[l].max_passes, g->max_passes.p, 4, cudaMemcpyDeviceToHost, g->stream),
-       "read counters");
-    CU(cudaMemsetAsync(g->max_passes.p, 0, 4, g->stream), "reset counters");
+    CU(cudaMemcpyAsync(&rec[l], g->head.p, sizeof(GridHead), cudaMemcpyDeviceToHost, g->stream), "read argmax");
     CU(cudaEventRecord(g->lat_ev[(size_t)l], g->stream), "record event");
   }
-  align_status st = collect_status(g);  // synchronises the stream
+  align_status st = read_head(g, 0);
+  if (st == ALIGN_OK) st = collect_status(g);
   if (st != ALIGN_OK) return st;
   g->lat_pending = false;
   for (int32_t l = std::max(0, levels - 2); l < levels; ++l) {
-    if (rec[l].am < 0 || rec[l].am >= P) return fail(ALIGN_E_INTERNAL, "argmax out of range");
-    lattice_sample(c[(size_t)l].data(), r[(size_t)l].data(), m, rec[l].am, c[(size_t)l + 1].data());
+    if (rec[l].argmax < 0 || rec[l].argmax >= P) return fail(ALIGN_E_INTERNAL, "argmax out of range");
+    lattice_sample(c[(size_t)l].data(), r[(size_t)l].data(), m, rec[l].argmax, c[(size_t)l + 1].data());
   }
   for (int32_t l = 0; l < levels; ++l) {
     passes_used = std::max(passes_used, rec[l].max_passes);
-    if (level_best) level_best[l] = rec[l].am;
+    if (level_best) level_best[l] = rec[l].argmax;
   }
   g->stats[0] = passes_used;
   std::memcpy(T_out, c[(size_t)levels].data(), 6 * sizeof(double));
@@ -1233,14 +1212,14 @@ align_status align_destroy_grid(align_grid* g) {
   if (!g) return ALIGN_OK;
   cudaSetDevice(g->device);
   cudaStreamSynchronize(g->stream);
-  for (DevBuf* b : {&g->symA, &g->sat, &g->xyz, &g->poses, &g->out_c, &g->out_box, &g->mi, &g->hist, &g->best,
-                    &g->argmax, &g->err, &g->max_passes, &g->wide_count, &g->wide, &g->dump, &g->pts4,
-                    &g->pose_src, &g->rots, &g->redo_list, &g->redo_count, &g->items, &g->ovf, &g->lat_c,
+  for (DevBuf* b : {&g->symA, &g->sat, &g->xyz, &g->poses, &g->out_c, &g->out_box, &g->mi, &g->hist, &g->head,
+                    &g->wide, &g->dump, &g->pts4,
+                    &g->pose_src, &g->rots, &g->redo_list, &g->redo_count, &g->ovf, &g->lat_c,
                     &g->lat_cand, &g->ref_pts, &g->ref_pose, &g->ref_cnt, &g->ref_s1, &g->ref_s2, &g->ref_box,
                     &g->units, &g->lat_units, &g->spill, &g->lattice_ws, &g->lattice_order, &g->scatter_sums,
                     &g->scatter_list, &g->scatter_n})
     b->release();
-  for (HostBuf* b : {&g->lat_cand_h, &g->lat_rec_h, &g->lat_c_h, &g->ref_box_h}) b->release();
+  for (HostBuf* b : {&g->head_h, &g->hist_h, &g->lat_cand_h, &g->lat_rec_h, &g->lat_c_h, &g->ref_box_h}) b->release();
   for (cudaEvent_t e : g->lat_ev) cudaEventDestroy(e);
   for (auto* v : {&g->ev_pending, &g->ev_pool})
     for (auto& evs : *v)
@@ -1269,7 +1248,7 @@ align_status align_set_reference(align_grid* g, const float* xyzA, int64_t nA, i
   if (nA < 0 || nA >= INT32_MAX) return fail(ALIGN_E_INVALID, "nA out of range");
   if (nA > 0 && !xyzA) return fail(ALIGN_E_INVALID, "xyzA is NULL");
   g->has_ref = false;
-  st = ensure_status_words(g);
+  st = ensure_head(g);
   if (st != ALIGN_OK) return st;
   const GridConst& gc = g->gc;
   const size_t V = (size_t)g->V;
@@ -1382,14 +1361,12 @@ static align_status eval_common(align_grid* g, const float* xyzB, int64_t nB, in
     if (argmax_out) {
       o.argmax = argmax_out;
     } else {
-      CU(g->argmax.ensure(8), "allocate argmax");
-      o.argmax = g->argmax.as<int64_t>();
+      o.argmax = &g->dev_head()->argmax;
     }
   } else {
-    CU(g->mi.ensure((size_t)P * 4), "allocate MI");
-    CU(g->argmax.ensure(8), "allocate argmax");
-    o.mi = g->mi.as<float>();
-    o.argmax = g->argmax.as<int64_t>();
+    if (P > kHeadPoses) CU(g->mi.ensure((size_t)P * 4), "allocate MI");
+    o.mi = P > kHeadPoses ? g->mi.as<float>() : reinterpret_cast<float*>(g->dev_head() + 1);
+    o.argmax = &g->dev_head()->argmax;
     if (hist_out) {
       CU(g->hist.ensure((size_t)P * KK * 4), "allocate histograms");
       o.hist = g->hist.as<uint32_t>();
@@ -1399,10 +1376,20 @@ static align_status eval_common(align_grid* g, const float* xyzB, int64_t nB, in
   align_status st = enqueue_eval(g, n_tiles, d_poses, h_poses, P, o);
   if (st != ALIGN_OK) return st;
   if (out_dev) return ALIGN_OK;
-  if (mi_out) CU(cudaMemcpyAsync(mi_out, o.mi, (size_t)P * 4, cudaMemcpyDeviceToHost, g->stream), "read MI");
-  if (argmax_out) CU(cudaMemcpyAsync(argmax_out, o.argmax, 8, cudaMemcpyDeviceToHost, g->stream), "read argmax");
+  // small results through page-locked memory, all read by one synchronisation; a pageable copy waits
+  const size_t hist_bytes = hist_out ? (size_t)P * KK * 4 : 0;
+  const bool head_mi = P <= kHeadPoses, stage_hist = hist_bytes > 0 && hist_bytes <= kHistStage;
+  if (mi_out && !head_mi)
+    CU(cudaMemcpyAsync(mi_out, o.mi, (size_t)P * 4, cudaMemcpyDeviceToHost, g->stream), "read MI");
+  if (stage_hist) CU(g->hist_h.ensure(hist_bytes), "allocate pinned histograms");
   if (hist_out)
-    CU(cudaMemcpyAsync(hist_out, o.hist, (size_t)P * KK * 4, cudaMemcpyDeviceToHost, g->stream), "read histograms");
+    CU(cudaMemcpyAsync(stage_hist ? g->hist_h.p : hist_out, o.hist, hist_bytes, cudaMemcpyDeviceToHost, g->stream),
+       "read histograms");
+  st = read_head(g, head_mi ? P : 0);
+  if (st != ALIGN_OK) return st;
+  if (mi_out && head_mi) std::memcpy(mi_out, g->head_h.as<GridHead>() + 1, (size_t)P * 4);
+  if (argmax_out) *argmax_out = g->head_h.as<GridHead>()->argmax;
+  if (stage_hist) std::memcpy(hist_out, g->hist_h.p, hist_bytes);
   return collect_status(g);
 }
 
@@ -1428,7 +1415,7 @@ align_status align_eval_mi(align_grid* g, const float* xyzB, int64_t nB, int fla
     }
     return ALIGN_OK;
   }
-  st = ensure_status_words(g);
+  st = ensure_head(g);
   if (st != ALIGN_OK) return st;
   return eval_common(g, xyzB, nB, flags, poses12, eta6, P, mi_out, argmax_out, hist_out, nullptr, false, 0);
 }
@@ -1439,7 +1426,7 @@ align_status align_accumulate(align_grid* g, const float* xyzB, int64_t nB, int 
   if (st != ALIGN_OK) return st;
   if (!g->has_ref) return fail(ALIGN_E_NOREF, "no reference scan set");
   if (!pose12) return fail(ALIGN_E_INVALID, "pose12 is NULL");
-  st = ensure_status_words(g);
+  st = ensure_head(g);
   if (st != ALIGN_OK) return st;
   const size_t bytes = (size_t)g->V * 3 * sizeof(int64_t);
   CU(g->dump.ensure(bytes), "allocate sums");
@@ -1468,7 +1455,7 @@ align_status align_search_ex(align_grid* g, const float* xyzB, int64_t nB, int f
     P *= counts[a];
     if (P >= (1 << 26)) return fail(ALIGN_E_INVALID, "lattice too large");
   }
-  st = ensure_status_words(g);
+  st = ensure_head(g);
   if (st != ALIGN_OK) return st;
   int32_t n_tiles = 0;
   st = upload_points(g, xyzB, nB, flags, &n_tiles);
@@ -1492,9 +1479,10 @@ align_status align_search_ex(align_grid* g, const float* xyzB, int64_t nB, int f
     st = eval_common(g, xyzB, nB, ALIGN_OUT_DEVICE, poses.data(), nullptr, P, g->mi.as<float>(), nullptr,
                      nullptr, nullptr, true, n_tiles);
     if (st != ALIGN_OK) return st;
-    CU(cudaMemcpyAsync(&am, g->argmax.p, 8, cudaMemcpyDeviceToHost, g->stream), "read argmax");
-    st = collect_status(g);
+    st = read_head(g, 0);
+    if (st == ALIGN_OK) st = collect_status(g);
     if (st != ALIGN_OK) return st;
+    am = g->head_h.as<GridHead>()->argmax;
     if (am < 0 || am >= P) return fail(ALIGN_E_INTERNAL, "argmax out of range");
     CU(cudaMemcpy(&best_mi, g->mi.as<float>() + am, 4, cudaMemcpyDeviceToHost), "read MI");
     if (level_best) level_best[l] = am;
@@ -1571,7 +1559,7 @@ align_status align_refine_nm(align_grid* g, const float* xyzB, int64_t nB, int f
   for (int a = 0; a < 6; ++a)
     if (!std::isfinite(step[a])) return fail(ALIGN_E_INVALID, "step not finite");
   if (S == 0) return ALIGN_OK;
-  st = ensure_status_words(g);
+  st = ensure_head(g);
   if (st != ALIGN_OK) return st;
   int32_t n_tiles = 0;
   st = upload_points(g, xyzB, nB, flags, &n_tiles);
