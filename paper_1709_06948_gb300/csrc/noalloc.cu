@@ -160,7 +160,7 @@ extern "C" align_status align_reference_noalloc(const align_grid_desc* desc, con
   if (e != cudaSuccess) return report_cuda_error(e, "launch clear");
   e = launch_ref_accumulate(gc, xyzA, nA, pose_dev, cnt, s1, s2, s);
   if (e != cudaSuccess) return report_cuda_error(e, "launch accumulate");
-  e = launch_ref_symbols(gc, cnt, s1, s2, symA, boxA, s);
+  e = launch_ref_symbols(gc, cnt, s1, s2, symA, boxA, nullptr, s);
   if (e != cudaSuccess) return report_cuda_error(e, "launch symbols");
   return ALIGN_OK;
 }

@@ -1215,7 +1215,8 @@ align_status align_destroy_grid(align_grid* g) {
   for (DevBuf* b : {&g->symA, &g->sat, &g->xyz, &g->poses, &g->out_c, &g->out_box, &g->mi, &g->hist, &g->head,
                     &g->wide, &g->dump, &g->pts4,
                     &g->pose_src, &g->rots, &g->redo_list, &g->redo_count, &g->ovf, &g->lat_c,
-                    &g->lat_cand, &g->ref_pts, &g->ref_pose, &g->ref_cnt, &g->ref_s1, &g->ref_s2, &g->ref_box,
+                    &g->lat_cand, &g->ref_pts, &g->ref_pose, &g->ref_cnt, &g->ref_s1, &g->ref_s2, &g->ref_box, &g->ref_rows,
+                    &g->ref_list,
                     &g->units, &g->lat_units, &g->spill, &g->lattice_ws, &g->lattice_order, &g->scatter_sums,
                     &g->scatter_list, &g->scatter_n})
     b->release();
@@ -1277,12 +1278,23 @@ align_status align_set_reference(align_grid* g, const float* xyzA, int64_t nA, i
       TRY(cudaStreamSynchronize(g->stream), "synchronize");
       g->ref_pose_set = true;
     }
-    TRY(cnt.ensure(V * 4), "allocate A counts");
-    TRY(s1.ensure(V * 8), "allocate A sums");
-    TRY(s2.ensure(V * 8), "allocate A sums");
-    TRY(cudaMemsetAsync(cnt.p, 0, V * 4, g->stream), "clear");
-    TRY(cudaMemsetAsync(s1.p, 0, V * 8, g->stream), "clear");
-    TRY(cudaMemsetAsync(s2.p, 0, V * 8, g->stream), "clear");
+    if (!g->ref_clean) {
+      TRY(cnt.ensure(V * 4), "allocate A counts");
+      TRY(s1.ensure(V * 8), "allocate A sums");
+      TRY(s2.ensure(V * 8), "allocate A sums");
+      TRY(cudaMemsetAsync(cnt.p, 0, V * 4, g->stream), "clear");
+      TRY(cudaMemsetAsync(s1.p, 0, V * 8, g->stream), "clear");
+      TRY(cudaMemsetAsync(s2.p, 0, V * 8, g->stream), "clear");
+    }
+    g->ref_clean = false;
+    // prefix sums from the list of occupied voxels (at most one per point)
+    const bool by_list = ref_sat_by_list(gc);
+    const size_t n_rows = (size_t)(gc.K - 1) * gc.Y + 1;
+    if (by_list) {
+      TRY(g->ref_rows.ensure(n_rows * 4), "allocate A rows");
+      TRY(g->ref_list.ensure(std::max<size_t>(1, std::min<size_t>(V, (size_t)nA)) * 4), "allocate A list");
+      TRY(cudaMemsetAsync(g->ref_rows.p, 0, n_rows * 4, g->stream), "clear");
+    }
     TRY(launch_ref_accumulate(gc, pts.as<float>(), nA, pose.as<float>(), cnt.as<uint32_t>(),
                               s1.as<unsigned long long>(), s2.as<unsigned long long>(), g->stream),
         "launch reference accumulate");
@@ -1293,12 +1305,20 @@ align_status align_set_reference(align_grid* g, const float* xyzA, int64_t nA, i
     for (int i = 0; i < 6; ++i) box_h[i] = i < 3 ? INT_MAX : INT_MIN;
     TRY(cudaMemcpyAsync(box.p, box_h, sizeof(int32_t) * 6, cudaMemcpyHostToDevice, g->stream), "init box");
     TRY(launch_ref_symbols(gc, cnt.as<uint32_t>(), s1.as<unsigned long long>(), s2.as<unsigned long long>(),
-                           g->symA.as<uint8_t>(), box.as<int32_t>(), g->stream),
+                           g->symA.as<uint8_t>(), box.as<int32_t>(), by_list ? g->ref_rows.as<uint32_t>() : nullptr,
+                           g->stream),
         "launch reference symbols");
+    g->ref_clean = true;
     const size_t sat_elems = (size_t)(gc.K - 1) * (gc.Z + 1) * (gc.Y + 1) * (gc.X + 1);
     TRY(g->sat.ensure(std::max<size_t>(1, sat_elems) * 4), "allocate prefix sums");
-    TRY(cudaMemsetAsync(g->sat.p, 0, std::max<size_t>(1, sat_elems) * 4, g->stream), "clear prefix sums");
-    TRY(launch_ref_sat(gc, g->symA.as<uint8_t>(), g->sat.as<int32_t>(), g->stream), "launch prefix sums");
+    if (by_list) {
+      TRY(launch_ref_sat_list(gc, g->symA.as<uint8_t>(), g->ref_rows.as<uint32_t>(), g->ref_list.as<uint32_t>(),
+                              g->sat.as<int32_t>(), g->n_sm, g->stream),
+          "launch prefix sums");
+    } else {
+      TRY(cudaMemsetAsync(g->sat.p, 0, std::max<size_t>(1, sat_elems) * 4, g->stream), "clear prefix sums");
+      TRY(launch_ref_sat(gc, g->symA.as<uint8_t>(), g->sat.as<int32_t>(), g->stream), "launch prefix sums");
+    }
     int32_t* hb = box_h + 6;
     TRY(cudaMemcpyAsync(hb, box.p, sizeof(int32_t) * 6, cudaMemcpyDeviceToHost, g->stream), "read box");
     TRY(cudaStreamSynchronize(g->stream), "synchronize");

@@ -141,7 +141,8 @@ struct align_grid {
   // device-built lattice levels (align_search_ex): centres, rotation tables, read-backs
   mialign::DevBuf lat_c, lat_cand;
   // reference-build working buffers (align_set_reference)
-  mialign::DevBuf ref_pts, ref_pose, ref_cnt, ref_s1, ref_s2, ref_box;
+  mialign::DevBuf ref_pts, ref_pose, ref_cnt, ref_s1, ref_s2, ref_box, ref_rows, ref_list;
+  bool ref_clean = false;  // ref_cnt, ref_s1, ref_s2 hold zeros (the symbols kernel clears what it read)
   mialign::HostBuf ref_box_h;
   bool ref_pose_set = false;
   mialign::HostBuf lat_cand_h, lat_rec_h, lat_c_h;

@@ -1,0 +1,37 @@
+"""A's prefix sums from the list of its occupied voxels: the marginals of A over any overlap box, at the
+edges of the strips and warps they are written in."""
+import numpy as np
+import pytest
+
+import oracle
+import scangen
+from tests.helpers import lib_grid, mi_tolerance, oracle_grid
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dims,res", [((1, 1, 1), 4.0), ((31, 63, 5), 0.7), ((32, 64, 8), 0.7), ((33, 65, 7), 0.7),
+                                      ((160, 66, 3), 0.1), ((161, 66, 3), 0.1), ((416, 130, 3), 0.1), ((417, 130, 3), 0.1), ((2048, 9, 4), 0.02), ((2049, 9, 4), 0.02), ((5, 300, 40), 0.2)])
+@pytest.mark.parametrize("feature", [0, 1, 2])
+def test_reference_symbols_and_marginals(dims, res, feature):
+    """Histograms (their phi column and A's row sums come from the prefix sums) against the oracle, for
+    two references in turn on one grid (the second finds the sums cleared) and an empty one."""
+    from paper_1709_06948_gb300 import align
+    rng = np.random.default_rng(sum(dims) + feature)
+    size = np.array(dims) * res
+    spec = scangen.GridSpec(origin=tuple(-size / 2), res_m=res, dims=dims, feature=feature, count_levels=7,
+                            var_levels=8 if feature == 2 else 15)
+    L, G = lib_grid(spec), oracle_grid(spec)
+    etas = rng.uniform(-0.3, 0.3, (12, 6)) * np.concatenate([size, np.full(3, 0.2)])
+    poses = align.align_round_poses(spec.origin, etas)
+    B = (rng.uniform(-0.5, 0.5, (3000, 3)) * size).astype(np.float32)
+    for n in (4000, 700, 0):
+        A = (rng.uniform(-0.55, 0.55, (n, 3)) ** 3 * 4 * size).astype(np.float32)
+        align.align_set_reference(L, A)
+        symA, boxA = G.reference(A)
+        sym, box = align.align_get_reference(L)
+        assert np.array_equal(sym, symA) and np.array_equal(box, boxA)
+        mi, _, hist = align.align_eval_mi(L, B, eta6=etas, with_hist=True)
+        mo, ho, _ = G.eval_mi(symA, boxA, B, poses, nthreads=oracle.host_cores(), with_hist=True)
+        assert np.array_equal(hist, ho) and np.max(np.abs(mi.astype(np.float64) - mo)) <= mi_tolerance()
+    L.close()
