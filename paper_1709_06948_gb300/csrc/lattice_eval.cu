@@ -58,9 +58,22 @@ __device__ __forceinline__ float ordered_float(int32_t o) {
 }
 constexpr int32_t kOrderedMax = 0x7F7FFFFF;  // FLT_MAX
 
-// The smallest float u with k(u) >= k.
+// Inverse of ordered_float.
+__device__ __forceinline__ int32_t float_order(float f) {
+  const int32_t b = __float_as_int(f);
+  return b >= 0 ? b : (int32_t)(0x80000000u - (uint32_t)b);
+}
+// The smallest float u with k(u) >= k: searched around k res - t, whose rounding errors (of u, u + t
+// and the product) are some spacings of the larger of u and t wide, else among all floats.
 __device__ float axis_threshold(int k, float t, float inv_res, int D) {
   int32_t lo = -kOrderedMax, hi = kOrderedMax;  // k(hi) >= k: the largest float is past the grid
+  const float at = __fsub_rn(__fdiv_rn((float)k, inv_res), t);
+  const float wide = fmaxf(fabsf(at), fabsf(t)) * 4e-6f + 1e-30f;
+  const float a = at - wide, b = at + wide;
+  if (isfinite(a) && isfinite(b) && axis_k(a, t, inv_res, D) < k && axis_k(b, t, inv_res, D) >= k) {
+    lo = float_order(a) + 1;
+    hi = float_order(b);
+  }
   while (lo < hi) {
     const int32_t mid = (int32_t)(((int64_t)lo + hi) >> 1);
     if (axis_k(ordered_float(mid), t, inv_res, D) >= k) hi = mid;
@@ -75,9 +88,10 @@ __device__ __forceinline__ const float* pose_row(const LatticeArgs& a, int r, in
 
 // Cell of u among the m translations t.
 __device__ __forceinline__ uint32_t axis_cell(float u, const float* t, int m, float inv_res, int D) {
-  uint32_t s = 0u;
-  for (int i = 0; i < m; ++i) s += (uint32_t)(axis_k(u, t[i], inv_res, D) + 1);
-  return s;
+  int s = m;
+#pragma unroll 8
+  for (int i = 0; i < m; ++i) s += axis_k(u, t[i], inv_res, D);
+  return (uint32_t)s;
 }
 
 __global__ void __launch_bounds__(256) setup_kernel(const __grid_constant__ LatticeArgs a) {
@@ -280,7 +294,7 @@ __host__ __device__ constexpr int hist_words(int K) { return (K * K + 1) / 2 / 3
 __host__ __device__ constexpr int row_batch(int threads) { return threads < 512 ? threads : 512; }
 struct EvalMem {
   uint32_t hist;     // byte offsets
-  uint32_t row_of, by, cell_u, since, bx, rows, ring, arena, arena_bytes;
+  uint32_t row_of, by, cell_u, since, bx, rows, ends, ring, arena, arena_bytes;
 };
 template <int kNT>
 __host__ __device__ inline EvalMem eval_mem(int K, int gx, int X, int Y, int nsy, int nsx, uint32_t total) {
@@ -298,6 +312,7 @@ __host__ __device__ inline EvalMem eval_mem(int K, int gx, int X, int Y, int nsy
   m.since = take((uint32_t)nsx * 4u);
   m.bx = take((uint32_t)gx * (uint32_t)(X + 1) * 2u);
   m.rows = take((uint32_t)row_batch(kNT) * (2u + 4u + 4u));
+  m.ends = take((uint32_t)row_batch(kNT) * 8u);
   m.ring = take((uint32_t)(kNT / 32) * kRing * 2u);
   m.arena = off;
   m.arena_bytes = total > off ? (total - off) & ~15u : 0u;
@@ -336,6 +351,10 @@ __device__ __forceinline__ uint2 load_element_cell(const uint4* p) {
   return v;
 }
 
+__device__ __forceinline__ void copy_async4(uint32_t to, const uint32_t* from) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to), "l"(from) : "memory");
+}
+
 // Number of thresholds reached (a prefix of the ascending list), by descending powers of two.
 __device__ __forceinline__ uint32_t count_level32(const uint32_t* ct, int top, uint32_t n) {
   uint32_t pos = 0u;
@@ -364,6 +383,8 @@ __global__ void __launch_bounds__(kNT, 1024 / kNT) lattice_eval_kernel(const __g
   uint32_t* row_key = reinterpret_cast<uint32_t*>(sm + mem.rows);
   uint32_t* row_kk = row_key + kRowBatch;
   uint16_t* row_local = reinterpret_cast<uint16_t*>(row_kk + kRowBatch);
+  const uint32_t* ends = reinterpret_cast<const uint32_t*>(sm + mem.ends);
+  const uint32_t ends_at = (uint32_t)__cvta_generic_to_shared(sm + mem.ends);
   uint32_t* bits = reinterpret_cast<uint32_t*>(sm + mem.arena);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint32_t lane_lt;
@@ -466,15 +487,15 @@ __global__ void __launch_bounds__(kNT, 1024 / kNT) lattice_eval_kernel(const __g
       if (part == 0u) row = 0;
       if (part == n_split - 1u) row_end = n_rows;
     }
-    // first elements of the next rows, one row per thread (loaded before the plan needs them)
-    uint32_t next_o0 = 0u, next_o1 = 0u;
+    // First and last elements of the next rows, one row per thread: copied to shared memory while the
+    // chunk before is evaluated (held in registers they are spilled, and the spill waits for them).
     auto fetch_rows = [&]() {
       const int lin = row + tid;
       if (tid < kRowBatch && lin < row_end) {
         const int kz = lin / Y, ky = lin - kz * Y;
         const uint32_t* o = off + (size_t)kz * a.nsy;
-        next_o0 = __ldg(o + by[ky]);
-        next_o1 = __ldg(o + by[ky + 1]);
+        copy_async4(ends_at + 8u * tid, o + by[ky]);
+        copy_async4(ends_at + 8u * tid + 4u, o + by[ky + 1]);
       }
     };
     fetch_rows();
@@ -501,10 +522,13 @@ __global__ void __launch_bounds__(kNT, 1024 / kNT) lattice_eval_kernel(const __g
       // ---- plan: as many of the next rows as fit the arena ----
       // cells of a row: at most its elements; `share` (of 256) of that bound as the last chunks had it
       uint32_t flag = 0u, cells = 0u;
-      const uint32_t o0 = next_o0, o1 = next_o1;
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      uint32_t o0 = 0u, o1 = 0u;
       const int lin = row + tid;
       const int n_here = min(kRowBatch, row_end - row);
       if (tid < n_here) {
+        o0 = ends[2 * tid];
+        o1 = ends[2 * tid + 1];
         flag = o1 > o0 ? 1u : 0u;
         cells = min(o1 - o0, sx_end);
       }
@@ -606,13 +630,14 @@ __global__ void __launch_bounds__(kNT, 1024 / kNT) lattice_eval_kernel(const __g
       // more cells than planned: the rows again, by their bound
       if (M > 8190u || 24u * n_words4 + 8u + 16u * (M + 1u) > mem.arena_bytes) {
         if (share == 256u) break;  // never: the bound holds
-        share = 256u;
+        share = min(256u, max(share + 1u, (M * 280u) / bound + 8u));  // as these rows have it
         row = row0;
         fetch_rows();
         __syncthreads();
         continue;
       }
-      share = min(256u, (M * 300u) / bound + 8u);
+      // (rows of one layer differ: falling slowly saves planning them twice)
+      share = max(min(256u, (M * 290u) / bound + 8u), share - share / 8u);
       auto store = [&](uint32_t i, uint32_t k) {
         const uint32_t p1 = s_w + (k & 0xFFu), p2 = p1 + ((k >> 8) & 0xFFu), p3 = p2 + ((k >> 16) & 0xFFu);
         reinterpret_cast<uint2*>(place)[i] = make_uint2(s_w | p1 << 16, p2 | p3 << 16);
