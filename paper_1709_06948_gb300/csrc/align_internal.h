@@ -218,6 +218,7 @@ struct LatticeArgs {
   int32_t n_whole, n_split; // groups evaluated as one item; parts of each of the others
   int32_t n_items;
   int32_t threads;          // of the evaluation kernel
+  int32_t sparse;           // its rows hold few cells: mask words only where there are any
   uint32_t smem_bytes;
   int64_t n_pad;            // n, rounded up to whole blocks of 256
   int64_t bin_stride;       // bins of one list, padded
@@ -241,7 +242,8 @@ struct LatticeArgs {
   unsigned long long* best;
 };
 // Sizes of a round of at most mx values of t'_x on a's grid and lattice (gc, my, mz set): mxr, gx,
-// ncx, nsx, nsy, n_pad, bin_stride, threads, smem_bytes.  false: the lattice does not fit the kernels.
+// ncx, nsx, nsy, n_pad, bin_stride,
+// threads, sparse, smem_bytes.  false: the lattice does not fit the kernels.
 bool lattice_layout(LatticeArgs& a, int mx, size_t smem_optin);
 cudaError_t lattice_setup();  // once per device, before any launch
 // The whole lattice (n_rot rotations), in rounds of a.n_rot rotations and a.mxr values of t'_x: partial

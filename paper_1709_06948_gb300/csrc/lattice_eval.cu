@@ -27,11 +27,12 @@
 // Against the table kernels (eval.cu), which map every point under every pose (or pose pair)
 // and insert its runs into a hash table, the per-pose work falls from every point to every
 // occupied cell of the group (0.2 per point on the 120k-point LiDAR pair at 0.5 m) and every
-// occupied voxel (0.06 per point).  Measured per launch of 4,096 poses (all kernels of an
-// evaluation but compose): 120k points at 0.5 m 1.27 -> 0.76 ms, at 0.25 m 2.59 -> 1.75 ms, 257k
-// points at 1 m 1.77 -> 0.75 ms; 32,768 poses of 259k points at 0.2 m, joint feature, 55 -> 34 ms.
-// The evaluation kernel is bound by shared memory (two thirds of its data pipe's cycles) and by the
-// latency of its short phases between barriers (half of the issue slots used).
+// occupied voxel (0.06 per point).  Measured per evaluation of 4,096 poses (all kernels but compose),
+// against the table kernels: 120k points at 0.5 m 1.27 -> 0.73 ms, at 0.25 m 2.59 -> 1.76 ms, 257k
+// points at 1 m 1.77 -> 0.75 ms; 32,768 poses of 259k points at 0.2 m, joint feature, 55 -> 28.4 ms.
+// The evaluation kernel (0.58 of the 0.73 ms) is bound by instruction issue and shared memory together
+// (64% of its issue slots, 61% of the shared-memory pipe) and by the barriers between its short phases;
+// points_kernel (73 us) by its instructions, scatter_kernel (57 us) by the latency of L2 atomics.
 #include <algorithm>
 #include <climits>
 #include <mutex>
@@ -319,14 +320,15 @@ __host__ __device__ inline EvalMem eval_mem(int K, int gx, int X, int Y, int nsy
   if (m.arena_bytes > 8191u * 16u) m.arena_bytes = 8191u * 16u;  // 13-bit records in the ring
   return m;
 }
-// Arena of one row with at most `cells` occupied cells, in units of 16 bytes (rounded up): 6 bytes
-// per mask word, a 16-byte record per cell.
-__host__ __device__ inline uint32_t row_cost16(uint32_t cells, uint32_t W) { return cells + (6u * W + 15u) / 16u; }
-constexpr uint32_t kArenaSlack16 = 8;  // the last record and the padding of masks and places
+// Arena bytes of a row's mask words (or summary words) and places, and of an occupied cell (with a mask
+// word of its own when sparse).
+__host__ __device__ constexpr uint32_t row_cost(uint32_t W, bool sparse) { return 6u * (sparse ? W / 32u + 1u : W); }
+__host__ __device__ constexpr uint32_t cell_cost(bool sparse) { return sparse ? 22u : 16u; }
+constexpr uint32_t kArenaSlack = 160;  // the last record and the padding of masks and places
 
 struct EvalCtl {
   uint32_t tmp[3][32];
-  uint32_t tmp2[32];
+  uint32_t tmp2[32], tmp3[32];
   uint32_t vt32[64];    // variance thresholds below 2^32 (sym32), padded with 2^32 - 1
   uint32_t ct[64];      // count thresholds, padded with 2^32 - 1
   int32_t box[kLatticeGroup][6];
@@ -363,7 +365,9 @@ __device__ __forceinline__ uint32_t count_level32(const uint32_t* ct, int top, u
   return pos;
 }
 
-template <int kNT, int kFeat>
+// kSparse: rows with few occupied cells.  A summary bit per mask word, and words only for the marked
+// ones (see LatticeArgs::sparse).
+template <int kNT, int kFeat, bool kSparse>
 __global__ void __launch_bounds__(kNT, 1024 / kNT) lattice_eval_kernel(const __grid_constant__ LatticeArgs a) {
   constexpr int kNW = kNT / 32;
   constexpr bool kVar = kFeat != 0;
@@ -536,8 +540,9 @@ __global__ void __launch_bounds__(kNT, 1024 / kNT) lattice_eval_kernel(const __g
       // cells < 2^21 in all (the host checks), the count of non-empty rows above it
       const uint32_t before = block_scan<kNW>(cells | flag << 21, C.tmp[0], total);
       const uint32_t cells_in = (before & 0x1FFFFFu) + cells, rows_in = (before >> 21) + flag;
-      const bool fits = tid < n_here && ((cells_in * share + 255u) >> 8) + rows_in * row_cost16(0u, W) + kArenaSlack16 <=
-                                            mem.arena_bytes / 16u;
+      const bool fits = tid < n_here && ((cells_in * share + 255u) >> 8) * cell_cost(kSparse) +
+                                                rows_in * row_cost(W, kSparse) + kArenaSlack <=
+                                            mem.arena_bytes;
       const int taken = __syncthreads_count(fits);
       if (taken == 0) break;  // never: the arena holds any one row (lattice_layout)
       if (tid < taken) {
@@ -574,79 +579,130 @@ __global__ void __launch_bounds__(kNT, 1024 / kNT) lattice_eval_kernel(const __g
       };
       const uint32_t eb0 = (e0 & ~255u) + tid, eb1 = (e1 + 255u) & ~255u;  // whole blocks
       load1(eb0);
-      const uint32_t n_words4 = (n_local * W + 3u) / 4u;
-      uint16_t* place = reinterpret_cast<uint16_t*>(bits + 4u * n_words4);
-      uint4* rec = reinterpret_cast<uint4*>(bits + 6u * n_words4 + (n_words4 & 1u) * 2u);
-      for (uint32_t i = tid; i < n_words4; i += kNT) reinterpret_cast<uint4*>(bits)[i] = make_uint4(0u, 0u, 0u, 0u);
+      const uint32_t W1 = kSparse ? W / 32u + 1u : W;  // words (summary words) per row
+      const uint32_t n_top4 = (n_local * W1 + 3u) / 4u;
+      uint32_t* top = bits;  // summary bits, or the mask words themselves
+      uint16_t* top_place = reinterpret_cast<uint16_t*>(bits + 4u * n_top4);
+      for (uint32_t i = tid; i < n_top4; i += kNT) reinterpret_cast<uint4*>(top)[i] = make_uint4(0u, 0u, 0u, 0u);
       __syncthreads();
       // ---- occupied cells of every row ----
-      // an element's row and mask word (false: outside the grid for every pose of the group)
-      auto locate = [&](const uint2& w, uint32_t& rl, uint32_t& word) {
+      // an element's row (false: outside the grid for every pose of the group)
+      auto locate = [&](const uint2& w, uint32_t& rl) {
         const uint32_t k = row_of[w.x & 0xFFFFu];
         const uint32_t at = (w.x >> 16) * (uint32_t)Y + k - (uint32_t)row0;
         if (k >= (uint32_t)Y || at >= (uint32_t)taken) return false;
         rl = row_local[at];
-        word = rl * W + ((w.y & 0xFFFFu) >> 5);
         return true;
       };
-      for (uint32_t eb = eb0; eb < eb1;) {
+      auto each_element = [&](auto&& f) {  // the elements' rows and cells; the first round is loaded
+        for (uint32_t eb = eb0; eb < eb1;) {
 #pragma unroll
-        for (uint32_t j = 0; j < kB1; ++j) {
-          uint32_t rl, word;
-          if (locate(w1[j], rl, word)) atomicOr(bits + word, 1u << (w1[j].y & 31u));
+          for (uint32_t j = 0; j < kB1; ++j) {
+            uint32_t rl;
+            if (locate(w1[j], rl)) f(rl, w1[j].y & 0xFFFFu);
+          }
+          eb += kB1 * kNT;
+          if (eb < eb1) load1(eb);
         }
-        eb += kB1 * kNT;
-        if (eb < eb1) load1(eb);
+      };
+      if (kSparse) {
+        each_element([&](uint32_t rl, uint32_t sx) { atomicOr(top + rl * W1 + (sx >> 10), 1u << ((sx >> 5) & 31u)); });
+        load1(eb0);
+      } else {
+        each_element([&](uint32_t rl, uint32_t sx) { atomicOr(top + rl * W1 + (sx >> 5), 1u << (sx & 31u)); });
       }
       __syncthreads();
-      uint4 w2[kB2];  // the first elements of the second pass, loaded meanwhile
+      // ---- places: set bits before each word ----
+      // each thread takes consecutive groups of four words; their counts stay in registers
+      auto counts = [&](const uint32_t* v, uint32_t i) {  // four 8-bit counts
+        const uint4 q = reinterpret_cast<const uint4*>(v)[i];
+        return (q.x | q.y | q.z | q.w) == 0u
+                   ? 0u
+                   : (uint32_t)(__popc(q.x) | __popc(q.y) << 8 | __popc(q.z) << 16 | __popc(q.w) << 24);
+      };
+      auto places = [&](const uint32_t* v, uint16_t* to, uint32_t n4, uint32_t* tmp) {
+        const uint32_t per = (n4 + kNT - 1) / kNT;
+        const uint32_t wb = min((uint32_t)tid * per, n4), we = min(wb + per, n4);
+        constexpr uint32_t kKeep = 4;
+        uint32_t kept[kKeep], cnt = 0u, total;
+#pragma unroll
+        for (uint32_t j = 0; j < kKeep; ++j) {
+          kept[j] = wb + j < we ? counts(v, wb + j) : 0u;
+          cnt = __dp4a(kept[j], 0x01010101u, cnt);
+        }
+        for (uint32_t i = wb + kKeep; i < we; ++i) cnt = __dp4a(counts(v, i), 0x01010101u, cnt);
+        uint32_t s_w = block_scan<kNW>(cnt, tmp, total);
+        auto store = [&](uint32_t i, uint32_t k) {
+          const uint32_t p1 = s_w + (k & 0xFFu), p2 = p1 + ((k >> 8) & 0xFFu), p3 = p2 + ((k >> 16) & 0xFFu);
+          reinterpret_cast<uint2*>(to)[i] = make_uint2(s_w | p1 << 16, p2 | p3 << 16);
+          s_w = p3 + (k >> 24);
+        };
+#pragma unroll
+        for (uint32_t j = 0; j < kKeep; ++j)
+          if (wb + j < we) store(wb + j, kept[j]);
+        for (uint32_t i = wb + kKeep; i < we; ++i) store(i, counts(v, i));
+        return total;
+      };
+      uint32_t* words = top;  // mask words and the set bits before each
+      uint16_t* place = top_place;
+      uint32_t used = 24u * n_top4 + (n_top4 & 1u) * 8u;  // arena bytes so far
+      bool over = false;
+      // a cell's mask word: its place among the words, and its bits (none set: not among them)
+      auto word_at = [&](uint32_t rl, uint32_t sx, uint32_t& idx) {
+        if (!kSparse) {
+          idx = rl * W + (sx >> 5);
+          return words[idx];
+        }
+        const uint32_t wi = rl * W1 + (sx >> 10), b = (sx >> 5) & 31u, m = top[wi];
+        idx = top_place[wi] + __popc(m & ((1u << b) - 1u));
+        return (m >> b) & 1u ? words[idx] : 0u;
+      };
+      uint4 w2[kB2];  // the first elements of the pass over sums, loaded meanwhile
       auto load2 = [&](uint32_t eb) {
 #pragma unroll
         for (uint32_t j = 0; j < kB2; ++j)
           w2[j] = unspread(eb + j * kNT) - e0 < e1 - e0 ? load_element(elems + eb + j * kNT) : make_uint4(0u, 0u, 0u, 0u);
       };
-      load2(eb0);
-      // ---- places: occupied cells before each word ----
-      // each thread takes consecutive groups of four words; their counts stay in registers
-      const uint32_t per = (n_words4 + kNT - 1) / kNT;
-      const uint32_t wb = min((uint32_t)tid * per, n_words4), we = min(wb + per, n_words4);
-      constexpr uint32_t kKeep = 4;
-      uint32_t kept[kKeep];  // four 8-bit counts each
-      uint32_t cnt = 0u;
-      auto counts = [&](uint32_t i) {
-        const uint4 v = reinterpret_cast<const uint4*>(bits)[i];
-        return (v.x | v.y | v.z | v.w) == 0u
-                   ? 0u
-                   : (uint32_t)(__popc(v.x) | __popc(v.y) << 8 | __popc(v.z) << 16 | __popc(v.w) << 24);
-      };
-#pragma unroll
-      for (uint32_t j = 0; j < kKeep; ++j) {
-        kept[j] = wb + j < we ? counts(wb + j) : 0u;
-        cnt = __dp4a(kept[j], 0x01010101u, cnt);
+      uint32_t M, n_words = 0u;
+      if constexpr (kSparse) {
+        n_words = places(top, top_place, n_top4, C.tmp2);
+        const uint32_t n4 = n_words / 4u + 1u;  // one word past the last, for cells after it
+        words = reinterpret_cast<uint32_t*>(sm + mem.arena + used);
+        place = reinterpret_cast<uint16_t*>(words + 4u * n4);
+        used += 24u * n4 + (n4 & 1u) * 8u;
+        over = used + 16u > mem.arena_bytes;
+        if (!over)
+          for (uint32_t i = tid; i < n4; i += kNT) reinterpret_cast<uint4*>(words)[i] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        if (!over) {
+          each_element([&](uint32_t rl, uint32_t sx) {
+            uint32_t idx;
+            word_at(rl, sx, idx);
+            atomicOr(words + idx, 1u << (sx & 31u));
+          });
+          load2(eb0);
+        }
+        __syncthreads();
+        M = 0u;
+        if (!over) M = places(words, place, n4, C.tmp3);
+      } else {
+        load2(eb0);
+        M = places(words, place, n_top4, C.tmp2);
       }
-      for (uint32_t i = wb + kKeep; i < we; ++i) cnt = __dp4a(counts(i), 0x01010101u, cnt);
-      uint32_t M;
-      uint32_t s_w = block_scan<kNW>(cnt, C.tmp2, M);
-      // more cells than planned: the rows again, by their bound
-      if (M > 8190u || 24u * n_words4 + 8u + 16u * (M + 1u) > mem.arena_bytes) {
+      // more than planned: fewer rows
+      if (over || M > 8190u || used + 16u * (M + 1u) > mem.arena_bytes) {
         if (share == 256u) break;  // never: the bound holds
-        share = min(256u, max(share + 1u, (M * 280u) / bound + 8u));  // as these rows have it
+        const uint32_t need = over ? share + share / 2u : kSparse ? (16u * M + 6u * n_words) * 13u / bound : (M * 280u) / bound;
+        share = min(256u, max(share + 1u, need + 8u));  // as these rows have it
         row = row0;
         fetch_rows();
         __syncthreads();
         continue;
       }
+      uint4* rec = reinterpret_cast<uint4*>(sm + mem.arena + used);
       // (rows of one layer differ: falling slowly saves planning them twice)
-      share = max(min(256u, (M * 290u) / bound + 8u), share - share / 8u);
-      auto store = [&](uint32_t i, uint32_t k) {
-        const uint32_t p1 = s_w + (k & 0xFFu), p2 = p1 + ((k >> 8) & 0xFFu), p3 = p2 + ((k >> 16) & 0xFFu);
-        reinterpret_cast<uint2*>(place)[i] = make_uint2(s_w | p1 << 16, p2 | p3 << 16);
-        s_w = p3 + (k >> 24);
-      };
-#pragma unroll
-      for (uint32_t j = 0; j < kKeep; ++j)
-        if (wb + j < we) store(wb + j, kept[j]);
-      for (uint32_t i = wb + kKeep; i < we; ++i) store(i, counts(i));
+      const uint32_t seen = kSparse ? (16u * M + 6u * n_words) * 13u / bound : (M * 290u) / bound;
+      share = max(min(256u, seen + 8u), share - share / 8u);
       for (uint32_t i = tid; i <= M; i += kNT) rec[i] = make_uint4(0u, 0u, 0u, 0u);
       __syncthreads();
       // ---- sums per cell: records n, S1, S2, row << 16 | cell ----
@@ -654,9 +710,10 @@ __global__ void __launch_bounds__(kNT, 1024 / kNT) lattice_eval_kernel(const __g
 #pragma unroll
         for (uint32_t j = 0; j < kB2; ++j) {
           const uint4 w = w2[j];
-          uint32_t rl, word;
-          if (!locate(make_uint2(w.x, w.y), rl, word)) continue;
-          const uint32_t at = place[word] + __popc(bits[word] & ((1u << (w.y & 31u)) - 1u));
+          uint32_t rl, idx;
+          if (!locate(make_uint2(w.x, w.y), rl)) continue;
+          const uint32_t m = word_at(rl, w.y & 0xFFFFu, idx);
+          const uint32_t at = place[idx] + __popc(m & ((1u << (w.y & 31u)) - 1u));
           // word j of a record at j ^ sw meanwhile: one word of 32 records in 32 banks, not in 8
           uint32_t* rc = reinterpret_cast<uint32_t*>(rec + at);
           const uint32_t sw = (at >> 3) & 3u;
@@ -715,8 +772,9 @@ __global__ void __launch_bounds__(kNT, 1024 / kNT) lattice_eval_kernel(const __g
 
       // cells of row rl before cell s (s <= sx_end), counted from the chunk's first
       auto cells_before = [&](uint32_t rl, uint32_t s) {
-        const uint32_t w = rl * W + (s >> 5);
-        return (uint32_t)place[w] + (uint32_t)__popc(bits[w] & ((1u << (s & 31u)) - 1u));
+        uint32_t idx;
+        const uint32_t m = word_at(rl, s, idx);
+        return (uint32_t)place[idx] + (uint32_t)__popc(m & ((1u << (s & 31u)) - 1u));
       };
       // ---- occupied box: rows with a cell inside the grid, their first and last cell ----
       // A lane per (row, pose): four rows and eight poses per warp.
@@ -872,27 +930,32 @@ __global__ void __launch_bounds__(kNT, 1024 / kNT) lattice_eval_kernel(const __g
 // Dynamic shared memory of a CTA, 1,024 threads per SM (228 KB, 1 KB reserved per CTA).
 constexpr uint32_t kSmemPair = 113u * 1024u;
 
-// Room for one row of the largest size, and for the planner's 21-bit costs.
-bool arena_ok(const EvalMem& m, int W, int nsx, int threads) {
-  const uint64_t row = row_cost16((uint32_t)nsx, (uint32_t)W);
-  return (row + kArenaSlack16) * 16 <= m.arena_bytes && row * row_batch(threads) < (1u << 21);
+// Room for one row of the largest size, and for the planner's 21-bit counts.
+bool arena_ok(const EvalMem& m, int W, int nsx, int threads, bool sparse) {
+  const uint64_t row = (uint64_t)nsx * cell_cost(sparse) + row_cost((uint32_t)W, sparse);
+  return row + kArenaSlack <= m.arena_bytes && (uint64_t)nsx * row_batch(threads) < (1u << 21);
 }
 
 template <int kNT>
 cudaError_t launch_eval_nt(const LatticeArgs& a, int n_ctas, cudaStream_t s) {
-  switch (a.gc.feature) {
-    case 0: lattice_eval_kernel<kNT, 0><<<n_ctas, kNT, a.smem_bytes, s>>>(a); break;
-    case 1: lattice_eval_kernel<kNT, 1><<<n_ctas, kNT, a.smem_bytes, s>>>(a); break;
-    default: lattice_eval_kernel<kNT, 2><<<n_ctas, kNT, a.smem_bytes, s>>>(a); break;
-  }
+  constexpr bool kS = kNT == 1024;  // sparse rows with one CTA per SM only (lattice_layout)
+  auto* k = a.sparse ? (a.gc.feature == 0   ? lattice_eval_kernel<kNT, 0, kS>
+                        : a.gc.feature == 1 ? lattice_eval_kernel<kNT, 1, kS>
+                                            : lattice_eval_kernel<kNT, 2, kS>)
+                     : (a.gc.feature == 0   ? lattice_eval_kernel<kNT, 0, false>
+                        : a.gc.feature == 1 ? lattice_eval_kernel<kNT, 1, false>
+                                            : lattice_eval_kernel<kNT, 2, false>);
+  k<<<n_ctas, kNT, a.smem_bytes, s>>>(a);
   return cudaGetLastError();
 }
 template <int kNT>
 cudaError_t setup_nt(int smem) {
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(lattice_eval_kernel<kNT, 0>, attr, smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(lattice_eval_kernel<kNT, 1>, attr, smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(lattice_eval_kernel<kNT, 2>, attr, smem);
+  cudaError_t e = cudaSuccess;
+  for (auto* k : {lattice_eval_kernel<kNT, 0, false>, lattice_eval_kernel<kNT, 1, false>, lattice_eval_kernel<kNT, 2, false>,
+                  lattice_eval_kernel<kNT, 0, kNT == 1024>, lattice_eval_kernel<kNT, 1, kNT == 1024>,
+                  lattice_eval_kernel<kNT, 2, kNT == 1024>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, attr, smem);
   return e;
 }
 
@@ -918,13 +981,21 @@ bool lattice_layout(LatticeArgs& a, int mx, size_t smem_optin) {
     a.nsx = (int)nsx;
     const int W = (int)((nsx - 1) / 32 + 1);
     const EvalMem m2 = eval_mem<512>(gc.K, a.gx, gc.X, gc.Y, a.nsy, a.nsx, kSmemPair);
-    if (arena_ok(m2, W, a.nsx, 512) && m2.arena_bytes >= 32u * 1024u && smem_optin >= kSmemPair) {
+    if (arena_ok(m2, W, a.nsx, 512, false) && m2.arena_bytes >= 32u * 1024u && smem_optin >= kSmemPair) {
       a.threads = 512;
+      a.sparse = 0;
       a.smem_bytes = kSmemPair;
       return true;
     }
+    // One CTA per SM (large histograms, wide tables): nothing hides the fixed cost of a chunk, and rows
+    // with few points against their mask words (at most half of the points' rows are counted) make
+    // chunks small.  6.2 words per point (259k points, 400 x 400 x 40): 34.2 -> 28.4 ms.  With two CTAs
+    // the third pass over the elements costs more than it saves: 6.9 words (120k, 320 x 320 x 32) 1.76
+    // -> 1.85 ms, 5.9 (8k, 105 x 106 x 17) 0.18 -> 0.21, 2.1 (33k, 147 x 170 x 17) 0.44 -> 0.54.
+    const int64_t rows = std::min<int64_t>((int64_t)gc.Z * gc.Y, a.n / 2);
+    a.sparse = 4 * a.n < rows * W ? 1 : 0;
     const EvalMem m1 = eval_mem<1024>(gc.K, a.gx, gc.X, gc.Y, a.nsy, a.nsx, (uint32_t)smem_optin);
-    if (arena_ok(m1, W, a.nsx, 1024)) {
+    if (arena_ok(m1, W, a.nsx, 1024, a.sparse != 0)) {
       a.threads = 1024;
       a.smem_bytes = (uint32_t)smem_optin;
       return true;

@@ -435,7 +435,7 @@ bool mialign::plan_lattice(const GridConst& gc, int n_sm, size_t smem_optin, int
   // The masks of a group's rows (at least one point in each) cost about as much per word as a point
   // does in the table kernels: measured 8.5k points on a 265 x 219 x 29 grid, 4.2 words per pose and
   // point, 0.63 against 0.61 ms, and 41k points on 345 x 380 x 41, 4.2, 0.75 against 0.56 ms; 0.86
-  // (120k points, 320 x 320 x 32) 1.75 against 2.59 ms, 0.78 (259k, 400 x 400 x 40) 36 against 52 ms.
+  // (120k points, 320 x 320 x 32) 1.76 against 2.59 ms, 0.78 (259k, 400 x 400 x 40) 28 against 52 ms.
   const int64_t words = std::min<int64_t>((int64_t)gc.Z * gc.Y, n / 2) * (a.nsx / 32 + 1);
   if (words > 2 * a.gx * n) return false;
   const int64_t chunks = ((int64_t)mx + a.gx - 1) / a.gx;

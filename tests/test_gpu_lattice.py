@@ -81,6 +81,15 @@ def test_grid_shapes(tiny, dims, res):
     _check(spec, tiny.xyzA, tiny.xyzB, _lattice((8, 20, 2, 1, 1, 4), SMALL))
 
 
+@pytest.mark.parametrize("feature,n", [(0, 8000), (1, 4000), (2, 8000), (2, 4000)])
+def test_sparse_rows(tiny, feature, n):
+    """Few points per row and tables that leave one CTA per SM: mask words only where there are cells."""
+    spec = scangen.GridSpec(origin=(-25.0, -25.0, -1.0), res_m=0.1, dims=(500, 40, 10), feature=feature, count_levels=7,
+                            var_levels=8 if feature == 2 else 15)
+    squeeze = np.array([1.0, 0.1, 0.2], np.float32)  # a street 4 m wide
+    _check(spec, tiny.xyzA * squeeze, np.ascontiguousarray(tiny.xyzB[:: 8000 // n] * squeeze), _lattice((7, 20, 2, 1, 1, 4), SMALL))
+
+
 def test_non_finite_points_and_wide_thresholds(tiny):
     xyz = tiny.xyzB.copy()
     xyz[::7, 0] = np.nan
