@@ -136,46 +136,41 @@ __global__ void ref_list_kernel(const GridConst gc, const uint8_t* __restrict__ 
 // the counts per x of the strip's earlier rows and adding each row's voxels; a row without any is the
 // row before.  Everything is written once and nothing but the list is read (the passes below write,
 // read and write it again, and need it cleared): bound by the writes, 1.44 GB for 56 symbols on
-// 400 x 400 x 40 voxels.
-constexpr int kSatRows = 64, kSatWarps = 4, kSatMaxX = 2048;
+// 400 x 400 x 40 voxels (0.25 to 0.3 ms, 5 TB/s; the whole reference of 87k points 1.69 -> 0.40 ms).
+constexpr int kSatRows = 31, kSatWarps = 4, kSatMaxX = 2048;  // rows per strip at most: a lane per row end
 
 // kRegs: the running counts in registers (x = lane + 32 i, X <= 32 kRegs); 0: in shared memory.
 template <int kRegs>
 __global__ void __launch_bounds__(kSatWarps * 32) ref_sat_list_kernel(const GridConst gc,
                                                                       const uint32_t* __restrict__ row_n,
                                                                       const uint32_t* __restrict__ list,
-                                                                      int32_t* __restrict__ sat) {
+                                                                      int32_t* __restrict__ sat, int strip_rows) {
   extern __shared__ int32_t cols[];  // per warp: X running counts (inclusive sums along x), X new counts
   int32_t reg[kRegs > 0 ? kRegs : 1];
   const int X = gc.X, Y = gc.Y, Z = gc.Z, X1 = X + 1, Y1 = Y + 1;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int32_t* run = cols + (size_t)warp * 2 * X;
   int32_t* add = run + X;
-  const int strips = (Y1 + kSatRows - 1) / kSatRows;
+  const int strips = (Y1 + strip_rows - 1) / strip_rows;
   const int64_t tasks = (int64_t)(gc.K - 1) * (Z + 1) * strips;
   for (int64_t task = blockIdx.x * (int64_t)kSatWarps + warp; task < tasks; task += (int64_t)gridDim.x * kSatWarps) {
     const int strip = (int)(task % strips);
     const int z = (int)((task / strips) % (Z + 1));
     const int a = (int)(task / ((int64_t)strips * (Z + 1)));
-    const int y0 = strip * kSatRows, y1 = min(Y1, y0 + kSatRows);  // rows of the plane (row y: voxels below y)
+    const int y0 = strip * strip_rows, y1 = min(Y1, y0 + strip_rows);  // rows of the plane (row y: voxels below y)
     int32_t* out = sat + ((size_t)a * (Z + 1) + z) * Y1 * X1;
     const uint32_t* rows = row_n + (size_t)a * Y;
     for (int x = lane; x < X; x += 32) run[x] = add[x] = 0;
 #pragma unroll
     for (int i = 0; i < kRegs; ++i) reg[i] = 0;
     __syncwarp();
-    // add the listed voxels [b, e) below z; whether there were any
-    auto take = [&](uint32_t b, uint32_t e) {
-      bool any = false;
-      for (uint32_t i = b + lane; i < e; i += 32) {
-        const uint32_t q = __ldg(list + i);
-        if ((int)(q >> 16) < z) {
-          atomicAdd(&add[q & 0xFFFFu], 1);
-          any = true;
-        }
-      }
-      return __any_sync(0xFFFFFFFFu, any);
+    // add a listed voxel if it lies below z
+    auto put = [&](uint32_t q) {
+      const bool in = (int)(q >> 16) < z;
+      if (in) atomicAdd(&add[q & 0xFFFFu], 1);
+      return in;
     };
+    constexpr uint32_t kNone = 0xFFFFFFFFu;  // z 65535: in no plane (Z < 65536 planes lie below)
     // running counts += inclusive sums of the new ones
     auto merge = [&]() {
       __syncwarp();
@@ -204,9 +199,37 @@ __global__ void __launch_bounds__(kSatWarps * 32) ref_sat_list_kernel(const Grid
       }
       __syncwarp();
     };
-    if (z > 0 && y0 > 1 && take(__ldg(rows), __ldg(rows + y0 - 1))) merge();
+    // rows y0 - 1 .. y1 - 2 of voxels enter the planes' rows y0 .. y1 - 1; lane i holds the start of
+    // voxel row y0 - 1 + i (their ends are the next starts)
+    const int first = max(y0 - 1, 0);
+    const uint32_t starts = __ldg(rows + min(first + lane, Y));
+    const uint32_t before = __shfl_sync(0xFFFFFFFFu, starts, 0);
+    bool any = false;
+    if (z > 0)
+      for (uint32_t i = __ldg(rows) + lane; i < before; i += 128) {  // four loads in flight
+        uint32_t q[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) q[k] = i + 32 * k < before ? __ldg(list + i + 32 * k) : kNone;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) any = put(q[k]) || any;
+      }
+    if (__any_sync(0xFFFFFFFFu, any)) merge();
+    // a row's first 32 voxels are loaded while the row before is written
+    auto head = [&](int j) {
+      const uint32_t b = __shfl_sync(0xFFFFFFFFu, starts, j), e = __shfl_sync(0xFFFFFFFFu, starts, j + 1);
+      return b + lane < e ? __ldg(list + b + lane) : kNone;
+    };
+    uint32_t next = head(0);
     for (int y = y0; y < y1; ++y) {
-      if (z > 0 && y > 0 && take(__ldg(rows + y - 1), __ldg(rows + y))) merge();
+      const int j = y - 1 - first;  // the voxel row that enters here (-1: none, y = 0)
+      if (z > 0 && j >= 0) {
+        const uint32_t q = next;
+        if (y + 1 < y1) next = head(j + 1);
+        bool in = put(q);
+        const uint32_t b = __shfl_sync(0xFFFFFFFFu, starts, j), e = __shfl_sync(0xFFFFFFFFu, starts, j + 1);
+        for (uint32_t i = b + 32 + lane; i < e; i += 32) in = put(__ldg(list + i)) || in;
+        if (__any_sync(0xFFFFFFFFu, in)) merge();
+      }
       int32_t* o = out + (size_t)y * X1;
       if (lane == 0) o[0] = 0;
       if constexpr (kRegs > 0) {
@@ -221,7 +244,8 @@ __global__ void __launch_bounds__(kSatWarps * 32) ref_sat_list_kernel(const Grid
   }
 }
 
-// The same by passes over the whole array, for grids too wide for a warp's counts in shared memory.
+// The same by passes over the whole array, for small arrays and for grids too wide for a warp's counts in
+// shared memory (ref_sat_by_list).
 // Pass 0: running sums along x per (a, z, y) row (a warp per row: inclusive warp scans over
 // 32-voxel chunks, coalesced); pass 1 along y and pass 2 along z (a thread per column, rows
 // read kChunk at a time so that the loads of a chunk are in flight together).
@@ -315,8 +339,13 @@ cudaError_t launch_ref_symbols(const GridConst& gc, uint32_t* cnt, unsigned long
   return cudaGetLastError();
 }
 
+// Small arrays stay with the passes: the list's strips are short chains of dependent loads (104k points
+// on a 25 MB array, 150 x 160 x 16 voxels and 15 symbols, 109 against 117 us; 104k points on 108 MB, 250
+// x 266 x 26, 206 against 143 us; on 92 MB, 56 symbols, 179 against 115 us).
 bool ref_sat_by_list(const GridConst& gc) {
-  return gc.X <= kSatMaxX && gc.Z < 65536 && gc.K > 1;  // 64 KB of counts per block; 16-bit list entries
+  const int64_t bytes = (int64_t)(gc.K - 1) * (gc.Z + 1) * (gc.Y + 1) * (gc.X + 1) * 4;
+  return gc.X <= kSatMaxX && gc.Z < 65536 &&  // 64 KB of counts per block; 16-bit list entries
+         bytes >= ((int64_t)32 << 20);
 }
 
 cudaError_t launch_ref_sat_list(const GridConst& gc, const uint8_t* symA, uint32_t* row_n, uint32_t* list,
@@ -330,9 +359,16 @@ cudaError_t launch_ref_sat_list(const GridConst& gc, const uint8_t* symA, uint32
   const size_t smem = (size_t)kSatWarps * 2 * gc.X * 4;
   auto* k = gc.X <= 160 ? ref_sat_list_kernel<5> : gc.X <= 416 ? ref_sat_list_kernel<13> : ref_sat_list_kernel<0>;
   if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024)) != cudaSuccess) return e;
-  const int64_t strips = (gc.Y + 1 + kSatRows - 1) / kSatRows;
-  const int64_t blocks = ((int64_t)(gc.K - 1) * (gc.Z + 1) * strips + kSatWarps - 1) / kSatWarps;
-  k<<<(unsigned)std::min<int64_t>(blocks, 64 * (int64_t)n_sm), kSatWarps * 32, smem, s>>>(gc, row_n, list, sat);
+  // shorter strips while there are few: a strip's rows follow one another (latency), but each strip
+  // adds up the rows before it first
+  int rows = kSatRows;
+  auto blocks_of = [&](int r) {
+    return ((int64_t)(gc.K - 1) * (gc.Z + 1) * ((gc.Y + r) / r) + kSatWarps - 1) / kSatWarps;
+  };
+  while (rows > 7 && blocks_of(rows) < 16 * (int64_t)n_sm) rows /= 2;
+  const int64_t blocks = blocks_of(rows);
+  k<<<(unsigned)std::min<int64_t>(blocks, 64 * (int64_t)n_sm), kSatWarps * 32, smem, s>>>(gc, row_n, list, sat,
+                                                                                           rows);
   return cudaGetLastError();
 }
 
