@@ -151,16 +151,16 @@ def code_digest(path):
 
 
 def committed_traffic():
-    """Per-launch DRAM bytes of the eval kernel from the committed ncu summary, if it was
-    taken on the current kernel code (else None)."""
-    path = os.path.join(ROOT, "profiles", "eval_pair_kernel_lidar120k.md")
-    src = os.path.join(ROOT, "paper_1709_06948_gb300", "csrc", "eval.cu")
+    """Per-launch DRAM bytes of the lattice evaluation kernel from the committed ncu summary,
+    if it was taken on the current kernel code (else None)."""
+    path = os.path.join(ROOT, "profiles", "lattice_eval_kernel_lidar120k.md")
+    src = os.path.join(ROOT, "paper_1709_06948_gb300", "csrc", "lattice_eval.cu")
     try:
         text = open(path).read()
         digest = code_digest(src)
     except Exception:
         return None
-    m_sha = re.search(r"eval\.cu code sha256[^:]*:\s*([0-9a-f]{64})", text)
+    m_sha = re.search(r"lattice_eval\.cu code sha256[^:]*:\s*([0-9a-f]{64})", text)
     m_b = re.search(r"traffic_bytes_per_full_launch:\s*([0-9.eE+]+)", text)
     if not m_sha or not m_b or m_sha.group(1) != digest:
         return None
@@ -616,7 +616,10 @@ def run_ours(args):
     ops_per_launch = P * nB * OPS_MAP
     achieved = ops_per_launch / (eval_ms / 1000.0) / 1e12
     achieved_am = P * nB * OPS_MAP_AMORTISED / (eval_ms / 1000.0) / 1e12
-    traffic = committed_traffic()
+    sweep = align.align_eval_stats(L)["sweep"]
+    traffic = committed_traffic() if sweep == 3 else None
+    kernel = ("lattice groups (cells and lists of points, lattice_eval_kernel, exact path)" if sweep == 3
+              else f"table kernels ({align.SWEEP_KINDS.get(sweep, sweep)})")
     if peaks is not None:
         peak = peaks["alu_lane_ops_per_s"] / 1e12
         basis = (f"measured: fastest of FP32 FFMA and INT32 add/xor issue micro-benchmarks on this GPU at "
@@ -625,21 +628,24 @@ def run_ours(args):
         peak = dev_props.multi_processor_count * 128 * 2070.0e6 / 1e12
         basis = "derived: SMs x 128 lanes x 2,070 MHz (of derived peak; micro-benchmarks skipped)"
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tops/s", "frac": achieved / peak,
-                "traffic": traffic, "kernel": "eval_pair_kernel (pose pairs; eval_kernel for single poses)",
-                "eval_kernel_ms": eval_ms,
+                "traffic": traffic, "kernel": kernel, "eval_kernel_ms": eval_ms,
                 "ops_per_launch": ops_per_launch,
-                "ops_basis": f"{OPS_MAP} lane-ops per (point, pose) x {nB} points x {P} poses",
+                "ops_basis": f"{OPS_MAP} lane-ops per (point, pose) x {nB} points x {P} poses: what a map of every "
+                             "point under every pose costs; lattice groups share it between poses, so the "
+                             "fraction counts the work asked for, not the instructions issued",
                 "achieved_amortised": achieved_am, "frac_amortised": achieved_am / peak,
                 "amortised_basis": f"{OPS_MAP_AMORTISED} lane-ops per (point, pose): the rotation shared by the "
-                                   "translations of a lattice (the kernel reads pre-rotated copies)",
+                                   "translations of a lattice",
                 "peak_basis": basis,
                 "kernel_share_of_step": (prof[0] / total_ms) if total_ms > 0 else None}
     if peaks is not None:
-        atom = P * occ * ATOMICS_PER_VOXEL / (eval_ms / 1000.0)
+        # groups: the joint histogram's atomic per voxel (their cells' sums are shared by up to 8 poses)
+        per_voxel = 1 if sweep == 3 else ATOMICS_PER_VOXEL
+        atom = P * occ * per_voxel / (eval_ms / 1000.0)
         roofline["shared_atomics"] = {
             "achieved_per_s": atom, "peak_per_s": peaks["smem_red_random_per_s"],
             "frac": atom / peaks["smem_red_random_per_s"],
-            "basis": f"{ATOMICS_PER_VOXEL} atomics per occupied voxel x {occ} occupied voxels (lattice centre) x "
+            "basis": f"{per_voxel} atomics per occupied voxel x {occ} occupied voxels (lattice centre) x "
                      f"{P} poses; peak: shared red.add on random words (measured)"}
         roofline["mix_peak"] = {"lane_ops_per_s": peaks["keymix_lane_ops_per_s"],
                                 "frac": achieved * 1e12 / peaks["keymix_lane_ops_per_s"],
