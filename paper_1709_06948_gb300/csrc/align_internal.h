@@ -109,7 +109,13 @@ struct EvalArgs {
   uint4* spill;
   int64_t spill_cap;
   int32_t spill_np;
+  // compose_kernel, one item: CTAs done (0 between launches); and, for poses of scatter_eval.cu, their
+  // list counters: each pose's histogram, box and counter are reset once read.
+  uint32_t* done;
+  uint32_t* list_n;
 };
+// Box of no voxel, as a memset can write it.
+constexpr int32_t kNoBoxLo = 0x7F7F7F7F, kNoBoxHi = (int32_t)0x80808080;
 
 // One point-tile PackCopy of a batch: scan xyz (n points) -> out (n_out float4), raw
 // (rotate == 0) or pre-rotated by R.
@@ -150,13 +156,12 @@ struct EvalKernels {
   cudaError_t (*launch_pack_points)(const float* xyz, int64_t n, int64_t n_out, const float* rots, int n_rot,
                                     float4* out, cudaStream_t s);
   cudaError_t (*launch_pack_batch)(const PackCopy* copies, int n_copies, int64_t max_out, cudaStream_t s);
-  // Overlap box, phi column, MI and the running argmax of every pose.
+  // Overlap box, phi column, MI and the running argmax of every pose; a single item's argmax.
   cudaError_t (*launch_compose)(const EvalArgs& a, cudaStream_t s);
   // The redo kernel alone, over one item whose points are read from EvalItem::xyz.
   cudaError_t (*launch_redo_raw)(const EvalArgs& a, int n_ctas, int vw, cudaStream_t s);
-  // Each item's argmax from its packed running maximum.
+  // Each item's argmax from its packed running maximum (launches of several items).
   cudaError_t (*launch_argmax_finalize)(const EvalItem* items, int n_items, cudaStream_t s);
-  cudaError_t (*launch_argmax_one)(const EvalItem& item, cudaStream_t s);  // a single item's
 };
 constexpr int kEvalShapes = 3;
 // Table value words per slot for a launch over grids with constants gc: 1 without z sums
@@ -195,6 +200,7 @@ struct LatticeLevel {
 };
 cudaError_t launch_lattice_level(const LatticeLevel& L, cudaStream_t s);
 
+constexpr size_t kLatticeBudget = (size_t)5 << 28;  // workspace of a round of a pose lattice (1.25 GiB)
 // A pose lattice evaluated group by group (lattice_eval.cu): every combination of n_rot
 // rotations and mx, my, mz values of t'_x, t'_y, t'_z, or a round of it (n_rot rotations from r0
 // on, mxr values of t'_x from ix0 on).
@@ -264,12 +270,11 @@ struct ScatterArgs {
   unsigned long long* sums;  // P x V x 2 (1 without z sums), zero between calls
   uint32_t* list;            // P x list_cap: occupied voxels
   int64_t list_cap;
-  uint32_t* list_n;          // P
+  uint32_t* list_n;          // P, zero between calls
   uint32_t* wide_count;      // voxels past the 32-bit sums
-  uint32_t* out_c;           // P x K x K, and up to 3 words of padding
-  int32_t* out_box;          // P x 6
-  uint32_t* redo_count;      // set to 0 (no pose needs the exact path)
-  unsigned long long* best;
+  uint32_t* out_c;           // P x K x K, zero between calls
+  int32_t* out_box;          // P x 6, kNoBoxLo and kNoBoxHi between calls
+  unsigned long long* best;  // reset
 };
 size_t scatter_pose_bytes(const GridConst& gc, int64_t n);  // sums and list of one pose
 cudaError_t launch_scatter(const ScatterArgs& a, int n_sm, cudaStream_t s, int32_t* launches);

@@ -687,6 +687,7 @@ align_status enqueue_eval_core(align_grid* g, int32_t n_tiles, const float* d_po
   a.n_units = pairs ? n_units : 0;
   a.cluster = cluster ? 1 : 0;
   a.err = &g->dev_head()->err;
+  a.done = &g->dev_head()->done;
   a.max_passes = &g->dev_head()->max_passes;
   a.wide_count = &g->dev_head()->wide_count;
   a.wide_poses = &g->dev_head()->wide_poses;
@@ -721,7 +722,6 @@ align_status enqueue_eval_core(align_grid* g, int32_t n_tiles, const float* d_po
   CU(ek.launch_eval(a, n_ctas, vw, rotate, g->stream), "launch eval kernel");
   if (g->profiling) CU(cudaEventRecord(evs[1], g->stream), "record event");
   CU(ek.launch_compose(a, g->stream), "launch compose kernel");
-  CU(ek.launch_argmax_one(item, g->stream), "launch argmax");
   if (g->profiling) {
     CU(cudaEventRecord(evs[2], g->stream), "record event");
     g->ev_pending.push_back(evs);
@@ -729,7 +729,7 @@ align_status enqueue_eval_core(align_grid* g, int32_t n_tiles, const float* d_po
   g->stats[2] = g->table_slots;
   g->stats[3] = n_ctas;
   g->stats[5] = pairs ? 1 : cluster ? 2 : 0;
-  g->stats[4] += 5;  // pack, eval, redo, compose, argmax
+  g->stats[4] += 4;  // pack, eval, redo, compose
   return ALIGN_OK;
 }
 
@@ -808,6 +808,7 @@ align_status enqueue_lattice(align_grid* g, LatticeArgs a, const float* d_poses,
   e.n_buckets = e.table_slots / 4;
   e.passes0 = 1;
   e.err = &g->dev_head()->err;
+  e.done = &g->dev_head()->done;
   e.max_passes = &g->dev_head()->max_passes;
   e.wide_count = &g->dev_head()->wide_count;
   e.redo_list = a.redo_list;
@@ -826,9 +827,8 @@ align_status enqueue_lattice(align_grid* g, LatticeArgs a, const float* d_poses,
   CU(ek.launch_redo_raw(e, redo_ctas, vw, g->stream), "launch redo kernel");
   if ((st = profile_event(g, evs, 1)) != ALIGN_OK) return st;
   CU(ek.launch_compose(e, g->stream), "launch compose kernel");
-  CU(ek.launch_argmax_one(item, g->stream), "launch argmax");
   if ((st = profile_event(g, evs, 2)) != ALIGN_OK) return st;
-  g->stats[4] += launches + 3;  // and redo, compose, argmax
+  g->stats[4] += launches + 2;  // and redo, compose
   g->stats[3] = g->n_sm * (1024 / a.threads);
   g->stats[5] = 3;
   g->last_lattice = true;
@@ -848,25 +848,32 @@ align_status enqueue_scatter(align_grid* g, const float* d_poses, int64_t P, con
   a.V = g->V;
   a.list_cap = std::min<int64_t>(g->V, std::max<int64_t>(a.n, 1));
   const size_t words = g->gc.feature != ALIGN_FEAT_COUNT ? 16 : 8;
-  const size_t sum_bytes = (size_t)P * (size_t)g->V * words;
-  if (g->scatter_sums.cap < sum_bytes || g->scatter_sums.p == nullptr) {
-    if (g->scatter_sums.ensure(sum_bytes) != cudaSuccess) {
+  const size_t KK = (size_t)g->gc.K * g->gc.K;
+  // the buffers that the kernels leave cleared: cleared here when they are new
+  DevBuf* const cleared[] = {&g->scatter_sums, &g->scatter_c, &g->scatter_n};
+  const size_t bytes[] = {(size_t)P * (size_t)g->V * words, (size_t)P * KK * 4, (size_t)P * 4};
+  for (int i = 0; i < 3; ++i) {
+    if (cleared[i]->p != nullptr && cleared[i]->cap >= bytes[i]) continue;
+    if (cleared[i]->ensure(bytes[i]) != cudaSuccess) {
       (void)cudaGetLastError();
       return ALIGN_OK;
     }
-    CU(cudaMemsetAsync(g->scatter_sums.p, 0, g->scatter_sums.cap, g->stream), "clear sums");
+    CU(cudaMemsetAsync(cleared[i]->p, 0, cleared[i]->cap, g->stream), "clear sums");
+  }
+  if (g->scatter_box.p == nullptr) {  // 3 words of kNoBoxLo, 3 of kNoBoxHi per pose
+    uint8_t* const b = g->scatter_box.ensure(kScatterMaxPoses * 24) == cudaSuccess ? g->scatter_box.as<uint8_t>() : nullptr;
+    if (b == nullptr) {
+      (void)cudaGetLastError();
+      return ALIGN_OK;
+    }
+    CU(cudaMemset2DAsync(b, 24, 0x7F, 12, kScatterMaxPoses, g->stream), "clear boxes");
+    CU(cudaMemset2DAsync(b + 12, 24, 0x80, 12, kScatterMaxPoses, g->stream), "clear boxes");
   }
   if (g->scatter_list.ensure((size_t)P * (size_t)a.list_cap * 4) != cudaSuccess) {
     (void)cudaGetLastError();
     return ALIGN_OK;
   }
   *taken = true;
-  const size_t KK = (size_t)g->gc.K * g->gc.K;
-  CU(g->out_c.ensure((size_t)P * KK * sizeof(uint32_t) + 16), "allocate histograms");
-  CU(g->out_box.ensure((size_t)P * 6 * sizeof(int32_t)), "allocate boxes");
-  CU(g->redo_list.ensure((size_t)P * 4), "allocate redo list");
-  CU(g->redo_count.ensure(16), "allocate redo count");
-  CU(g->scatter_n.ensure((size_t)P * 4), "allocate list sizes");
   align_status st = ensure_head(g);
   if (st != ALIGN_OK) return st;
   a.symA = g->symA.as<uint8_t>();
@@ -876,9 +883,8 @@ align_status enqueue_scatter(align_grid* g, const float* d_poses, int64_t P, con
   a.list = g->scatter_list.as<uint32_t>();
   a.list_n = g->scatter_n.as<uint32_t>();
   a.wide_count = &g->dev_head()->wide_count;
-  a.out_c = g->out_c.as<uint32_t>();
-  a.out_box = g->out_box.as<int32_t>();
-  a.redo_count = g->redo_count.as<uint32_t>();
+  a.out_c = g->scatter_c.as<uint32_t>();
+  a.out_box = g->scatter_box.as<int32_t>();
   a.best = &g->dev_head()->best;
 
   EvalItem item{};
@@ -898,6 +904,8 @@ align_status enqueue_scatter(align_grid* g, const float* d_poses, int64_t P, con
   e.n_items = 1;
   e.P = (int32_t)P;
   e.K = g->gc.K;
+  e.done = &g->dev_head()->done;
+  e.list_n = a.list_n;
   const EvalKernels& ek = eval_shape(0);
   std::array<cudaEvent_t, 3> evs{};
   st = profile_event(g, evs, 0);
@@ -906,10 +914,9 @@ align_status enqueue_scatter(align_grid* g, const float* d_poses, int64_t P, con
   CU(launch_scatter(a, g->n_sm, g->stream, &launches), "launch scattered evaluation");
   if ((st = profile_event(g, evs, 1)) != ALIGN_OK) return st;
   CU(ek.launch_compose(e, g->stream), "launch compose kernel");
-  CU(ek.launch_argmax_one(item, g->stream), "launch argmax");
   if ((st = profile_event(g, evs, 2)) != ALIGN_OK) return st;
   g->stats[3] = 0;
-  g->stats[4] += launches + 2;  // and compose, argmax
+  g->stats[4] += launches + 1;  // and compose
   g->stats[5] = 4;
   g->last_lattice = true;  // no tables: nothing to learn
   return ALIGN_OK;
@@ -1218,7 +1225,7 @@ align_status align_destroy_grid(align_grid* g) {
                     &g->lat_cand, &g->ref_pts, &g->ref_pose, &g->ref_cnt, &g->ref_s1, &g->ref_s2, &g->ref_box, &g->ref_rows,
                     &g->ref_list,
                     &g->units, &g->lat_units, &g->spill, &g->lattice_ws, &g->lattice_order, &g->scatter_sums,
-                    &g->scatter_list, &g->scatter_n})
+                    &g->scatter_list, &g->scatter_n, &g->scatter_c, &g->scatter_box})
     b->release();
   for (HostBuf* b : {&g->head_h, &g->hist_h, &g->lat_cand_h, &g->lat_rec_h, &g->lat_c_h, &g->ref_box_h}) b->release();
   for (cudaEvent_t e : g->lat_ev) cudaEventDestroy(e);

@@ -89,7 +89,6 @@ constexpr size_t kScatterBudget = (size_t)1 << 30;  // sums and lists of poses s
 // they cross at 36 poses (0.25 m LiDAR grid), 42 (0.5 m), 56 (1 m), 22 on the 6.4M-voxel grid, where
 // the budget holds 10.
 constexpr int64_t kScatterMaxPoses = 32;
-constexpr size_t kLatticeBudget = (size_t)5 << 28;  // workspace of a round of a pose lattice (1.25 GiB)
 bool plan_lattice(const GridConst& gc, int n_sm, size_t smem_optin, int64_t n, int64_t n_rot, int32_t mx, int32_t my,
                   int32_t mz, double t_max, int min_groups, LatticeArgs& a);
 // The same for the levels of a lattice search over n points (align_search_ex).
@@ -110,6 +109,7 @@ struct GridHead {
   uint32_t err, max_passes, wide_count, wide_poses;
   int64_t argmax;
   unsigned long long best;
+  uint32_t done, pad;  // compose_kernel's CTAs that have finished: 0 between launches
 };
 constexpr size_t kHeadBytes = (size_t)1 << 16;
 constexpr int64_t kHeadPoses = (int64_t)((kHeadBytes - sizeof(GridHead)) / 4);
@@ -161,7 +161,8 @@ struct align_grid {
                               // whose request was admitted without the groups' memory)
   mialign::DevBuf lattice_ws, lattice_order;  // groups' workspace; a device-built level's pose order
   int32_t lattice_order_m[6] = {0, 0, 0, 0, 0, 0};
-  mialign::DevBuf scatter_sums, scatter_list, scatter_n;  // poses that share nothing (zeroed sums)
+  // poses that share nothing; all but the list as the kernels leave it between calls (zero, no box)
+  mialign::DevBuf scatter_sums, scatter_list, scatter_n, scatter_c, scatter_box;
   bool last_cluster = false;  // ... or ran one pose per 2-CTA cluster
   mialign::DevBuf units;    // pose pairs of the last pair launch with host poses
   mialign::DevBuf spill;    // runs queued for the later key partitions (EvalArgs::spill)

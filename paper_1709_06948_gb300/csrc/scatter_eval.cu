@@ -12,8 +12,10 @@
 //
 //   sums_kernel    points -> sums and lists of occupied voxels
 //   voxels_kernel  listed voxels -> feature symbols, joint histogram and occupied box per pose
-// compose_kernel (eval.cu) then gives MI and argmax.  Both kernels are bound by the latency of their
-// L2 atomics and scattered accesses.  Measured per call with device inputs and outputs, 120k points at
+// compose_kernel (eval.cu) then gives MI and argmax, and resets the histogram, box and list counter that
+// it has read: a call is these three kernels (with one to clear and one for the
+// argmax 64 us per one-pose call with its read-back, now 57; 16 simplices x 25 iterations 3.05 -> 2.78 ms).  Both kernels are bound by the latency of their
+// L2 atomics and scattered accesses.  Measured, before that, per call with device inputs and outputs, 120k points at
 // 0.5 m: 105 -> 46 us for one pose, 110 -> 70 us for 16; at 0.25 m 153 -> 54 and 161 -> 90 us; 259k
 // points on the 6.4M-voxel grid 315 -> 76 us and (10 poses) 344 -> 147 us.  Every sum is exact in 64 bits (at most
 // kScatterMaxPoints points), so no pose needs the exact path.
@@ -30,19 +32,6 @@ namespace {
 constexpr uint32_t kFullMask = 0xFFFFFFFFu;
 constexpr int kShiftN = 40;  // n above S1: S1 <= 2^22 points x 8,004 mm < 2^35
 constexpr int kSumThreads = 512, kVoxelThreads = 512;
-
-// Clears what the call accumulates into but the sums, which voxels_kernel leaves at zero.
-__global__ void __launch_bounds__(256) init_kernel(const __grid_constant__ ScatterArgs a) {
-  const int64_t g0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, gs = (int64_t)gridDim.x * blockDim.x;
-  const int64_t n_c = (int64_t)a.P * a.gc.K * a.gc.K;  // a multiple of 4 words is allocated
-  for (int64_t i = g0; i < (n_c + 3) / 4; i += gs) reinterpret_cast<uint4*>(a.out_c)[i] = make_uint4(0u, 0u, 0u, 0u);
-  for (int64_t i = g0; i < 6 * (int64_t)a.P; i += gs) a.out_box[i] = i % 6 < 3 ? INT_MAX : INT_MIN;
-  for (int64_t i = g0; i < a.P; i += gs) a.list_n[i] = 0u;
-  if (g0 == 0) {
-    *a.best = 0ull;
-    *a.redo_count = 0u;
-  }
-}
 
 // One thread per point and pose; blockIdx.y walks the poses.
 template <bool kVar>
@@ -116,6 +105,7 @@ __global__ void __launch_bounds__(kVoxelThreads) voxels_kernel(const __grid_cons
   const int tid = threadIdx.x, pose = blockIdx.y, K = gc.K, KK = K * K;
   const uint32_t n_list = __ldg(a.list_n + pose);
   const uint32_t step = gridDim.x * kVoxelThreads;
+  if (blockIdx.x == 0 && pose == 0 && tid == 0) *a.best = 0ull;
   if (blockIdx.x * kVoxelThreads >= n_list) return;
   for (int i = tid; i < KK; i += kVoxelThreads) hist[i] = 0u;
   for (int i = tid; i < kMaxLevels; i += kVoxelThreads) {
@@ -185,22 +175,21 @@ size_t scatter_pose_bytes(const GridConst& gc, int64_t n) {
 cudaError_t launch_scatter(const ScatterArgs& a, int n_sm, cudaStream_t s, int32_t* launches) {
   cudaError_t e;
   const bool var = a.gc.feature != 0;
-  init_kernel<<<n_sm, 256, 0, s>>>(a);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  *launches += 1;
-  if (a.n <= 0) return cudaSuccess;
-  const int64_t bx = (a.n + kSumThreads - 1) / kSumThreads;
-  // poses in turn once the points alone fill the GPU a few times over
-  const int64_t by = std::min<int64_t>(a.P, std::max<int64_t>(1, 32 * (int64_t)n_sm / bx));
-  const dim3 gp((unsigned)bx, (unsigned)by);
-  if (var) sums_kernel<true><<<gp, kSumThreads, 0, s>>>(a);
-  else sums_kernel<false><<<gp, kSumThreads, 0, s>>>(a);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (a.n > 0) {
+    const int64_t bx = (a.n + kSumThreads - 1) / kSumThreads;
+    // poses in turn once the points alone fill the GPU a few times over
+    const int64_t by = std::min<int64_t>(a.P, std::max<int64_t>(1, 32 * (int64_t)n_sm / bx));
+    const dim3 gp((unsigned)bx, (unsigned)by);
+    if (var) sums_kernel<true><<<gp, kSumThreads, 0, s>>>(a);
+    else sums_kernel<false><<<gp, kSumThreads, 0, s>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    *launches += 1;
+  }
   const dim3 gv((unsigned)std::max(1, std::min(16, 2 * n_sm / a.P)), (unsigned)a.P);
   if (var) voxels_kernel<true><<<gv, kVoxelThreads, 0, s>>>(a);
   else voxels_kernel<false><<<gv, kVoxelThreads, 0, s>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  *launches += 2;
+  *launches += 1;
   return cudaSuccess;
 }
 
