@@ -274,6 +274,7 @@ struct ScatterArgs {
   uint32_t* wide_count;      // voxels past the 32-bit sums
   uint32_t* out_c;           // P x K x K, zero between calls
   int32_t* out_box;          // P x 6, kNoBoxLo and kNoBoxHi between calls
+  uint32_t* redo_count;      // set to 0 (no pose needs the exact path)
   unsigned long long* best;  // reset
 };
 size_t scatter_pose_bytes(const GridConst& gc, int64_t n);  // sums and list of one pose

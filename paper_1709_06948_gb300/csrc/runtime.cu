@@ -874,6 +874,7 @@ align_status enqueue_scatter(align_grid* g, const float* d_poses, int64_t P, con
     return ALIGN_OK;
   }
   *taken = true;
+  CU(g->redo_count.ensure(16), "allocate redo count");
   align_status st = ensure_head(g);
   if (st != ALIGN_OK) return st;
   a.symA = g->symA.as<uint8_t>();
@@ -883,6 +884,7 @@ align_status enqueue_scatter(align_grid* g, const float* d_poses, int64_t P, con
   a.list = g->scatter_list.as<uint32_t>();
   a.list_n = g->scatter_n.as<uint32_t>();
   a.wide_count = &g->dev_head()->wide_count;
+  a.redo_count = g->redo_count.as<uint32_t>();
   a.out_c = g->scatter_c.as<uint32_t>();
   a.out_box = g->scatter_box.as<int32_t>();
   a.best = &g->dev_head()->best;

@@ -13,11 +13,12 @@
 //   sums_kernel    points -> sums and lists of occupied voxels
 //   voxels_kernel  listed voxels -> feature symbols, joint histogram and occupied box per pose
 // compose_kernel (eval.cu) then gives MI and argmax, and resets the histogram, box and list counter that
-// it has read: a call is these three kernels (with one to clear and one for the
-// argmax 64 us per one-pose call with its read-back, now 57; 16 simplices x 25 iterations 3.05 -> 2.78 ms).  Both kernels are bound by the latency of their
-// L2 atomics and scattered accesses.  Measured, before that, per call with device inputs and outputs, 120k points at
-// 0.5 m: 105 -> 46 us for one pose, 110 -> 70 us for 16; at 0.25 m 153 -> 54 and 161 -> 90 us; 259k
-// points on the 6.4M-voxel grid 315 -> 76 us and (10 poses) 344 -> 147 us.  Every sum is exact in 64 bits (at most
+// it has read: a call is these three kernels.  (With a kernel to clear and one for the argmax a one-pose
+// call with its read-back took 64 us, now 57; 16 simplices x 25 iterations 3.05, now 2.78 ms.)  Both are
+// bound by the latency of their L2 atomics and scattered accesses.  Against the table kernels, with
+// those two kernels still, per call with device inputs and outputs: 120k points at 0.5 m 105 -> 46 us
+// for one pose, 110 -> 70 us for 16; at 0.25 m 153 -> 54 and 161 -> 90 us; 259k points on the
+// 6.4M-voxel grid 315 -> 76 us and (10 poses) 344 -> 147 us.  Every sum is exact in 64 bits (at most
 // kScatterMaxPoints points), so no pose needs the exact path.
 #include <algorithm>
 #include <climits>
@@ -105,7 +106,10 @@ __global__ void __launch_bounds__(kVoxelThreads) voxels_kernel(const __grid_cons
   const int tid = threadIdx.x, pose = blockIdx.y, K = gc.K, KK = K * K;
   const uint32_t n_list = __ldg(a.list_n + pose);
   const uint32_t step = gridDim.x * kVoxelThreads;
-  if (blockIdx.x == 0 && pose == 0 && tid == 0) *a.best = 0ull;
+  if (blockIdx.x == 0 && pose == 0 && tid == 0) {
+    *a.best = 0ull;
+    *a.redo_count = 0u;
+  }
   if (blockIdx.x * kVoxelThreads >= n_list) return;
   for (int i = tid; i < KK; i += kVoxelThreads) hist[i] = 0u;
   for (int i = tid; i < kMaxLevels; i += kVoxelThreads) {

@@ -76,3 +76,31 @@ def test_dense_voxel_past_32_bit_sums():
     xyz = xyz.astype(np.float32)
     st = _check(spec, xyz, xyz, _poses(3, 11, 0.02))
     assert st["wide_voxels"] >= 1
+
+
+def test_calls_in_turn_leave_nothing_behind():
+    """Table kernels with exact-path poses, then scattered calls of other sizes, places and outputs on the
+    same grid: each as on a fresh one, and no pose of an earlier call listed as redone."""
+    from paper_1709_06948_gb300 import align
+    rng = np.random.default_rng(94)
+    spec = scangen.lidar_grid(0.5)
+    xyz = np.stack([rng.uniform(a, a + 0.2, 70000) for a in (1.15, 2.15, 0.15)], 1).astype(np.float32)
+    L = lib_grid(spec)
+    align.align_set_reference(L, xyz)
+    align.align_set_sweep(L, 0)
+    align.align_eval_mi(L, xyz, eta6=_poses(40, 12, 0.02))
+    assert len(align.align_eval_redo_poses(L)) > 0
+    align.align_set_sweep(L, -1)
+    away = _poses(2, 17)
+    away[:, 0] = 1000.0, -1000.0  # no point in the grid: an empty overlap
+    for n, etas in ((70000, _poses(4, 13, 0.02)), (70000, away), (0, _poses(1, 14)), (9, _poses(9, 15)), (70000, _poses(2, 16))):
+        got = align.align_eval_mi(L, xyz[:n], eta6=etas, with_hist=n != 9)
+        assert align.align_eval_stats(L)["sweep"] == 4 and len(align.align_eval_redo_poses(L)) == 0
+        F = lib_grid(spec)
+        align.align_set_reference(F, xyz)
+        align.align_set_sweep(F, 0)
+        want = align.align_eval_mi(F, xyz[:n], eta6=etas, with_hist=n != 9)
+        assert np.array_equal(got[0].view(np.int32), want[0].view(np.int32)) and got[1] == want[1]
+        assert n == 9 or np.array_equal(got[2], want[2])
+        F.close()
+    L.close()
