@@ -5,8 +5,9 @@
 // constants (EvalItem).  The launch sequence (clear, pack, eval + redo, compose, argmax)
 // can be captured as a CUDA graph and replayed while the batch keeps its shape; inputs are
 // copied into the batch's own buffers before each launch, so the graph's pointers stay
-// valid.  The kernel shape is fixed, the default, or picked by timing the candidates on the
-// batch itself (tuner below).
+// valid.  Pairs whose poses are a lattice are evaluated by groups (lattice_eval.cu), one after
+// another from one workspace; the others by the table kernels, whose shape is fixed, the default,
+// or picked by timing the candidates on the batch itself (tuner below).
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -15,7 +15,8 @@
 //
 // Memory: the budget covers the references and every slot's workspace, which keeps the
 // buffers of the largest request it has run (re-allocating between requests would
-// synchronise the device under the other slots' work).  When the request at the head of
+// synchronise the device under the other slots' work).  A request counts as the larger of what
+// the pose groups and the table kernels need: either may run its levels.  When the request at the head of
 // the queue fits only without them and nothing runs, idle slots release their workspaces.
 #include <cuda_runtime.h>
 
