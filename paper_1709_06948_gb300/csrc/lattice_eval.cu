@@ -493,7 +493,10 @@ __global__ void __launch_bounds__(kNT, 1024 / kNT) lattice_eval_kernel(const __g
     }
     // First and last elements of the next rows, one row per thread: copied to shared memory while the
     // chunk before is evaluated (held in registers they are spilled, and the spill waits for them).
+    // A thread's copies are not ordered among themselves: those of the rows fetched before (a chunk
+    // that is planned again) land first, or the plan could read them in place of the new ones.
     auto fetch_rows = [&]() {
+      asm volatile("cp.async.wait_all;" ::: "memory");
       const int lin = row + tid;
       if (tid < kRowBatch && lin < row_end) {
         const int kz = lin / Y, ky = lin - kz * Y;

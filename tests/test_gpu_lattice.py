@@ -90,6 +90,24 @@ def test_sparse_rows(tiny, feature, n):
     _check(spec, tiny.xyzA * squeeze, np.ascontiguousarray(tiny.xyzB[:: 8000 // n] * squeeze), _lattice((7, 20, 2, 1, 1, 4), SMALL))
 
 
+@pytest.mark.parametrize("feature", [0, 1, 2])
+def test_rows_planned_again(feature):
+    """Layers of points that share a few cells (chunks are planned ever larger) between layers of points
+    with cells of their own: the chunk after each change holds more cells than planned and is planned
+    again, with other rows' ends copied into the same words."""
+    rng = np.random.default_rng(96)
+    spec = scangen.GridSpec(origin=(-25.0, -3.0, 0.0), res_m=0.25, dims=(200, 24, 8), feature=feature, count_levels=7,
+                            var_levels=8 if feature == 2 else 15)
+    n = 24 * 600
+    layers = []
+    for k in range(8):
+        x = rng.uniform(-24, 24, 10)[rng.integers(0, 10, n)] if k % 2 == 0 else rng.uniform(-24, 24, n)
+        y = -2.875 + 0.25 * rng.integers(0, 24, n) if k % 2 == 0 else rng.uniform(-3, 3, n)
+        layers.append(np.stack([x, y, np.full(n, 0.25 * k + 0.12) + rng.uniform(-0.1, 0.1, n) * (k % 2)], 1))
+    xyz = np.concatenate(layers).astype(np.float32)
+    _check(spec, xyz, xyz, _lattice((8, 20, 2, 1, 1, 4), (0.8, 0.7, 0.25, 0.0, 0.0, 0.01)), sample=8)
+
+
 def test_non_finite_points_and_wide_thresholds(tiny):
     xyz = tiny.xyzB.copy()
     xyz[::7, 0] = np.nan
