@@ -112,20 +112,26 @@ __global__ void ref_list_kernel(const GridConst gc, const uint8_t* __restrict__ 
   const int64_t V = (int64_t)gc.X * gc.Y * gc.Z;
   for (int64_t v0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 16; v0 < V;
        v0 += (int64_t)gridDim.x * blockDim.x * 16) {
-    uint8_t s[16];
+    uint32_t q[4] = {0u, 0u, 0u, 0u};  // 16 symbols, the first in the lowest byte
     if (v0 + 16 <= V) {
-      *reinterpret_cast<uint4*>(s) = *reinterpret_cast<const uint4*>(symA + v0);
-      const uint4 q = *reinterpret_cast<const uint4*>(s);
-      if ((q.x | q.y | q.z | q.w) == 0u) continue;
+      const uint4 w = *reinterpret_cast<const uint4*>(symA + v0);  // v0 is a multiple of 16
+      q[0] = w.x, q[1] = w.y, q[2] = w.z, q[3] = w.w;
     } else {
-      for (int k = 0; k < 16; ++k) s[k] = v0 + k < V ? symA[v0 + k] : 0;
+#pragma unroll
+      for (int k = 0; k < 16; ++k)
+        if (v0 + k < V) q[k / 4] |= (uint32_t)symA[v0 + k] << (8 * (k % 4));
     }
-    for (int k = 0; k < 16; ++k) {
-      if (s[k] == 0) continue;
-      const int64_t v = v0 + k;
-      const uint32_t kx = (uint32_t)(v % gc.X), ky = (uint32_t)((v / gc.X) % gc.Y),
-                     kz = (uint32_t)(v / ((int64_t)gc.X * gc.Y));
-      list[atomicAdd(&row_n[(size_t)(s[k] - 1) * gc.Y + ky + 1], 1u)] = kx | kz << 16;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      for (uint32_t left = q[j]; left != 0u;) {
+        const int k = (__ffs(left) - 1) / 8;
+        const uint32_t sym = (left >> (8 * k)) & 0xFFu;
+        left &= ~(0xFFu << (8 * k));
+        const int64_t v = v0 + 4 * j + k;
+        const uint32_t kx = (uint32_t)(v % gc.X), ky = (uint32_t)((v / gc.X) % gc.Y),
+                       kz = (uint32_t)(v / ((int64_t)gc.X * gc.Y));
+        list[atomicAdd(&row_n[(size_t)(sym - 1u) * gc.Y + ky + 1], 1u)] = kx | kz << 16;
+      }
     }
   }
 }

@@ -38,3 +38,29 @@ def test_reference_symbols_and_marginals(dims, res, feature):
         mo, ho, _ = G.eval_mi(symA, boxA, B, poses, nthreads=oracle.host_cores(), with_hist=True)
         assert np.array_equal(hist, ho) and np.max(np.abs(mi.astype(np.float64) - mo)) <= mi_tolerance()
     L.close()
+
+
+@pytest.mark.parametrize("dims,res", [((161, 62, 17), 0.1), ((160, 64, 17), 0.1), ((419, 131, 3), 0.1)])
+def test_reference_with_every_voxel_occupied(dims, res):
+    """Sixteen symbols of a list thread's words all set, and the last thread's part of them (the sizes of
+    the grids leave 14, 0 and 11 voxels for it)."""
+    from paper_1709_06948_gb300 import align
+    rng = np.random.default_rng(95)
+    size = np.array(dims) * res
+    spec = scangen.GridSpec(origin=tuple(-size / 2), res_m=res, dims=dims, feature=2, count_levels=7, var_levels=8)
+    k = np.stack(np.meshgrid(*(np.arange(d) for d in dims), indexing="ij"), -1).reshape(-1, 3)
+    k = k[np.repeat(np.arange(len(k)), rng.integers(1, 4, len(k)))]
+    A = ((k + rng.uniform(0.3, 0.7, k.shape)) * res - size / 2).astype(np.float32)
+    L, G = lib_grid(spec), oracle_grid(spec)
+    align.align_set_reference(L, A)
+    symA, boxA = G.reference(A)
+    assert np.count_nonzero(symA) == len(symA.reshape(-1))
+    sym, box = align.align_get_reference(L)
+    assert np.array_equal(sym, symA) and np.array_equal(box, boxA)
+    etas = rng.uniform(-0.3, 0.3, (6, 6)) * np.concatenate([size, np.full(3, 0.1)])
+    B = A[rng.integers(0, len(A), 4000)]
+    _, _, hist = align.align_eval_mi(L, B, eta6=etas, with_hist=True)
+    _, ho, _ = G.eval_mi(symA, boxA, B, align.align_round_poses(spec.origin, etas), nthreads=oracle.host_cores(),
+                         with_hist=True)
+    assert np.array_equal(hist, ho)
+    L.close()
