@@ -525,6 +525,11 @@ __global__ void __launch_bounds__(kNT, 1024 / kNT) lattice_eval_kernel(const __g
       }
     };
 
+    // The item's remaining rows are left out: its poses are finished by the exact path.
+    auto give_up = [&]() {
+      if (tid < G) C.wide[tid] = 1u;
+    };
+
     while (row < row_end) {
       // ---- plan: as many of the next rows as fit the arena ----
       // cells of a row: at most its elements; `share` (of 256) of that bound as the last chunks had it
@@ -547,7 +552,10 @@ __global__ void __launch_bounds__(kNT, 1024 / kNT) lattice_eval_kernel(const __g
                                                 rows_in * row_cost(W, kSparse) + kArenaSlack <=
                                             mem.arena_bytes;
       const int taken = __syncthreads_count(fits);
-      if (taken == 0) break;  // never: the arena holds any one row (lattice_layout)
+      if (taken == 0) {  // never: the arena holds any one row (lattice_layout); else the exact path has its poses
+        give_up();
+        break;
+      }
       if (tid < taken) {
         const uint32_t rl = before >> 21;
         row_local[tid] = flag ? (uint16_t)rl : (uint16_t)kNoRow;
@@ -694,7 +702,10 @@ __global__ void __launch_bounds__(kNT, 1024 / kNT) lattice_eval_kernel(const __g
       }
       // more than planned: fewer rows
       if (over || M > 8190u || used + 16u * (M + 1u) > mem.arena_bytes) {
-        if (share == 256u) break;  // never: the bound holds
+        if (share == 256u) {  // never: the bound holds
+          give_up();
+          break;
+        }
         const uint32_t need = over ? share + share / 2u : kSparse ? (16u * M + 6u * n_words) * 13u / bound : (M * 280u) / bound;
         share = min(256u, max(share + 1u, need + 8u));  // as these rows have it
         row = row0;
