@@ -600,7 +600,7 @@ align_status enqueue_eval(align_grid* g, int32_t n_tiles, const float* d_poses, 
     }
   }
   // poses that share no rotations (or a single pose): spread over the GPU
-  if ((rotate || P == 1) && P <= kScatterMaxPoses && out.dump == nullptr && g->sweep_mode < 0) {
+  if ((rotate || P == 1) && P <= kScatterMaxPoses && out.dump == nullptr && g->sweep_mode < 0 && g->scatter_on) {
     bool taken = false;
     align_status st = enqueue_scatter(g, d_poses, P, out, &taken);
     if (st != ALIGN_OK || taken) return st;

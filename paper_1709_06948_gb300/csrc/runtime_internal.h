@@ -159,6 +159,8 @@ struct align_grid {
   bool last_lattice = false;  // ... or a pose lattice by groups
   int32_t lattice_on = 1;     // 0: pose lattices go through the table kernels (a server's workspace
                               // whose request was admitted without the groups' memory)
+  int32_t scatter_on = 1;     // 0: poses that share nothing go through the table kernels (a server's
+                              // workspace: its requests' estimates hold no dense sums)
   mialign::DevBuf lattice_ws, lattice_order;  // groups' workspace; a device-built level's pose order
   int32_t lattice_order_m[6] = {0, 0, 0, 0, 0, 0};
   // poses that share nothing; all but the list as the kernels leave it between calls (zero, no box)

@@ -146,6 +146,7 @@ align_grid* workspace_create(int device, int n_sm, size_t smem_optin, cudaStream
   g->n_sm = n_sm;
   g->smem_optin = smem_optin;
   g->stream = stream;
+  g->scatter_on = 0;  // up to 1 GiB of sums per slot that no estimate counts
   return g;
 }
 

@@ -190,3 +190,28 @@ def test_poll_and_errors(world):
         align.align_submit(s, 99, world.tiny.xyzB, np.zeros(6), RNG_T, levels=1)
     assert e.value.status == align.ALIGN_E_INVALID
     s.close()
+
+
+def test_few_pose_request_stays_within_its_estimate(world):
+    """A search of 8 headings and no translations (more rotations than a quarter of its poses): its
+    workspace holds no more device memory than the server counts for it, and it gives the result of
+    align_search_ex alone."""
+    import torch
+    from paper_1709_06948_gb300 import align
+    spec = scangen.GridSpec(origin=(-37.5, -37.5, -1.0), res_m=0.25, dims=(300, 300, 30), feature=1, var_levels=15)
+    counts = (1, 1, 1, 1, 1, 8)
+    args = (np.zeros(6), RNG_L)
+    L = lib_grid(spec)
+    align.align_set_reference(L, world.lp.xyzA)
+    T, mi, _ = align.align_search(L, world.lp.xyzB, *args, levels=3, counts=counts)
+    L.close()
+    s = align.align_server_create(8 << 30, 1)
+    ref = align.align_server_add_reference(s, world.lp.xyzA, spec.origin, spec.res_m, spec.dims, spec.feature,
+                                           spec.count_levels, spec.var_levels)
+    held0, free0 = align.align_server_stats(s)["bytes_held"], torch.cuda.mem_get_info()[0]
+    r = align.align_wait(s, align.align_submit(s, ref, world.lp.xyzB, *args, levels=3, counts=counts), 60000)
+    held, used = align.align_server_stats(s)["bytes_held"] - held0, free0 - torch.cuda.mem_get_info()[0]
+    assert r["status"] == 0 and r["T"].tolist() == T.tolist() and r["mi"] == mi
+    # each allocation is rounded up by the driver (a few MB)
+    assert used <= held + (64 << 20), (used, held)
+    s.close()
