@@ -972,7 +972,7 @@ align_status collect_status(align_grid* g) {
   // packed-layout poses that a voxel past nlim_pack sent to the exact path: the grid's scans
   // are dense enough for the three-word layout (a limit several times larger, fewer slots)
   if (h.wide_poses > 0 && g->last_vw == 2 && !g->last_lattice) g->layout_min = 3;
-  g->stats[0] = h.max_passes;
+  if (!g->last_lattice) g->stats[0] = h.max_passes;  // else no table of partitions: as the last one left it
   g->stats[1] = h.wide_count;
   if (h.err & kErrDzBound) return fail(ALIGN_E_INTERNAL, "a z offset exceeded its proven bound");
   if (h.err & kErrPassLimit) return fail(ALIGN_E_INTERNAL, "key partitioning limit reached");
@@ -1165,7 +1165,7 @@ align_status search_pipelined(align_grid* g, int32_t n_tiles, const double c0[6]
     passes_used = std::max(passes_used, rec[l].max_passes);
     if (level_best) level_best[l] = rec[l].argmax;
   }
-  g->stats[0] = passes_used;
+  if (!by_groups) g->stats[0] = passes_used;
   std::memcpy(T_out, c[(size_t)levels].data(), 6 * sizeof(double));
   if (mi_out) {  // the MI of the last level's argmax, from its packed running maximum
     const uint32_t ord = (uint32_t)(rec[levels - 1].best >> 32);

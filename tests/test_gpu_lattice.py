@@ -131,6 +131,33 @@ def test_dense_voxel_goes_to_the_exact_path():
     assert len(redo) > 0
 
 
+def test_partition_count_stays_as_the_tables_left_it():
+    """align_eval_stats' key partitions are the table kernels': neither groups whose redone poses need
+    several (a voxel past the 32-bit sums, more voxels than a table holds) nor scattered poses change them."""
+    from paper_1709_06948_gb300 import align
+    rng = np.random.default_rng(97)
+    spec = scangen.lidar_grid(0.5)
+    dense = np.stack([rng.uniform(a, a + 0.2, 70000) for a in (1.15, 2.15, 0.15)], 1)
+    rest = np.stack([rng.uniform(-39, 39, 60000), rng.uniform(-39, 39, 60000), rng.uniform(-0.9, 6.5, 60000)], 1)
+    xyz = np.concatenate([dense, rest]).astype(np.float32)
+    etas = _lattice((2, 40, 2, 1, 1, 2), (0.05, 0.05, 0.05, 0.0, 0.0, 0.001))
+    L = lib_grid(spec)
+    align.align_set_reference(L, xyz)
+
+    def passes(kind, e):
+        align.align_eval_mi(L, xyz, eta6=e)
+        st = align.align_eval_stats(L)
+        assert st["sweep"] == kind
+        return st["passes"]
+    assert passes(3, etas) == 1 and len(align.align_eval_redo_poses(L)) > 0
+    align.align_set_sweep(L, 0)
+    n = passes(0, etas[:40])
+    assert n > 1
+    align.align_set_sweep(L, -1)
+    assert passes(4, etas[:1]) == n and passes(3, etas) == n
+    L.close()
+
+
 def test_not_a_lattice_keeps_the_table_kernels(tiny):
     """A pose missing, repeated or moved: not every combination, so the poses go to the tables."""
     etas = _lattice((4, 20, 2, 1, 1, 4), SMALL)
