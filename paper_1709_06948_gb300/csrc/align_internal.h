@@ -67,8 +67,6 @@ struct EvalItem {
   uint32_t* hist;             // optional P x K x K full joint histograms
   unsigned long long* best;   // packed (MI, ~index) running maximum (zeroed before the launch)
   int64_t* argmax;            // one
-  const float* xyz;           // the scan itself (n_xyz x 3), for a redo without tiles (launch_redo_raw)
-  int32_t n_xyz;
   int64_t* dump;              // optional: V x 3 (n, S1, S2) of pose 0 (parity checks; S1, S2
                               // are accumulated whenever dump is set, whatever the feature)
   uint32_t* item_passes;      // optional: running max of the partitions this item's poses used
@@ -158,8 +156,8 @@ struct EvalKernels {
   cudaError_t (*launch_pack_batch)(const PackCopy* copies, int n_copies, int64_t max_out, cudaStream_t s);
   // Overlap box, phi column, MI and the running argmax of every pose; a single item's argmax.
   cudaError_t (*launch_compose)(const EvalArgs& a, cudaStream_t s);
-  // The redo kernel alone, over one item whose points are read from EvalItem::xyz.
-  cudaError_t (*launch_redo_raw)(const EvalArgs& a, int n_ctas, int vw, cudaStream_t s);
+  // The redo kernel alone, over one item of raw tiles.
+  cudaError_t (*launch_redo)(const EvalArgs& a, int n_ctas, int vw, cudaStream_t s);
   // Each item's argmax from its packed running maximum (launches of several items).
   cudaError_t (*launch_argmax_finalize)(const EvalItem* items, int n_items, cudaStream_t s);
 };
@@ -199,6 +197,14 @@ struct LatticeLevel {
   uint32_t* err;            // error bits
 };
 cudaError_t launch_lattice_level(const LatticeLevel& L, cudaStream_t s);
+
+// A raw tile copy of a scan for the table kernels of one shape (threads, points per thread and tile):
+// n_out places, the scan's points and NaN.
+struct RawTiles {
+  float4* out;
+  int64_t n_out;
+  int32_t threads, ppt;
+};
 
 constexpr size_t kLatticeBudget = (size_t)5 << 28;  // workspace of a round of a pose lattice (1.25 GiB)
 // A pose lattice evaluated group by group (lattice_eval.cu): every combination of n_rot
@@ -240,6 +246,7 @@ struct LatticeArgs {
   uint4* elems;             // n_pad: elements in bin order
   uint32_t* next_item;
   uint32_t* redo_mark;      // P
+  RawTiles tiles;           // the scan for the exact path, written by the first round
   // outputs, as the table kernels'
   uint32_t* out_c;          // P x K x K, and up to 3 words of padding
   int32_t* out_box;         // P x 6

@@ -43,11 +43,11 @@ struct PairPlan {
   int64_t nB = 0, P = 0;
   int32_t n_tiles = 0;
   int64_t n_pad = 0;
-  int n_copies = 1;          // tile copies: rotations (pre-rotated) or 1 (raw)
+  int n_copies = 1;           // tile copies to pack: rotations (pre-rotated), 1 (raw) or 0 (groups)
   bool prerot = false;
   std::vector<float> hposes;  // host fp32 poses (when given on the host)
   PoseSet set;                // their structure (rotations, lattice)
-  bool by_groups = false;     // a lattice evaluated by groups (no tiles, no table)
+  bool by_groups = false;     // a lattice evaluated by groups (tiles and tables for the exact path only)
   LatticeArgs lat{};
   int64_t order_off = 0;      // its poses' order (in order)
   std::vector<int32_t> units; // pose pairs (pair kernel), two local pose indices per unit
@@ -195,7 +195,7 @@ align_status enqueue_launch(align_batch* b, const Launch& L, int32_t* launches) 
     if (k > 0) BCU(cudaMemsetAsync(b->redo_count.p, 0, 4, s), "clear redo count");
     if (L.lat_rots[k] > 0) {
       BCU(launch_lattice(L.lats[k], L.lat_rots[k], b->n_sm, s, launches), "launch lattice evaluation");
-      BCU(eval_shape(0).launch_redo_raw(L.evals[k], b->n_sm, L.vws[k], s), "launch redo kernel");
+      BCU(L.ek->launch_redo(L.evals[k], b->n_sm, L.vws[k], s), "launch redo kernel");
       *launches += 1;
     } else {
       BCU(L.ek->launch_eval(L.evals[k], L.n_ctas, L.vws[k], L.rotate, s), "launch eval kernel");
@@ -438,7 +438,7 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
     if (pp.by_groups) order_n += pp.P;
     xyz_f += pp.nB * 3;
     poses_n += pp.P;
-    pts_n += (int64_t)pp.n_copies * pp.n_pad;
+    pts_n += std::max(1, pp.n_copies) * pp.n_pad;  // groups: raw tiles for the exact path, written by their kernels
     outc_n += (pp.P * (int64_t)pp.g->gc.K * pp.g->gc.K + 3) / 4 * 4;  // cleared four words at a time
     n_copies += pp.n_copies;
     max_out = std::max(max_out, pp.n_pad);
@@ -451,7 +451,7 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
   for (const PairPlan& pp : plans) {
     if (pp.by_groups) {  // the redo kernel's tables
       vws.push_back(pp.g->gc.feature != ALIGN_FEAT_COUNT ? 2 : 1);
-      Ts.push_back(eval_shape(0).table_slots_for(pp.g->gc.K, vws.back(), b->smem_optin, 1));
+      Ts.push_back(ek.table_slots_for(pp.g->gc.K, vws.back(), b->smem_optin, 1));
       T = std::max(T, Ts.back());
       continue;
     }
@@ -542,8 +542,6 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
     it.sat = g->sat.as<int32_t>();
     it.src = b->pts.as<float4>() + pp.pts_off;
     it.src_stride = (uint64_t)pp.n_pad;
-    it.xyz = b->xyz.as<float>() + pp.xyz_off;
-    it.n_xyz = (int32_t)pp.nB;
     it.pose_src = pp.prerot ? b->pose_src.as<int32_t>() + pp.pose_off : nullptr;
     it.poses = b->poses.as<float>() + pp.pose_off * 12;
     it.n_tiles = pp.n_tiles;
@@ -633,10 +631,11 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
       const EvalItem& it = hitems[(size_t)i];
       lattice_carve(la, b->lattice.as<uint8_t>());
       la.symA = it.symA;
-      la.xyz = it.xyz;
+      la.xyz = b->xyz.as<float>() + plans[(size_t)i].xyz_off;
       la.poses = it.poses;
       la.pose_of = b->order.as<int32_t>() + plans[(size_t)i].order_off;
       la.pose_base = it.pose_base;
+      la.tiles = RawTiles{b->pts.as<float4>() + plans[(size_t)i].pts_off, plans[(size_t)i].n_pad, ek.threads, ek.ppt};
       la.out_c = it.out_c;
       la.out_box = it.out_box;
       la.best = it.best;

@@ -57,6 +57,18 @@ __device__ __forceinline__ uint32_t voxel_key(const Pose12& P, float x, float y,
                      dz);
 }
 
+// Scan point i (or padding past the scan) into a raw tile copy: thread s of a CTA walks the points
+// s L .. s L + L - 1, ppt of them per tile (load_tile and stream_of in eval.cu).
+__device__ __forceinline__ void store_raw_point(const RawTiles& T, int64_t i, float x, float y, float z) {
+  const uint32_t L = (uint32_t)(T.n_out / T.threads), warps = (uint32_t)T.threads >> 5, tile = (uint32_t)(T.threads * T.ppt);
+  const uint32_t s = (uint32_t)i / L, w = (uint32_t)i - s * L;
+  const uint32_t t = w / (uint32_t)T.ppt, j = w - t * (uint32_t)T.ppt;
+  const uint32_t pos = j * (uint32_t)T.threads + (s % warps) * 32u + s / warps;
+  float4* to = T.out + (size_t)t * tile;
+  reinterpret_cast<float2*>(to)[pos] = make_float2(x, y);
+  (reinterpret_cast<float*>(to) + 2 * (size_t)tile)[pos] = z;
+}
+
 // ---------------------------------------------------------------------------------
 // Feature symbol of one voxel from its exact integer sums (Sec. III-A features; phi = 0).
 // count level    = #{ j : n >= ct[j] }                     (ct ascending)

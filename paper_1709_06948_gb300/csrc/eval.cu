@@ -793,7 +793,8 @@ __device__ __forceinline__ void load_pose(const float* poses, PoseRegs& P) {
   for (int i = 0; i < 3; ++i) P.t[i] = __ldg(poses + 9 + i);
 }
 
-// Tile layout (kTile float4 slots of storage per tile): x,y of the tile's points as float2
+// Tile layout (kTile float4 slots of storage per tile; store_raw_point in device_common.cuh writes it
+// for any shape): x,y of the tile's points as float2
 // in the first half, z as float in the next quarter (12 bytes read per point).  `src` is
 // the copy's base plus this thread's index.
 __device__ __forceinline__ void load_tile(const float4* src, int t, float4* v) {
@@ -1687,8 +1688,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 // Poses that eval_kernel could not finish: plain sweeps; each run goes straight into the
 // table with 64-bit side sums for voxels beyond the 32-bit bound; a full table restarts
 // the pose with twice the key partitions.
-// kRaw: the points are read from the item's scan instead of tiles (kRot: the kernel rotates).
-template <int kVW, bool kRot, bool kRaw = false>
+template <int kVW, bool kRot>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) redo_kernel(const __grid_constant__ EvalArgs a) {
   constexpr bool kVar = kVW > 1;
   extern __shared__ __align__(128) uint8_t smem_raw[];
@@ -1713,8 +1713,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) redo_kernel(const __grid
     const uint32_t run_lim = S.gc->nlim;  // runs with 32-bit sums of dz and dz^2, cut at nlim
     PoseRegs P;
     load_pose(I.poses + 12 * (size_t)lp, P);
-    const float4* src = kRaw ? nullptr : pose_tiles(I, lp) + tid;
-    const int n_tiles = kRaw ? (int)(((int64_t)I.n_xyz + kTile - 1) / kTile) : I.n_tiles;
+    const float4* src = pose_tiles(I, lp) + tid;
     // Start from the item's partition count: a pose redone for its wide sums needs no more,
     // one redone for a full table doubles below until its partitions fit.
     int passes = max(1, min(I.passes0 > 0 ? I.passes0 : a.passes0, kMaxPasses));
@@ -1724,19 +1723,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) redo_kernel(const __grid
       // plain runs: count n, S1 (two's complement) and S2, cut at nlim points
       uint32_t rkey = kEmptyKey, rn = 0u, rs1 = 0u, rs2 = 0u;
       uint32_t bad = 0u;
-      for (int t = 0; t < n_tiles; ++t) {
+      for (int t = 0; t < I.n_tiles; ++t) {
         float4 v[kPPT];
-        if constexpr (kRaw) {
-#pragma unroll
-          for (int j = 0; j < kPPT; ++j) {
-            const int64_t p = (int64_t)t * kTile + j * kThreads + tid;
-            const float nan = __int_as_float(0x7fc00000);  // past the scan: outside every grid
-            v[j] = p < I.n_xyz ? make_float4(__ldg(I.xyz + 3 * p), __ldg(I.xyz + 3 * p + 1), __ldg(I.xyz + 3 * p + 2), 0.0f)
-                               : make_float4(nan, nan, nan, 0.0f);
-          }
-        } else {
-          load_tile(src, t, v);
-        }
+        load_tile(src, t, v);
 #pragma unroll
         for (int j = 0; j < kPPT; ++j) {
           uint32_t key;
@@ -1785,7 +1774,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) redo_kernel(const __grid
 
 // Stream (stretch of consecutive scan points) walked by thread `tid`: lane l of warp w takes
 // stream l * kWarps + w, so every warp samples the whole scan and the warps of a CTA finish
-// their sweeps (and drains) at about the same time.
+// their sweeps (and drains) at about the same time.  (store_raw_point follows the same order.)
 __device__ __forceinline__ int stream_of(int tid) { return (tid & 31) * kWarps + (tid >> 5); }
 
 // xyz -> float4 tiles, optionally one rotated copy per rotation.  Tile t, position
@@ -1994,8 +1983,6 @@ cudaError_t setup_t(int smem) {
     e = cudaFuncSetAttribute(eval_kernel<kVW, kRot, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(redo_kernel<kVW, kRot>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e == cudaSuccess && kRot)
-    e = cudaFuncSetAttribute(redo_kernel<kVW, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e == cudaSuccess && !kRot)
     e = cudaFuncSetAttribute(eval_pair_kernel<kVW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e == cudaSuccess && !kRot)
@@ -2072,11 +2059,11 @@ cudaError_t launch_eval(const EvalArgs& a, int n_ctas, int vw, bool rotate, cuda
   }
 }
 
-cudaError_t launch_redo_raw(const EvalArgs& a, int n_ctas, int vw, cudaStream_t s) {
+cudaError_t launch_redo(const EvalArgs& a, int n_ctas, int vw, cudaStream_t s) {
   if (a.item_start != nullptr || a.units != nullptr || (vw != 1 && vw != 2)) return cudaErrorInvalidValue;
   const size_t smem = eval_smem_bytes(a.K, a.table_slots, vw, 1);
-  if (vw == 1) redo_kernel<1, true, true><<<n_ctas, kThreads, smem, s>>>(a);
-  else redo_kernel<2, true, true><<<n_ctas, kThreads, smem, s>>>(a);
+  if (vw == 1) redo_kernel<1, true><<<n_ctas, kThreads, smem, s>>>(a);
+  else redo_kernel<2, true><<<n_ctas, kThreads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -2140,7 +2127,7 @@ cudaError_t launch_argmax_finalize(const EvalItem* items, int n_items, cudaStrea
 const EvalKernels& MI_EVAL_SHAPE_FN() {
   static const EvalKernels k{MI_STR(MI_EVAL_SHAPE_FN), kThreads, kPPT, kCtasPerSm, eval_tile_points, eval_ovf_cap, eval_min_tiles,
                              eval_smem_bytes, eval_table_slots_for, eval_setup, launch_eval, launch_pack_points,
-                             launch_pack_batch, launch_compose, launch_redo_raw, launch_argmax_finalize};
+                             launch_pack_batch, launch_compose, launch_redo, launch_argmax_finalize};
   return k;
 }
 

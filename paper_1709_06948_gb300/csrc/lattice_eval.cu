@@ -109,6 +109,8 @@ __global__ void __launch_bounds__(256) setup_kernel(const __grid_constant__ Latt
     for (int64_t i = g0; i < (n_c + 3) / 4; i += gs) reinterpret_cast<uint4*>(a.out_c)[i] = make_uint4(0u, 0u, 0u, 0u);
     for (int64_t i = g0; i < 6 * (int64_t)a.P; i += gs) a.out_box[i] = i % 6 < 3 ? INT_MAX : INT_MIN;
     for (int64_t i = g0; i < a.P; i += gs) a.redo_mark[i] = 0u;
+    const float nan = __int_as_float(0x7fc00000);
+    for (int64_t i = a.n + g0; i < a.tiles.n_out; i += gs) store_raw_point(a.tiles, i, nan, nan, nan);
   }
   if (g0 == 0) {
     *a.next_item = 0u;
@@ -163,7 +165,9 @@ __global__ void __launch_bounds__(256) points_kernel(const __grid_constant__ Lat
   if (p0 >= a.n) return;
   const int64_t q = min(p, a.n - 1);
   float ux, uy, uz;
-  rotate_point(R, __ldg(a.xyz + 3 * q), __ldg(a.xyz + 3 * q + 1), __ldg(a.xyz + 3 * q + 2), ux, uy, uz);
+  const float px = __ldg(a.xyz + 3 * q), py = __ldg(a.xyz + 3 * q + 1), pz = __ldg(a.xyz + 3 * q + 2);
+  if (a.first && r == 0 && p < a.n) store_raw_point(a.tiles, p, px, py, pz);
+  rotate_point(R, px, py, pz, ux, uy, uz);
   // a non-finite point (or one that overflows) is outside the grid under every pose
   bool in_p = p < a.n && isfinite(ux) && isfinite(uy) && isfinite(uz);
   const uint32_t sy = axis_cell(uy, ty, a.my, gc.inv_res, gc.Y);

@@ -780,16 +780,23 @@ align_status enqueue_lattice(align_grid* g, LatticeArgs a, const float* d_poses,
   a.redo_count = g->redo_count.as<uint32_t>();
   a.best = &g->dev_head()->best;
 
-  // poses with a voxel past the 32-bit sums: the redo kernel, reading the scan itself
+  // Poses with a voxel past the 32-bit sums: the redo kernel, over raw tiles that the lattice's kernels
+  // write beside their own work.  (Reading the scan itself, a point per thread, it merged no runs: 120k
+  // points on a 4 m grid, all 4,096 poses redone, 8.4 ms against 3.1; a launch that packs the tiles when
+  // there are such poses costs 3 us when there are none.)
   const EvalKernels& ek = eval_shape(0);
+  const int64_t n_pad = std::max<int64_t>(ek.min_tiles(), (a.n + ek.tile_points() - 1) / ek.tile_points()) * ek.tile_points();
+  CU(g->pts4.ensure((size_t)n_pad * 16), "allocate tiles");
+  a.tiles = RawTiles{g->pts4.as<float4>(), n_pad, ek.threads, ek.ppt};
   const int vw = g->gc.feature != ALIGN_FEAT_COUNT ? 2 : 1;
   const int redo_ctas = (int)std::min<int64_t>(P, g->n_sm);
   EvalItem item{};
   item.gc = g->gc;
   item.symA = a.symA;
   item.sat = g->sat.as<int32_t>();
-  item.xyz = a.xyz;
-  item.n_xyz = (int32_t)a.n;
+  item.src = g->pts4.as<float4>();
+  item.src_stride = (uint64_t)n_pad;
+  item.n_tiles = (int32_t)(n_pad / ek.tile_points());
   item.poses = d_poses;
   item.P = (int32_t)P;
   item.passes0 = 1;
@@ -824,7 +831,7 @@ align_status enqueue_lattice(align_grid* g, LatticeArgs a, const float* d_poses,
   if ((st = profile_event(g, evs, 0)) != ALIGN_OK) return st;
   int32_t launches = 0;
   CU(launch_lattice(a, n_rot, g->n_sm, g->stream, &launches), "launch lattice evaluation");
-  CU(ek.launch_redo_raw(e, redo_ctas, vw, g->stream), "launch redo kernel");
+  CU(ek.launch_redo(e, redo_ctas, vw, g->stream), "launch redo kernel");
   if ((st = profile_event(g, evs, 1)) != ALIGN_OK) return st;
   CU(ek.launch_compose(e, g->stream), "launch compose kernel");
   if ((st = profile_event(g, evs, 2)) != ALIGN_OK) return st;

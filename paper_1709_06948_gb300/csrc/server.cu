@@ -136,7 +136,8 @@ size_t request_bytes(int64_t nB, const int32_t m[6], int K, int T, int n_sm, int
 size_t groups_bytes(LatticeArgs a, const GridConst& gc, int n_sm, size_t smem_optin) {
   const int64_t per_pose = (int64_t)gc.K * gc.K * 4 + 24 + 4 + 48 + 4 + 4 + 4;
   const int T = eval_shape(0).table_slots_for(gc.K, 2, smem_optin, 1);
-  return lattice_carve(a, nullptr) + (size_t)(a.n * 12 + a.P * per_pose + (int64_t)n_sm * 2 * T * 8);
+  const int64_t n_pad = std::max<int64_t>(3, (a.n + 1023) / 1024) * 1024;  // raw tiles of the exact path
+  return lattice_carve(a, nullptr) + (size_t)(a.n * 12 + n_pad * 16 + a.P * per_pose + (int64_t)n_sm * 2 * T * 8);
 }
 
 align_grid* workspace_create(int device, int n_sm, size_t smem_optin, cudaStream_t stream) {

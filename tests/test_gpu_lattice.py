@@ -131,6 +131,35 @@ def test_dense_voxel_goes_to_the_exact_path():
     assert len(redo) > 0
 
 
+@pytest.mark.parametrize("feature", [1, 2])
+@pytest.mark.parametrize("n", [300, 1024, 3073, 8000])
+def test_coarse_grids_redo_from_tiles(tiny, feature, n):
+    """8 m voxels of hundreds of points: past the 32-bit sums (267), so poses are redone from the tiles
+    that the groups' kernels wrote, at sizes around tiles and streams; one call with fewer points after
+    one with more, and the same in a batch beside a pair for the table kernels, whose shape the tuner picks."""
+    from paper_1709_06948_gb300 import align
+    spec = scangen.GridSpec(origin=(-20.0, -20.0, -1.0), res_m=8.0, dims=(5, 5, 2), feature=feature, count_levels=7,
+                            var_levels=8 if feature == 2 else 15)
+    squeeze = np.array([0.05, 0.05, 1.0] if n < 8000 else [1.0, 1.0, 1.0], np.float32)  # dense at any size
+    B = np.ascontiguousarray(tiny.xyzB[:n] * squeeze)
+    etas = _lattice((4, 20, 2, 1, 1, 4), (6.0, 5.0, 0.3, 0.0, 0.0, 0.5))
+    assert len(_check(spec, tiny.xyzA, B, etas)) > 0
+    L, other = lib_grid(spec), lib_grid(tiny.grid)
+    align.align_set_reference(L, tiny.xyzA)
+    align.align_set_reference(other, tiny.xyzA)
+    rng = np.random.default_rng(98)
+    pairs = [(L, tiny.xyzB, etas), (other, tiny.xyzB, tiny.T + rng.uniform(-0.5, 0.5, (40, 6))), (L, B, etas)]
+    b = align.align_batch_create()
+    for tune in (False, True):
+        got = align.align_eval_batch(b, pairs, tune=tune)
+        for (mi, am), (G, xyz, e) in zip(got, pairs):
+            align.align_set_sweep(G, 0)
+            mi0, am0, _ = align.align_eval_mi(G, xyz, eta6=e)
+            align.align_set_sweep(G, -1)
+            assert np.array_equal(mi.view(np.int32), mi0.view(np.int32)) and am == am0
+    align.align_batch_destroy(b)
+
+
 def test_partition_count_stays_as_the_tables_left_it():
     """align_eval_stats' key partitions are the table kernels': neither groups whose redone poses need
     several (a voxel past the 32-bit sums, more voxels than a table holds) nor scattered poses change them."""
