@@ -439,7 +439,16 @@ bool mialign::plan_lattice(const GridConst& gc, int n_sm, size_t smem_optin, int
   const int64_t words = std::min<int64_t>((int64_t)gc.Z * gc.Y, n / 2) * (a.nsx / 32 + 1);
   if (words > 2 * a.gx * n) return false;
   const int64_t chunks = ((int64_t)mx + a.gx - 1) / a.gx;
-  if (n_rot * mz * my * chunks < min_groups) return false;
+  const int64_t groups = n_rot * mz * my * chunks;
+  if (groups < min_groups) return false;
+  // A list serves my groups and a group gx poses, at costs that depend little on gx: with few of both
+  // the table kernels' pairs are faster.  Pairs' time over groups' (2,048 to 4,096 poses, 8k to 120k
+  // points, 0.25 to 1 m): gx 2 0.38 to 1.1 (0.53 to 0.86 from 30k points on, whatever my is), gx 3 x my
+  // 2 0.74 to 1.3, 8 x 1 0.79 to 1.3, 4 x 2 0.81 to 1.2; 3 x 3 0.96 to 1.35, 5 x 2 1.07 to 1.6; with 8
+  // t'_z, which share a list's rotation, 3 x 2 1.13 to 1.4.  Small lattices stay: they differ by less
+  // than 0.1 ms.
+  const bool shared = a.gx >= 3 && (my * a.gx >= 9 || (my >= 2 && mz >= 8));
+  if (!shared && groups >= 2 * (int64_t)n_sm) return false;
   a.n_rot = 1;
   const size_t fixed = (size_t)P * 4;
   const size_t one = lattice_carve(a, nullptr) - fixed;

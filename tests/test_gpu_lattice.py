@@ -196,6 +196,14 @@ def test_not_a_lattice_keeps_the_table_kernels(tiny):
         _check(tiny.grid, tiny.xyzA, tiny.xyzB, e, sweep=1)
 
 
+@pytest.mark.parametrize("counts,sweep", [((2, 16, 2, 2, 2, 3), 1), ((2, 2, 2, 5, 5, 5), 1), ((8, 1, 2, 5, 5, 8), 1),
+                                          ((4, 2, 2, 5, 5, 8), 1), ((3, 3, 2, 5, 5, 3), 3), ((5, 2, 2, 5, 5, 4), 3),
+                                          ((3, 2, 8, 3, 3, 3), 3), ((8, 8, 1, 2, 2, 10), 3)])
+def test_few_poses_per_list_keep_the_table_kernels(tiny, counts, sweep):
+    """Lattices whose lists and groups serve few poses go to the tables from 2 groups per SM on."""
+    _check(tiny.grid, tiny.xyzA, tiny.xyzB, _lattice(counts, SMALL), sweep=sweep, sample=8)
+
+
 def test_search_levels_by_groups_equal_table_kernels():
     """The six-level search of a LiDAR pair: the same poses and MI with either kind of kernel."""
     from paper_1709_06948_gb300 import align
