@@ -293,11 +293,12 @@ cudaError_t launch_ref_accumulate(const GridConst& gc, const float* xyz, int64_t
 // cnt, s1, s2 are cleared again; row_n (may be NULL): (K - 1) x Y + 1 counts, zero before.
 cudaError_t launch_ref_symbols(const GridConst& gc, uint32_t* cnt, unsigned long long* s1, unsigned long long* s2,
                                uint8_t* symA, int32_t* box, uint32_t* row_n, cudaStream_t s);
-// Prefix sums from the list of A's occupied voxels (row_n as launch_ref_symbols left it; list: one
-// word per occupied voxel), where ref_sat_by_list says so; the whole of sat is written.
+// Prefix sums from the list of A's occupied voxels (row_n as launch_ref_symbols left it; list: a word
+// per occupied voxel), where ref_sat_by_list says so; the whole of sat is written.  Or nothing but *few
+// = 0, for a scan with too many voxels of one symbol: launch_ref_sat is then the faster.
 bool ref_sat_by_list(const GridConst& gc);
 cudaError_t launch_ref_sat_list(const GridConst& gc, const uint8_t* symA, uint32_t* row_n, uint32_t* list,
-                                int32_t* sat, int n_sm, cudaStream_t s);
+                                int32_t* few, int32_t* sat, int n_sm, cudaStream_t s);
 cudaError_t launch_ref_sat(const GridConst& gc, const uint8_t* symA, int32_t* sat, cudaStream_t s);
 
 // Host helpers shared by the C-ABI translation units (defined in runtime.cu).

@@ -61,7 +61,10 @@ __global__ void ref_symbols_kernel(const GridConst gc, uint32_t* __restrict__ cn
       mn[i] = min(mn[i], k[i]);
       mx[i] = max(mx[i], k[i]);
     }
-    if (row_n != nullptr) atomicAdd(&row_n[(size_t)(sym - 1) * gc.Y + ky + 1], 1u);
+    if (row_n != nullptr) {  // one add per row and warp: neighbours share it
+      const uint32_t row = (uint32_t)((sym - 1) * gc.Y + ky), same = __match_any_sync(__activemask(), row);
+      if ((int)(threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(&row_n[(size_t)row + 1], (uint32_t)__popc(same));
+    }
   }
   __syncwarp();
 #pragma unroll
@@ -74,8 +77,9 @@ __global__ void ref_symbols_kernel(const GridConst gc, uint32_t* __restrict__ cn
   }
 }
 
-// Exclusive prefix sums of n values in place, one block.
-__global__ void __launch_bounds__(1024) ref_rows_kernel(uint32_t* v, int64_t n) {
+// Exclusive prefix sums of n values in place, one block; *few: whether no symbol (Y values from entry 1
+// on) counts more than `most` voxels.
+__global__ void __launch_bounds__(1024) ref_rows_kernel(uint32_t* v, int64_t n, int Y, uint32_t most, int32_t* few) {
   __shared__ uint32_t tot[2][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   uint32_t carry = 0u;
@@ -103,12 +107,20 @@ __global__ void __launch_bounds__(1024) ref_rows_kernel(uint32_t* v, int64_t n) 
     if (i < n) v[i] = before + inc - x;
     carry += all;
   }
+  __syncthreads();  // entry 1 + a Y holds the start of symbol a's rows, the last entry that of the last row
+  bool ok = true;
+  const int64_t symbols = (n - 1) / Y;
+  for (int64_t a = threadIdx.x; a < symbols; a += blockDim.x)
+    ok = ok && (a + 1 < symbols ? v[1 + (a + 1) * Y] : carry) - v[1 + a * Y] <= most;
+  ok = __syncthreads_and(ok);
+  if (threadIdx.x == 0) *few = ok ? 1 : 0;
 }
 
 // The occupied voxels as x | z << 16, ordered by (symbol, y).  Entry r + 1 of row_n holds the start
 // of row r and ends as its end: afterwards entry r is the start of row r.
 __global__ void ref_list_kernel(const GridConst gc, const uint8_t* __restrict__ symA, uint32_t* row_n,
-                                uint32_t* __restrict__ list) {
+                                uint32_t* __restrict__ list, const int32_t* few) {
+  if (*few == 0) return;
   const int64_t V = (int64_t)gc.X * gc.Y * gc.Z;
   for (int64_t v0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 16; v0 < V;
        v0 += (int64_t)gridDim.x * blockDim.x * 16) {
@@ -143,14 +155,20 @@ __global__ void ref_list_kernel(const GridConst gc, const uint8_t* __restrict__ 
 // row before.  Everything is written once and nothing but the list is read (the passes below write,
 // read and write it again, and need it cleared): bound by the writes, 1.44 GB for 56 symbols on
 // 400 x 400 x 40 voxels (0.25 to 0.3 ms, 5 TB/s; the whole reference of 87k points 1.69 -> 0.40 ms).
+constexpr int64_t kSatMostBytes = 4096;  // sums' bytes per voxel of one symbol at least (launch_ref_sat_list)
 constexpr int kSatRows = 31, kSatWarps = 4, kSatMaxX = 2048;  // rows per strip at most: a lane per row end
 
-// kRegs: the running counts in registers (x = lane + 32 i, X <= 32 kRegs); 0: in shared memory.
+// kRegs: the running counts in registers (x = lane + 32 i, X <= 32 kRegs); 0: in shared memory.  Of a
+// whole reference of 106k points and 56 symbols: 64 x 64 x 200 voxels 162 us with 5 registers, 184 with
+// 13, 178 without; 160 x 160 x 16 125, 127, 126; 400 x 400 x 40 388 with 13, 390 without; 416 x 380 x 40,
+// 15 symbols, 226 and 232.
 template <int kRegs>
 __global__ void __launch_bounds__(kSatWarps * 32) ref_sat_list_kernel(const GridConst gc,
                                                                       const uint32_t* __restrict__ row_n,
                                                                       const uint32_t* __restrict__ list,
-                                                                      int32_t* __restrict__ sat, int strip_rows) {
+                                                                      int32_t* __restrict__ sat, int strip_rows,
+                                                                      const int32_t* few) {
+  if (*few == 0) return;
   extern __shared__ int32_t cols[];  // per warp: X running counts (inclusive sums along x), X new counts
   int32_t reg[kRegs > 0 ? kRegs : 1];
   const int X = gc.X, Y = gc.Y, Z = gc.Z, X1 = X + 1, Y1 = Y + 1;
@@ -250,23 +268,27 @@ __global__ void __launch_bounds__(kSatWarps * 32) ref_sat_list_kernel(const Grid
   }
 }
 
-// The same by passes over the whole array, for small arrays and for grids too wide for a warp's counts in
-// shared memory (ref_sat_by_list).
+// The same by passes over the whole array: for small arrays, for grids too wide for a warp's counts in
+// shared memory (ref_sat_by_list) and for scans with too many voxels of one symbol (launch_ref_sat_list).
 // Pass 0: running sums along x per (a, z, y) row (a warp per row: inclusive warp scans over
-// 32-voxel chunks, coalesced); pass 1 along y and pass 2 along z (a thread per column, rows
-// read kChunk at a time so that the loads of a chunk are in flight together).
+// 32-voxel chunks, coalesced) and the zero entries; pass 1 along y and pass 2 along z (a thread per
+// column, rows read kChunk at a time so that the loads of a chunk are in flight together).
 constexpr int kChunk = 8;
 
 __global__ void ref_sat_x_kernel(const GridConst gc, const uint8_t* __restrict__ symA, int32_t* __restrict__ sat) {
-  const int X = gc.X, Y = gc.Y, Z = gc.Z, X1 = X + 1, Y1 = Y + 1, Z1 = Z + 1;
-  const int64_t rows = (int64_t)(gc.K - 1) * Z * Y;
+  const int X = gc.X, Y = gc.Y, X1 = X + 1, Y1 = Y + 1, Z1 = gc.Z + 1;
+  const int64_t rows = (int64_t)(gc.K - 1) * Z1 * Y1;
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   for (int64_t r = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); r < rows; r += warps) {
-    const int y = (int)(r % Y);
-    const int z = (int)((r / Y) % Z);
-    const int a = (int)(r / ((int64_t)Y * Z)) + 1;
-    int32_t* out = sat + (((size_t)(a - 1) * Z1 + (z + 1)) * Y1 + (y + 1)) * X1;
+    const int y = (int)(r % Y1) - 1;  // row y of layer z ends in the entries of y + 1 and z + 1
+    const int z = (int)((r / Y1) % Z1) - 1;
+    const int a = (int)(r / ((int64_t)Y1 * Z1)) + 1;
+    int32_t* out = sat + (size_t)r * X1;
+    if (y < 0 || z < 0) {
+      for (int x = lane; x < X1; x += 32) out[x] = 0;
+      continue;
+    }
     const uint8_t* in = symA + ((size_t)z * Y + y) * X;
     if (lane == 0) out[0] = 0;
     int32_t carry = 0;
@@ -355,18 +377,27 @@ bool ref_sat_by_list(const GridConst& gc) {
 }
 
 cudaError_t launch_ref_sat_list(const GridConst& gc, const uint8_t* symA, uint32_t* row_n, uint32_t* list,
-                                int32_t* sat, int n_sm, cudaStream_t s) {
+                                int32_t* few, int32_t* sat, int n_sm, cudaStream_t s) {
   const int64_t V = (int64_t)gc.X * gc.Y * gc.Z;
-  ref_rows_kernel<<<1, 1024, 0, s>>>(row_n, (int64_t)(gc.K - 1) * gc.Y + 1);
+  const int64_t n_sat = (int64_t)(gc.K - 1) * (gc.Z + 1) * (gc.Y + 1) * (gc.X + 1);
+  // A strip adds up all of its symbol's voxels before it, 128 at a time: 4 ns per voxel of the symbol
+  // with the most, while the passes take about 1 us per MB more than the list's writes.  1M points
+  // spread evenly over 320 x 320 x 32 voxels, 15 symbols (196 MB): 3.2 ms by list, 0.48 by passes; 30k
+  // points 0.29 and 0.37; a LiDAR scan of 106k 0.19 and 0.32.
+  const int64_t most = n_sat * 4 / kSatMostBytes;
+  ref_rows_kernel<<<1, 1024, 0, s>>>(row_n, (int64_t)(gc.K - 1) * gc.Y + 1, gc.Y,
+                                   (uint32_t)std::min<int64_t>(most, UINT32_MAX), few);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  ref_list_kernel<<<blocks_for((V + 15) / 16, 256), 256, 0, s>>>(gc, symA, row_n, list);
+  ref_list_kernel<<<blocks_for((V + 15) / 16, 256), 256, 0, s>>>(gc, symA, row_n, list, few);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const size_t smem = (size_t)kSatWarps * 2 * gc.X * 4;
   auto* k = gc.X <= 160 ? ref_sat_list_kernel<5> : gc.X <= 416 ? ref_sat_list_kernel<13> : ref_sat_list_kernel<0>;
   if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024)) != cudaSuccess) return e;
   // shorter strips while there are few: a strip's rows follow one another (latency), but each strip
-  // adds up the rows before it first
+  // adds up the rows before it first.  Strips of 31 rows throughout: 160 x 160 x 16 voxels 140 us, 320 x
+  // 320 x 32 (15 symbols) 215, 1500 x 100 x 20 351; as here 126, 188, 214; 400 x 400 x 40 388 either way;
+  // strips of 7 everywhere 122, 175, 214, 385, but 64 x 64 x 200 175 against 162.
   int rows = kSatRows;
   auto blocks_of = [&](int r) {
     return ((int64_t)(gc.K - 1) * (gc.Z + 1) * ((gc.Y + r) / r) + kSatWarps - 1) / kSatWarps;
@@ -374,13 +405,13 @@ cudaError_t launch_ref_sat_list(const GridConst& gc, const uint8_t* symA, uint32
   while (rows > 7 && blocks_of(rows) < 16 * (int64_t)n_sm) rows /= 2;
   const int64_t blocks = blocks_of(rows);
   k<<<(unsigned)std::min<int64_t>(blocks, 64 * (int64_t)n_sm), kSatWarps * 32, smem, s>>>(gc, row_n, list, sat,
-                                                                                           rows);
+                                                                                           rows, few);
   return cudaGetLastError();
 }
 
 cudaError_t launch_ref_sat(const GridConst& gc, const uint8_t* symA, int32_t* sat, cudaStream_t s) {
   if (gc.K <= 1) return cudaSuccess;
-  const int64_t rows = (int64_t)(gc.K - 1) * gc.Z * gc.Y;
+  const int64_t rows = (int64_t)(gc.K - 1) * (gc.Z + 1) * (gc.Y + 1);
   ref_sat_x_kernel<<<blocks_for(rows * 32, 256), 256, 0, s>>>(gc, symA, sat);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;

@@ -1324,11 +1324,11 @@ align_status align_set_reference(align_grid* g, const float* xyzA, int64_t nA, i
                               s1.as<unsigned long long>(), s2.as<unsigned long long>(), g->stream),
         "launch reference accumulate");
     TRY(g->symA.ensure(V), "allocate A symbols");
-    TRY(box.ensure(sizeof(int32_t) * 6), "allocate box");
-    TRY(g->ref_box_h.ensure(sizeof(int32_t) * 12), "allocate pinned box");
+    TRY(box.ensure(sizeof(int32_t) * 7), "allocate box");  // and whether the list gave the sums
+    TRY(g->ref_box_h.ensure(sizeof(int32_t) * 14), "allocate pinned box");
     int32_t* box_h = g->ref_box_h.as<int32_t>();
-    for (int i = 0; i < 6; ++i) box_h[i] = i < 3 ? INT_MAX : INT_MIN;
-    TRY(cudaMemcpyAsync(box.p, box_h, sizeof(int32_t) * 6, cudaMemcpyHostToDevice, g->stream), "init box");
+    for (int i = 0; i < 7; ++i) box_h[i] = i < 3 ? INT_MAX : i < 6 ? INT_MIN : 1;
+    TRY(cudaMemcpyAsync(box.p, box_h, sizeof(int32_t) * 7, cudaMemcpyHostToDevice, g->stream), "init box");
     TRY(launch_ref_symbols(gc, cnt.as<uint32_t>(), s1.as<unsigned long long>(), s2.as<unsigned long long>(),
                            g->symA.as<uint8_t>(), box.as<int32_t>(), by_list ? g->ref_rows.as<uint32_t>() : nullptr,
                            g->stream),
@@ -1338,17 +1338,20 @@ align_status align_set_reference(align_grid* g, const float* xyzA, int64_t nA, i
     TRY(g->sat.ensure(std::max<size_t>(1, sat_elems) * 4), "allocate prefix sums");
     if (by_list) {
       TRY(launch_ref_sat_list(gc, g->symA.as<uint8_t>(), g->ref_rows.as<uint32_t>(), g->ref_list.as<uint32_t>(),
-                              g->sat.as<int32_t>(), g->n_sm, g->stream),
+                              box.as<int32_t>() + 6, g->sat.as<int32_t>(), g->n_sm, g->stream),
           "launch prefix sums");
     } else {
-      TRY(cudaMemsetAsync(g->sat.p, 0, std::max<size_t>(1, sat_elems) * 4, g->stream), "clear prefix sums");
       TRY(launch_ref_sat(gc, g->symA.as<uint8_t>(), g->sat.as<int32_t>(), g->stream), "launch prefix sums");
     }
-    int32_t* hb = box_h + 6;
-    TRY(cudaMemcpyAsync(hb, box.p, sizeof(int32_t) * 6, cudaMemcpyDeviceToHost, g->stream), "read box");
+    int32_t* hb = box_h + 7;
+    TRY(cudaMemcpyAsync(hb, box.p, sizeof(int32_t) * 7, cudaMemcpyDeviceToHost, g->stream), "read box");
     TRY(cudaStreamSynchronize(g->stream), "synchronize");
+    if (hb[6] == 0) {  // too many voxels of one symbol for the list: its kernels returned at once
+      TRY(launch_ref_sat(gc, g->symA.as<uint8_t>(), g->sat.as<int32_t>(), g->stream), "launch prefix sums");
+      TRY(cudaStreamSynchronize(g->stream), "synchronize");
+    }
     for (int i = 0; i < 6; ++i) g->boxA[i] = g->gc.boxA[i] = hb[i];
-    g->stats[4] += (nA > 0 ? 1 : 0) + 1 + (gc.K > 1 ? 3 : 0);
+    g->stats[4] += (nA > 0 ? 1 : 0) + 1 + (gc.K > 1 ? 3 : 0) + (hb[6] == 0 ? 3 : 0);
 #undef TRY
   } while (0);
   if (result != ALIGN_OK) return result;

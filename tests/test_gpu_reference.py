@@ -41,18 +41,24 @@ def test_reference_symbols_and_marginals(dims, res, feature):
 
 
 @pytest.mark.parametrize("dims,res", [((161, 62, 17), 0.1), ((160, 64, 17), 0.1), ((419, 131, 3), 0.1)])
-def test_reference_with_every_voxel_occupied(dims, res):
+@pytest.mark.parametrize("mixed", [True, False])
+def test_reference_with_every_voxel_occupied(dims, res, mixed):
     """Sixteen symbols of a list thread's words all set, and the last thread's part of them (the sizes of
-    the grids leave 14, 0 and 11 voxels for it)."""
+    the grids leave 14, 0 and 11 voxels for it): by list while no symbol has too many voxels (mixed counts
+    and heights), by the passes when one has (one to three points per voxel)."""
     from paper_1709_06948_gb300 import align
     rng = np.random.default_rng(95)
     size = np.array(dims) * res
     spec = scangen.GridSpec(origin=tuple(-size / 2), res_m=res, dims=dims, feature=2, count_levels=7, var_levels=8)
     k = np.stack(np.meshgrid(*(np.arange(d) for d in dims), indexing="ij"), -1).reshape(-1, 3)
-    k = k[np.repeat(np.arange(len(k)), rng.integers(1, 4, len(k)))]
-    A = ((k + rng.uniform(0.3, 0.7, k.shape)) * res - size / 2).astype(np.float32)
+    n = 2 ** rng.integers(2, 7, len(k)) if mixed else rng.integers(1, 4, len(k))
+    half = np.repeat(0.45 * 0.5 ** rng.uniform(0, 2.5, len(k)) if mixed else np.full(len(k), 0.2), n)
+    k = np.repeat(k, n, axis=0)
+    A = ((k + 0.5 + rng.uniform(-1, 1, k.shape) * half[:, None]) * res - size / 2).astype(np.float32)
     L, G = lib_grid(spec), oracle_grid(spec)
     align.align_set_reference(L, A)
+    launches = align.align_eval_stats(L)["kernel_launches"]
+    assert launches == (5 if mixed else 8)  # sums, symbols, and the list's three kernels (then the passes)
     symA, boxA = G.reference(A)
     assert np.count_nonzero(symA) == len(symA.reshape(-1))
     sym, box = align.align_get_reference(L)
