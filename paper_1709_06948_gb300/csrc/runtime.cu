@@ -852,11 +852,16 @@ align_status enqueue_lattice(align_grid* g, LatticeArgs a, const float* d_poses,
 }
 
 // Poses that share nothing: their points spread over the GPU (scatter_eval.cu).  *taken: whether
-// this path took them (not: more points than its sums hold, or no memory for the sums).
+// this path took them (not: more points than its sums hold, many poses on few voxels, or no memory for
+// the sums).
 align_status enqueue_scatter(align_grid* g, const float* d_poses, int64_t P, const EvalOut& out, bool* taken) {
   *taken = false;
   const size_t one = scatter_pose_bytes(g->gc, g->n_points);
   if (g->n_points > kScatterMaxPoints || one * (size_t)P > kScatterBudget) return ALIGN_OK;
+  // points in no order on few voxels: their adds take turns in L2 (32 poses of 120k shuffled points on 10
+  // x 10 x 1 voxels 274 against 195 us a CTA per pose, on 20 x 20 x 2 223 against 198, on 40 x 40 x 4 272
+  // against 407; 8 poses 148 against 190)
+  if (P > 16 && g->n_points > 64 * g->V) return ALIGN_OK;
   ScatterArgs a{};
   a.gc = g->gc;
   a.n = g->n_points;

@@ -59,6 +59,13 @@ def test_more_poses_keep_one_per_cta(tiny):
     _check(tiny.grid, tiny.xyzA, tiny.xyzB, _poses(33, 3), sweep=0)
 
 
+@pytest.mark.parametrize("n_poses,sweep", [(16, 4), (17, 0)])
+@pytest.mark.parametrize("feature", [0, 1])
+def test_many_poses_on_few_voxels_keep_one_per_cta(tiny, n_poses, sweep, feature):
+    spec = scangen.GridSpec(origin=(-20.0, -20.0, -1.0), res_m=8.0, dims=(5, 5, 2), feature=feature, count_levels=7)
+    _check(spec, tiny.xyzA, tiny.xyzB, _poses(n_poses, 19), sweep=sweep)
+
+
 def test_non_finite_points(tiny):
     xyz = tiny.xyzB.copy()
     xyz[::7, 0] = np.nan
