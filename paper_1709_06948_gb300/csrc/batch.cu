@@ -734,12 +734,16 @@ extern "C" align_status align_eval_batch(align_batch* b, const align_pair* pairs
   }
   // Lattices by groups, unless the caller fixed the table kernels' shape or poses per CTA: those with
   // a group per SM (smaller ones share the table kernels' launches, two per pair).
+  // (once a pair rotates in the kernel all table pairs do, and only lattices are looked for: 22 us of
+  // hashing per pair of 500 poses without shared rotations otherwise)
+  bool rotate = std::any_of(plans.begin(), plans.end(), [](const PairPlan& pp) { return pp.hposes.empty(); });
   for (PairPlan& pp : plans) {
-    if (pp.hposes.empty()) continue;
+    if (pp.hposes.empty() || (rotate && !may_be_lattice(pp.hposes.data(), pp.P))) continue;
     pp.set = pose_set(pp.hposes.data(), pp.P);
     pp.by_groups = b->shape_fixed < 0 && b->pairs_fixed < 0 && pp.set.lattice && pp.g->sweep_mode < 0 &&
                    plan_lattice(pp.g->gc, b->n_sm, b->smem_optin, pp.nB, pp.set.n_rot, pp.set.mx, pp.set.my, pp.set.mz,
                                 pp.set.t_max, b->n_sm, pp.lat);
+    rotate = rotate || (!pp.by_groups && pp.set.n_rot <= 0);
   }
   size_t lattice_bytes = 0;
   for (PairPlan& pp : plans)

@@ -487,6 +487,12 @@ struct AxisValues {
 };
 
 }  // namespace
+bool mialign::may_be_lattice(const float* poses12, int64_t P) {
+  int64_t n = 0;
+  for (int64_t p = 0; p < P; ++p) n += std::memcmp(poses12, poses12 + 12 * p, 36) == 0;
+  return n * std::max<int64_t>(1, P / 4) >= P;
+}
+
 PoseSet mialign::pose_set(const float* poses12, int64_t P) {
   PoseSet S;
   AxisValues ax[3];
@@ -494,8 +500,6 @@ PoseSet mialign::pose_set(const float* poses12, int64_t P) {
   std::vector<std::array<int32_t, 3>> c;
   S.src.resize((size_t)P);
   const int64_t max_rot = std::max<int64_t>(1, P / 4);
-  bool lattice = P >= 2;
-  if (lattice) c.resize((size_t)P);
   int32_t last = 0, n_rot = 0;
   for (int64_t p = 0; p < P; ++p) {
     const float* q = poses12 + 12 * p;
@@ -516,15 +520,18 @@ PoseSet mialign::pose_set(const float* poses12, int64_t P) {
       last = it.first->second;
     }
     S.src[(size_t)p] = last;
-    if (!lattice) continue;
+  }
+  S.n_rot = n_rot;
+  bool lattice = P >= 2;
+  if (lattice) c.resize((size_t)P);
+  for (int64_t p = 0; p < P && lattice; ++p) {
     for (int a = 0; a < 3; ++a) {
       uint32_t b;
-      std::memcpy(&b, q + 9 + a, 4);
+      std::memcpy(&b, poses12 + 12 * p + 9 + a, 4);
       c[(size_t)p][a] = ax[a].index(b);
     }
     lattice = ax[1].v.size() <= (size_t)kLatticeMaxY && ax[2].v.size() <= (size_t)kLatticeMaxZ;
   }
-  S.n_rot = n_rot;
   S.mx = (int32_t)ax[0].v.size();
   S.my = (int32_t)ax[1].v.size();
   S.mz = (int32_t)ax[2].v.size();

@@ -78,6 +78,9 @@ struct PoseSet {
   std::vector<int32_t> pose_of;
 };
 PoseSet pose_set(const float* poses12, int64_t P);
+// Whether the first pose's rotation occurs as often as a lattice's would: false for poses that
+// pose_set would find to be none, at a fraction of its time where no two rotations are alike.
+bool may_be_lattice(const float* poses12, int64_t P);
 align_status check_grid_device(align_grid* g);
 // Pose pairs for the pair kernel: poses with the same rotation (tile copy) and bitwise equal
 // t'_y, t'_z, two per unit (local indices; the second -1 for a single pose).  Returns the units.

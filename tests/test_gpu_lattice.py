@@ -246,3 +246,24 @@ def test_batch_mixes_groups_and_tables(tiny, graph):
             align.align_set_sweep(L, -1)
             assert np.array_equal(mi.view(np.int32), mi0.view(np.int32)) and am == am0
     align.align_batch_destroy(b)
+
+
+def test_batch_finds_lattices_after_other_pairs(tiny):
+    """A lattice behind a pair without shared rotations goes by groups as it does before one: the same
+    kernels, the same results; so does one whose rotations change fastest."""
+    from paper_1709_06948_gb300 import align
+    rng = np.random.default_rng(99)
+    L = lib_grid(tiny.grid)
+    align.align_set_reference(L, tiny.xyzA)
+    other = tiny.T + rng.uniform(-0.5, 0.5, (40, 6))
+    for order in ((3, 4, 5, 0, 1, 2), (0, 1, 2, 3, 4, 5)):
+        lat = _lattice((8, 8, 2, 2, 2, 4), SMALL, order)
+        seen = []
+        for pairs in ([(L, tiny.xyzB, lat), (L, tiny.xyzB, other)], [(L, tiny.xyzB, other), (L, tiny.xyzB, lat)]):
+            b = align.align_batch_create()
+            got = align.align_eval_batch(b, pairs)
+            k = 0 if pairs[0][2] is lat else 1
+            seen.append((align.align_batch_stats(b)["kernel_launches"], got[k][0].tobytes(), got[k][1], got[1 - k][0].tobytes()))
+            align.align_batch_destroy(b)
+        assert seen[0] == seen[1] and seen[0][0] == 3 + 6 + 2  # pack, compose, argmax; groups' six, eval and redo
+    L.close()
