@@ -65,7 +65,7 @@ struct PairPlan {
 // Workspace sizes of one launch; a change of any of them re-allocates and drops the graph.
 struct Sizes {
   size_t xyz = 0, poses = 0, pts = 0, pose_src = 0, copies = 0, items = 0, starts = 0, outc = 0, box = 0,
-         best = 0, mi = 0, argmax = 0, redo = 0, wide = 0, ipasses = 0, ovf = 0, units = 0, spill = 0, order = 0, lattice = 0;
+         best = 0, mi = 0, argmax = 0, redo = 0, wide = 0, ipasses = 0, ovf = 0, units = 0, spill = 0, order = 0;
 };
 
 std::string env_cache_path() {
@@ -127,7 +127,10 @@ struct align_batch {
   std::string device_name;
   int shape_fixed = -1;
   DevBuf xyz, poses, pts, pose_src, copies, items, starts, outc, box, best, mi, argmax, redo_list, redo_count, wide,
-      status, ipasses, ovf, units, spill, order, lattice;
+      status, ipasses, ovf, units, spill, order;
+  OptionalBuf lattice;
+  size_t optional_limit = 0;  // OptionalBuf::ensure
+  bool optional_on = true;    // false while a call that ran out of memory is run again without it
   // page-locked staging of the poses and their tile copies (asynchronous copies; a call's
   // copies are done when it returns, since every call synchronises its stream)
   mialign::HostBuf h_poses, h_src;
@@ -304,6 +307,7 @@ align_status align_batch_create(void* cuda_stream, align_batch** out) {
   b->device = dev;
   b->n_sm = prop.multiProcessorCount;
   b->smem_optin = prop.sharedMemPerBlockOptin;
+  b->optional_limit = prop.totalGlobalMem / kOptionalShare;
   b->device_name = prop.name;
   for (char& c : b->device_name)
     if (c == ' ') c = '_';
@@ -328,8 +332,9 @@ align_status align_batch_destroy(align_batch* b) {
   drop_graph(b);
   for (DevBuf* d : {&b->xyz, &b->poses, &b->pts, &b->pose_src, &b->copies, &b->items, &b->starts, &b->outc, &b->box,
                     &b->best, &b->mi, &b->argmax, &b->redo_list, &b->redo_count, &b->wide, &b->status, &b->ipasses, &b->ovf,
-                    &b->units, &b->spill, &b->order, &b->lattice})
+                    &b->units, &b->spill, &b->order})
     d->release();
+  b->lattice.release();
   b->h_poses.release();
   b->h_src.release();
   if (b->ev0) cudaEventDestroy(b->ev0);
@@ -680,9 +685,9 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
 
 }  // namespace
 
-extern "C" align_status align_eval_batch(align_batch* b, const align_pair* pairs, int32_t n_pairs, int flags) {
-  if (!b) return report_error(ALIGN_E_INVALID, "batch is NULL");
-  if (n_pairs < 0 || (n_pairs > 0 && !pairs)) return report_error(ALIGN_E_INVALID, "bad pair array");
+namespace {
+
+align_status eval_batch(align_batch* b, const align_pair* pairs, int32_t n_pairs, int flags) {
   BCU(cudaSetDevice(b->device), "cudaSetDevice");
   // work already queued on the caller's stream (device inputs) comes first
   BCU(cudaEventRecord(b->ev_in, b->user_stream), "record event");
@@ -751,7 +756,10 @@ extern "C" align_status align_eval_batch(align_batch* b, const align_pair* pairs
   if (lattice_bytes > 0) {
     BCU(lattice_setup(), "set up lattice kernels");  // before any capture
     // without the memory for it the table kernels take the poses
-    if (grow(b, b->lattice, b->cap.lattice, lattice_bytes, "allocate lattice workspace") != ALIGN_OK)
+    const void* const old = b->lattice.p;
+    const bool ok = b->optional_on && b->lattice.ensure(lattice_bytes, b->optional_limit);
+    if (b->lattice.p != old) drop_graph(b);
+    if (!ok)
       for (PairPlan& pp : plans) pp.by_groups = false;
   }
   const bool tables = std::any_of(plans.begin(), plans.end(), [](const PairPlan& pp) { return !pp.by_groups; });
@@ -828,3 +836,19 @@ extern "C" align_status align_eval_batch(align_batch* b, const align_pair* pairs
   }
   return collect(b);
 }
+
+}  // namespace
+
+extern "C" align_status align_eval_batch(align_batch* b, const align_pair* pairs, int32_t n_pairs, int flags) {
+  if (!b) return report_error(ALIGN_E_INVALID, "batch is NULL");
+  if (n_pairs < 0 || (n_pairs > 0 && !pairs)) return report_error(ALIGN_E_INVALID, "bad pair array");
+  align_status st = eval_batch(b, pairs, n_pairs, flags);
+  if (st != ALIGN_E_OOM || b->lattice.p == nullptr) return st;
+  drop_graph(b);  // once more without the groups' workspace (no results have been returned yet)
+  b->lattice.release();
+  b->optional_on = false;
+  st = eval_batch(b, pairs, n_pairs, flags);
+  b->optional_on = true;
+  return st;
+}
+

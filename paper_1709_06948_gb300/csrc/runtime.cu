@@ -765,11 +765,31 @@ align_status profile_event(align_grid* g, std::array<cudaEvent_t, 3>& evs, int i
   return ALIGN_OK;
 }
 
+// Frees what the grid holds for paths that it can do without; false: nothing.
+bool give_back(align_grid* g) {
+  bool any = false;
+  for (OptionalBuf* b : {&g->lattice_ws, &g->scatter_sums, &g->scatter_list}) {
+    any = any || b->p != nullptr;
+    b->release();  // (waits for the device's work)
+  }
+  return any;
+}
+
+// A call on a grid, and where it runs out of memory while the grid holds some that it can do without,
+// the call once more through the paths that need none (it has then returned no results yet).
+template <class F>
+align_status within_memory(align_grid* g, F&& call) {
+  align_status st = call();
+  if (st != ALIGN_E_OOM || !give_back(g)) return st;
+  g->optional_on = false;
+  st = call();
+  g->optional_on = true;
+  return st;
+}
+
 // The groups' workspace; without the memory for it the table kernels take the poses.
 bool reserve_lattice(align_grid* g, LatticeArgs a) {
-  if (g->lattice_ws.ensure(lattice_carve(a, nullptr)) == cudaSuccess) return true;
-  (void)cudaGetLastError();
-  return false;
+  return g->optional_on && g->lattice_ws.ensure(lattice_carve(a, nullptr), g->optional_limit);
 }
 
 // One evaluation of a pose lattice by groups (lattice_eval.cu): `a` as plan_lattice left it, the
@@ -863,6 +883,7 @@ align_status enqueue_lattice(align_grid* g, LatticeArgs a, const float* d_poses,
 // the sums).
 align_status enqueue_scatter(align_grid* g, const float* d_poses, int64_t P, const EvalOut& out, bool* taken) {
   *taken = false;
+  if (!g->optional_on) return ALIGN_OK;
   const size_t one = scatter_pose_bytes(g->gc, g->n_points);
   if (g->n_points > kScatterMaxPoints || one * (size_t)P > kScatterBudget) return ALIGN_OK;
   // points in no order on few voxels: their adds take turns in L2 (32 poses of 120k shuffled points on 10
@@ -878,9 +899,14 @@ align_status enqueue_scatter(align_grid* g, const float* d_poses, int64_t P, con
   const size_t words = g->gc.feature != ALIGN_FEAT_COUNT ? 16 : 8;
   const size_t KK = (size_t)g->gc.K * g->gc.K;
   // the buffers that the kernels leave cleared: cleared here when they are new
-  DevBuf* const cleared[] = {&g->scatter_sums, &g->scatter_c, &g->scatter_n};
-  const size_t bytes[] = {(size_t)P * (size_t)g->V * words, (size_t)P * KK * 4, (size_t)P * 4};
-  for (int i = 0; i < 3; ++i) {
+  const size_t sums = (size_t)P * (size_t)g->V * words;
+  if (g->scatter_sums.p == nullptr || g->scatter_sums.cap < sums) {
+    if (!g->scatter_sums.ensure(sums, g->optional_limit)) return ALIGN_OK;
+    CU(cudaMemsetAsync(g->scatter_sums.p, 0, g->scatter_sums.cap, g->stream), "clear sums");
+  }
+  DevBuf* const cleared[] = {&g->scatter_c, &g->scatter_n};
+  const size_t bytes[] = {(size_t)P * KK * 4, (size_t)P * 4};
+  for (int i = 0; i < 2; ++i) {
     if (cleared[i]->p != nullptr && cleared[i]->cap >= bytes[i]) continue;
     if (cleared[i]->ensure(bytes[i]) != cudaSuccess) {
       (void)cudaGetLastError();
@@ -897,10 +923,7 @@ align_status enqueue_scatter(align_grid* g, const float* d_poses, int64_t P, con
     CU(cudaMemset2DAsync(b, 24, 0x7F, 12, kScatterMaxPoses, g->stream), "clear boxes");
     CU(cudaMemset2DAsync(b + 12, 24, 0x80, 12, kScatterMaxPoses, g->stream), "clear boxes");
   }
-  if (g->scatter_list.ensure((size_t)P * (size_t)a.list_cap * 4) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return ALIGN_OK;
-  }
+  if (!g->scatter_list.ensure((size_t)P * (size_t)a.list_cap * 4, g->optional_limit)) return ALIGN_OK;
   *taken = true;
   CU(g->redo_count.ensure(16), "allocate redo count");
   align_status st = ensure_head(g);
@@ -1239,6 +1262,7 @@ align_status align_create_grid(const align_grid_desc* desc, void* cuda_stream, a
   g->device = dev;
   g->n_sm = prop.multiProcessorCount;
   g->smem_optin = prop.sharedMemPerBlockOptin;
+  g->optional_limit = prop.totalGlobalMem / kOptionalShare;
   g->table_slots = eval_shape(0).table_slots_for(gc.K, eval_layout(gc, gc.feature != ALIGN_FEAT_COUNT), g->smem_optin, 1);
   for (int i = 0; i < 6; ++i) g->boxA[i] = i < 3 ? INT_MAX : INT_MIN;
   *out = g;
@@ -1254,9 +1278,9 @@ align_status align_destroy_grid(align_grid* g) {
                     &g->pose_src, &g->rots, &g->redo_list, &g->redo_count, &g->ovf, &g->lat_c,
                     &g->lat_cand, &g->ref_pts, &g->ref_pose, &g->ref_cnt, &g->ref_s1, &g->ref_s2, &g->ref_box, &g->ref_rows,
                     &g->ref_list,
-                    &g->units, &g->lat_units, &g->spill, &g->lattice_ws, &g->lattice_order, &g->scatter_sums,
-                    &g->scatter_list, &g->scatter_n, &g->scatter_c, &g->scatter_box})
+                    &g->units, &g->lat_units, &g->spill, &g->lattice_order, &g->scatter_n, &g->scatter_c, &g->scatter_box})
     b->release();
+  give_back(g);
   for (HostBuf* b : {&g->head_h, &g->hist_h, &g->lat_cand_h, &g->lat_rec_h, &g->lat_c_h, &g->ref_box_h}) b->release();
   for (cudaEvent_t e : g->lat_ev) cudaEventDestroy(e);
   for (auto* v : {&g->ev_pending, &g->ev_pool})
@@ -1280,13 +1304,8 @@ align_status align_round_poses(const float origin[3], const double* eta6, int64_
   return ALIGN_OK;
 }
 
-align_status align_set_reference(align_grid* g, const float* xyzA, int64_t nA, int flags) {
-  align_status st = check_grid(g);
-  if (st != ALIGN_OK) return st;
-  if (nA < 0 || nA >= INT32_MAX) return fail(ALIGN_E_INVALID, "nA out of range");
-  if (nA > 0 && !xyzA) return fail(ALIGN_E_INVALID, "xyzA is NULL");
-  g->has_ref = false;
-  st = ensure_head(g);
+static align_status set_reference(align_grid* g, const float* xyzA, int64_t nA, int flags) {
+  align_status st = ensure_head(g);
   if (st != ALIGN_OK) return st;
   const GridConst& gc = g->gc;
   const size_t V = (size_t)g->V;
@@ -1369,6 +1388,15 @@ align_status align_set_reference(align_grid* g, const float* xyzA, int64_t nA, i
   if (result != ALIGN_OK) return result;
   g->has_ref = true;
   return ALIGN_OK;
+}
+
+align_status align_set_reference(align_grid* g, const float* xyzA, int64_t nA, int flags) {
+  align_status st = check_grid(g);
+  if (st != ALIGN_OK) return st;
+  if (nA < 0 || nA >= INT32_MAX) return fail(ALIGN_E_INVALID, "nA out of range");
+  if (nA > 0 && !xyzA) return fail(ALIGN_E_INVALID, "xyzA is NULL");
+  g->has_ref = false;
+  return within_memory(g, [&] { return set_reference(g, xyzA, nA, flags); });
 }
 
 align_status align_get_reference(align_grid* g, uint8_t* symA, int32_t boxA[6]) {
@@ -1477,16 +1505,14 @@ align_status align_eval_mi(align_grid* g, const float* xyzB, int64_t nB, int fla
   }
   st = ensure_head(g);
   if (st != ALIGN_OK) return st;
-  return eval_common(g, xyzB, nB, flags, poses12, eta6, P, mi_out, argmax_out, hist_out, nullptr, false, 0);
+  return within_memory(g, [&] {
+    return eval_common(g, xyzB, nB, flags, poses12, eta6, P, mi_out, argmax_out, hist_out, nullptr, false, 0);
+  });
 }
 
-align_status align_accumulate(align_grid* g, const float* xyzB, int64_t nB, int flags, const float pose12[12],
-                              int64_t* acc_out, int32_t box_out[6]) {
-  align_status st = check_grid(g);
-  if (st != ALIGN_OK) return st;
-  if (!g->has_ref) return fail(ALIGN_E_NOREF, "no reference scan set");
-  if (!pose12) return fail(ALIGN_E_INVALID, "pose12 is NULL");
-  st = ensure_head(g);
+static align_status accumulate(align_grid* g, const float* xyzB, int64_t nB, int flags, const float pose12[12],
+                               int64_t* acc_out, int32_t box_out[6]) {
+  align_status st = ensure_head(g);
   if (st != ALIGN_OK) return st;
   const size_t bytes = (size_t)g->V * 3 * sizeof(int64_t);
   CU(g->dump.ensure(bytes), "allocate sums");
@@ -1500,6 +1526,19 @@ align_status align_accumulate(align_grid* g, const float* xyzB, int64_t nB, int 
   if (box_out) CU(cudaMemcpy(box_out, g->out_box.p, 6 * sizeof(int32_t), cudaMemcpyDeviceToHost), "read box");
   return ALIGN_OK;
 }
+
+align_status align_accumulate(align_grid* g, const float* xyzB, int64_t nB, int flags, const float pose12[12],
+                              int64_t* acc_out, int32_t box_out[6]) {
+  align_status st = check_grid(g);
+  if (st != ALIGN_OK) return st;
+  if (!g->has_ref) return fail(ALIGN_E_NOREF, "no reference scan set");
+  if (!pose12) return fail(ALIGN_E_INVALID, "pose12 is NULL");
+  return within_memory(g, [&] { return accumulate(g, xyzB, nB, flags, pose12, acc_out, box_out); });
+}
+
+static align_status search(align_grid* g, const float* xyzB, int64_t nB, int flags, const double init[6],
+                           const double range[6], const int32_t counts[6], int32_t levels, int64_t P, double T_out[6],
+                           float* mi_out, int64_t* level_best);
 
 align_status align_search_ex(align_grid* g, const float* xyzB, int64_t nB, int flags, const double init[6],
                              const double range[6], const int32_t counts[6], int32_t levels, double T_out[6],
@@ -1515,7 +1554,13 @@ align_status align_search_ex(align_grid* g, const float* xyzB, int64_t nB, int f
     P *= counts[a];
     if (P >= (1 << 26)) return fail(ALIGN_E_INVALID, "lattice too large");
   }
-  st = ensure_head(g);
+  return within_memory(g, [&] { return search(g, xyzB, nB, flags, init, range, counts, levels, P, T_out, mi_out, level_best); });
+}
+
+static align_status search(align_grid* g, const float* xyzB, int64_t nB, int flags, const double init[6],
+                           const double range[6], const int32_t counts[6], int32_t levels, int64_t P, double T_out[6],
+                           float* mi_out, int64_t* level_best) {
+  align_status st = ensure_head(g);
   if (st != ALIGN_OK) return st;
   int32_t n_tiles = 0;
   st = upload_points(g, xyzB, nB, flags, &n_tiles);
@@ -1606,6 +1651,10 @@ align_status nm_eval(align_grid* g, int32_t n_tiles, const std::vector<const dou
 
 }  // namespace
 
+static align_status refine_nm(align_grid* g, const float* xyzB, int64_t nB, int flags, const double* starts, int32_t S,
+                              const double step[6], int32_t max_iter, double ftol, double* T_out, float* mi_out,
+                              int32_t* iters_out);
+
 align_status align_refine_nm(align_grid* g, const float* xyzB, int64_t nB, int flags, const double* starts,
                              int32_t S, const double step[6], int32_t max_iter, double ftol, double* T_out,
                              float* mi_out, int32_t* iters_out) {
@@ -1619,7 +1668,14 @@ align_status align_refine_nm(align_grid* g, const float* xyzB, int64_t nB, int f
   for (int a = 0; a < 6; ++a)
     if (!std::isfinite(step[a])) return fail(ALIGN_E_INVALID, "step not finite");
   if (S == 0) return ALIGN_OK;
-  st = ensure_head(g);
+  return within_memory(
+      g, [&] { return refine_nm(g, xyzB, nB, flags, starts, S, step, max_iter, ftol, T_out, mi_out, iters_out); });
+}
+
+static align_status refine_nm(align_grid* g, const float* xyzB, int64_t nB, int flags, const double* starts, int32_t S,
+                              const double step[6], int32_t max_iter, double ftol, double* T_out, float* mi_out,
+                              int32_t* iters_out) {
+  align_status st = ensure_head(g);
   if (st != ALIGN_OK) return st;
   int32_t n_tiles = 0;
   st = upload_points(g, xyzB, nB, flags, &n_tiles);

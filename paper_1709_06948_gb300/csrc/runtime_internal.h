@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <array>
+#include <atomic>
 #include <cstdint>
 #include <vector>
 
@@ -35,6 +36,44 @@ struct DevBuf {
   template <class T>
   T* as() const {
     return static_cast<T*>(p);
+  }
+};
+
+// Device memory that a faster path takes where it can and does without where it cannot (voxel sums of
+// scattered poses, lattice workspaces).  All objects of the process together hold at most `limit` of
+// it (kOptionalShare of the device's memory; 0: not counted, a server's budget covers it), so that what
+// other objects need is never taken by it; give_back returns an object's own when memory runs out.
+constexpr size_t kOptionalShare = 8;
+struct OptionalBuf : DevBuf {
+  bool counted = false;
+  bool ensure(size_t bytes, size_t limit) {
+    if (bytes <= cap && p != nullptr) return true;
+    const size_t want = std::max<size_t>(bytes, 256), had = counted ? cap : 0;
+    if (limit != 0) {
+      size_t h = held().load();
+      do {
+        if (h - had + want > limit) return false;
+      } while (!held().compare_exchange_weak(h, h - had + want));
+    } else if (counted) {
+      held() -= had;
+    }
+    counted = limit != 0;
+    if (DevBuf::ensure(want) == cudaSuccess) return true;
+    (void)cudaGetLastError();
+    if (counted) held() -= want;
+    counted = false;
+    return false;
+  }
+  void release() {
+    if (counted) held() -= cap;
+    counted = false;
+    DevBuf::release();
+  }
+
+ private:
+  static std::atomic<size_t>& held() {
+    static std::atomic<size_t> bytes{0};
+    return bytes;
   }
 };
 
@@ -164,10 +203,14 @@ struct align_grid {
                               // whose request was admitted without the groups' memory)
   int32_t scatter_on = 1;     // 0: poses that share nothing go through the table kernels (a server's
                               // workspace: its requests' estimates hold no dense sums)
-  mialign::DevBuf lattice_ws, lattice_order;  // groups' workspace; a device-built level's pose order
+  size_t optional_limit = 0;  // OptionalBuf::ensure
+  bool optional_on = true;    // false while a call that ran out of memory is run again without them
+  mialign::OptionalBuf lattice_ws;            // groups' workspace
+  mialign::DevBuf lattice_order;              // a device-built level's pose order
   int32_t lattice_order_m[6] = {0, 0, 0, 0, 0, 0};
   // poses that share nothing; all but the list as the kernels leave it between calls (zero, no box)
-  mialign::DevBuf scatter_sums, scatter_list, scatter_n, scatter_c, scatter_box;
+  mialign::OptionalBuf scatter_sums, scatter_list;
+  mialign::DevBuf scatter_n, scatter_c, scatter_box;
   bool last_cluster = false;  // ... or ran one pose per 2-CTA cluster
   mialign::DevBuf units;    // pose pairs of the last pair launch with host poses
   mialign::DevBuf spill;    // runs queued for the later key partitions (EvalArgs::spill)
