@@ -184,9 +184,11 @@ align_status align_eval_stats(align_grid* grid, int64_t out[6]);
 
 /* How this grid's launches sweep their poses (the kinds of align_eval_stats [5]): -1
    automatic (the default: a batch of poses that is a lattice, i.e. every combination of some
-   rotations and some t'_x, t'_y, t'_z, is evaluated by groups where these fill the GPU and no
-   histograms are asked for; up to 32 poses whose rotations do not repeat, or one pose,
-   are spread over the GPU; otherwise pairs while their tables need no more key partitions than
+   rotations and some t'_x, t'_y, t'_z, is evaluated by groups where these fill the GPU and serve
+   enough poses each and no histograms are asked for; up to 32 poses whose rotations do not repeat
+   (16 where voxels hold over 64 points), or one pose, are spread over the GPU; both need device
+   memory of their own, at most 1/8 of the device's for all grids and batches together, given back
+   when a call on the grid runs out of memory; otherwise pairs while their tables need no more key partitions than
    single poses', or, with spill queues and both partitioned, no more than twice as many up
    to 8; the cluster while single poses need 8 or more key partitions), 0 one pose per CTA, 1 pose
    pairs wherever the poses form pairs (single poses elsewhere), 2 one pose per 2-CTA
@@ -295,8 +297,8 @@ align_status align_batch_create(void* cuda_stream, align_batch** out);
 align_status align_batch_destroy(align_batch* b);
 
 /* Evaluate every pair's poses in one launch sequence: one packing launch for all pairs,
-   then per pair the persistent eval kernel (and its exact-path kernel) with the pair's own
-   table layout, then one composition and one argmax launch for all pairs.  Inputs are
+   then per pair the persistent eval kernel with the pair's own table layout, or the kernels of
+   a lattice's groups (as align_set_sweep's automatic choice), and the exact-path kernel, then one composition and one argmax launch for all pairs.  Inputs are
    copied into the batch's workspace first, so the caller's
    buffers may be reused when the call returns; the call waits for the results.  Pairs
    with P == 0 get argmax -1.  ALIGN_E_INVALID for bad arguments, ALIGN_E_NOREF if a grid

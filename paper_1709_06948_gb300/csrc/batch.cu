@@ -175,8 +175,8 @@ struct Launch {
   // one single-pair eval + redo launch per pair: its arguments (the pair in the parameter
   // bank, its poses p_begin..P-1 of the batch) and its table layout
   std::vector<EvalArgs> evals;
-  std::vector<LatticeArgs> lats;   // its lattice by groups instead (n_items 0: not)
-  std::vector<int32_t> lat_rots;   // ... and its rotations
+  std::vector<LatticeArgs> lats;   // its lattice by groups instead,
+  std::vector<int32_t> lat_rots;   // ... of this many rotations (0: by the table kernels)
   std::vector<int> vws;
   int n_ctas = 0;
   bool rotate = false;
@@ -443,7 +443,7 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
     if (pp.by_groups) order_n += pp.P;
     xyz_f += pp.nB * 3;
     poses_n += pp.P;
-    pts_n += std::max(1, pp.n_copies) * pp.n_pad;  // groups: raw tiles for the exact path, written by their kernels
+    pts_n += std::max(1, pp.n_copies) * pp.n_pad;  // groups write raw tiles for the exact path
     outc_n += (pp.P * (int64_t)pp.g->gc.K * pp.g->gc.K + 3) / 4 * 4;  // cleared four words at a time
     n_copies += pp.n_copies;
     max_out = std::max(max_out, pp.n_pad);
@@ -615,7 +615,7 @@ align_status eval_batch_shape(align_batch* b, std::vector<PairPlan>& plans, cons
   for (int i = 0; i < n; ++i) {
     EvalArgs ai = a;
     ai.one = hitems[(size_t)i];
-    ai.items = b->items.as<EvalItem>() + i;  // the redo kernel reads its one item here
+    ai.items = nullptr;  // a single item is read from the parameters
     ai.item_start = nullptr;
     ai.n_items = 1;
     ai.p_begin = (int32_t)plans[(size_t)i].pose_off;

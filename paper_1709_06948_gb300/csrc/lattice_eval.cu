@@ -12,7 +12,7 @@
 //                   cell, and the tables (y cell -> k_y per t'_y, x cell -> a float of that cell)
 //   points_kernel   per (rotation, t'_x chunk, t'_z): the cells (s_x, s_y, k_z) of consecutive
 //                   scan points, merged where they repeat (n, S1, S2), and the size of the bins
-//                   (k_z, s_y)
+//                   (k_z, s_y); the scan as raw tiles, for poses that the exact path finishes
 //   offsets_kernel  bin starts
 //   scatter_kernel  those elements in bin order: rows (k_z, k_y) of voxels are contiguous for
 //                   every t'_y
@@ -28,11 +28,13 @@
 // and insert its runs into a hash table, the per-pose work falls from every point to every
 // occupied cell of the group (0.2 per point on the 120k-point LiDAR pair at 0.5 m) and every
 // occupied voxel (0.06 per point).  Measured per evaluation of 4,096 poses (all kernels but compose),
-// against the table kernels: 120k points at 0.5 m 1.27 -> 0.73 ms, at 0.25 m 2.59 -> 1.76 ms, 257k
+// against the table kernels: 120k points at 0.5 m 1.27 -> 0.67 ms, at 0.25 m 2.59 -> 1.76 ms, 257k
 // points at 1 m 1.77 -> 0.75 ms; 32,768 poses of 259k points at 0.2 m, joint feature, 55 -> 28.4 ms.
-// The evaluation kernel (0.58 of the 0.73 ms) is bound by instruction issue and shared memory together
-// (64% of its issue slots, 61% of the shared-memory pipe) and by the barriers between its short phases;
-// points_kernel (73 us) by its instructions, scatter_kernel (57 us) by the latency of L2 atomics.
+// The evaluation kernel (0.52 of the 0.67 ms) is bound by instruction issue and shared memory together
+// (63% of its issue slots, 63% of the shared-memory pipe) and by the barriers between its short phases;
+// points_kernel (73 us) by its instructions, scatter_kernel (55 us) by the latency of L2 atomics.
+// Where most poses have a voxel past the 32-bit sums (2 m voxels and larger) the exact path binds: 120k
+// points at 4 m 3.1 ms against 2.9 by tables, at 2 m 1.8 against 2.4.
 #include <algorithm>
 #include <climits>
 #include <mutex>

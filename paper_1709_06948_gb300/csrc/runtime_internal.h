@@ -124,12 +124,12 @@ align_status check_grid_device(align_grid* g);
 // Pose pairs for the pair kernel: poses with the same rotation (tile copy) and bitwise equal
 // t'_y, t'_z, two per unit (local indices; the second -1 for a single pose).  Returns the units.
 int pair_units(const float* poses12, const PoseSet& set, int64_t P, std::vector<int32_t>& units);
-// Whether pose pairs are the automatic choice for a grid with these learned key-partition
-// counts (pairs, single poses).
 constexpr size_t kScatterBudget = (size_t)1 << 30;  // sums and lists of poses spread over the GPU
-// Beyond about this many poses a CTA per pose is faster (an L2 atomic per run, not a shared one):
-// they cross at 36 poses (0.25 m LiDAR grid), 42 (0.5 m), 56 (1 m), 22 on the 6.4M-voxel grid, where
-// the budget holds 10.
+// Beyond about this many poses a CTA per pose is faster (an L2 atomic per run, not a shared one): for
+// 120k points in scan order they cross at 36 poses (0.25 m LiDAR grid), 42 (0.5 m), 56 (1 m), 22 on the
+// 6.4M-voxel grid, where the budget holds 10 (as it holds 20 on the 0.25 m grid: 3.3M voxels).  Points in
+// no order cross earlier: at 32 poses 148 against 219 us (0.5 m), 190 against 214 (1 m); on fewer voxels
+// see enqueue_scatter.
 constexpr int64_t kScatterMaxPoses = 32;
 bool plan_lattice(const GridConst& gc, int n_sm, size_t smem_optin, int64_t n, int64_t n_rot, int32_t mx, int32_t my,
                   int32_t mz, double t_max, int min_groups, LatticeArgs& a);
@@ -137,6 +137,8 @@ bool plan_lattice(const GridConst& gc, int n_sm, size_t smem_optin, int64_t n, i
 bool plan_search(const align_grid* g, int64_t n, const int32_t m[6], const double c[6], const double r[6],
                  LatticeArgs& a);
 size_t lattice_carve(LatticeArgs& a, uint8_t* base);
+// Whether pose pairs are the automatic choice for a grid with these learned key-partition
+// counts (pairs, single poses).
 bool pairs_fit(const align_grid* g, int32_t seed_pair, int32_t seed_single);
 // One level of the coarse-to-fine lattice: FP64 poses around centre c (ranges r, m samples
 // per axis; order rx, ry, rz, tx, ty, tz with tz fastest) and their rounded FP32 form.

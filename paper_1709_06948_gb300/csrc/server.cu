@@ -16,7 +16,8 @@
 // Memory: the budget covers the references and every slot's workspace, which keeps the
 // buffers of the largest request it has run (re-allocating between requests would
 // synchronise the device under the other slots' work).  A request counts as the larger of what
-// the pose groups and the table kernels need: either may run its levels.  When the request at the head of
+// the pose groups and the table kernels need: either may run its levels (few poses are never spread over
+// the GPU here: no request is counted with the sums that takes).  When the request at the head of
 // the queue fits only without them and nothing runs, idle slots release their workspaces.
 #include <cuda_runtime.h>
 
@@ -129,8 +130,6 @@ size_t request_bytes(int64_t nB, const int32_t m[6], int K, int T, int n_sm, int
   return (size_t)(nB * 12 + n_rot * n_pad * 16 + P * per_pose + (int64_t)n_sm * (per_cta + spill));
 }
 
-// A workspace: a grid object that owns only evaluation buffers; the reference arrays it
-// reads are bound from a resident reference grid (and never released through it).
 // The same for a request whose lattices are evaluated by groups (plan `a`); the redo kernel's 64-bit
 // sums as the table kernels have them.
 size_t groups_bytes(LatticeArgs a, const GridConst& gc, int n_sm, size_t smem_optin) {
@@ -140,6 +139,8 @@ size_t groups_bytes(LatticeArgs a, const GridConst& gc, int n_sm, size_t smem_op
   return lattice_carve(a, nullptr) + (size_t)(a.n * 12 + n_pad * 16 + a.P * per_pose + (int64_t)n_sm * 2 * T * 8);
 }
 
+// A workspace: a grid object that owns only evaluation buffers; the reference arrays it
+// reads are bound from a resident reference grid (and never released through it).
 align_grid* workspace_create(int device, int n_sm, size_t smem_optin, cudaStream_t stream) {
   align_grid* g = new (std::nothrow) align_grid();
   if (!g) return nullptr;
